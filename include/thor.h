@@ -85,15 +85,14 @@ int thor_ctx_set_launch(thor_ctx_t ctx, int block_size, int blocks_per_sm);
  * photons than lanes spread them over all warps either way.  Results do not depend on
  * these settings. */
 int thor_ctx_set_tail(thor_ctx_t ctx, int spill_below, int max_phases);
-/* Pipelined events of the gridless photon loop on homologous shells.  In warps with at
- * most pipe_lanes live packets (0..32; 0 = never; default 32) each event first tries its
- * line-core form (start-point step inside the safety ball, resonant scattering at |x| <= 2,
- * u_par sample accepted within two trials), with the next event's random words, its optical depth and
- * the outgoing direction formed beside the frequency chain, and runs the general event
- * from the same words otherwise.  In warps with at most burst_lanes live packets (0..32;
- * default 1; only where events are pipelined) a packet runs up to 32 core events back to
- * back in one tight loop, for the lone lanes of a run's tail; with at most 10 such packets
- * the warp's other lanes form their next events' random words ahead (cooperative burst).  Both forms evaluate an event
+/* Core events in rounds, gridless photon loop on homologous shells.  In warps with at most
+ * pipe_lanes live packets (0..32; 0 = never; default 32) events of the line-core kind
+ * (start-point step inside the safety ball, resonant scattering at |x| <= 2, u_par sample
+ * accepted within two trials) run in rounds: the warp's 32 lanes first form what the next
+ * events of its packets take from their random words, then the packets run those events back
+ * to back; other events take the general path.  In warps with at most burst_lanes live
+ * packets (0..32; default 1), and in any warp with at most four, a packet runs up to 32 core
+ * events between general ones, elsewhere up to 16.  Both forms evaluate an event
  * exactly as the general event does, so results do not depend on these settings (only the
  * time to reach them does). */
 int thor_ctx_set_bursts(thor_ctx_t ctx, int pipe_lanes, int burst_lanes);
@@ -323,7 +322,7 @@ typedef struct {
                                 one per warp), -1 = off (every packet shares warps) */
   int32_t presort;           /* frequency pre-sorting of the packets in flight between rounds, so a
                                 warp's packets are of one kind: 1 = on, 0 = off (the default; on the
-                                measured stream it did not pay, the pipelined core events already
+                                measured stream it did not pay, the core events in rounds already
                                 keep core packets in step) */
   int32_t reserved;
 } thor_server_config;

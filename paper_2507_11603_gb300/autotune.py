@@ -7,7 +7,7 @@ short representative run for each candidate shape through the C ABI and keeps th
 fastest; ``tune_server`` does the same for ``events_per_round`` on a small burst of
 requests.  ``tune_modes`` times the execution modes that change no result -- for a grid,
 the one-kernel loop against the event-based loop with a few slot counts; for a shell, the
-lanes that run pipelined events and core bursts -- and keeps the fastest.  Results are
+lanes that run core events in rounds -- and keeps the fastest.  Results are
 cached per device name and workload key in a JSON file next to the built library.
 """
 from __future__ import annotations

@@ -32,8 +32,8 @@ struct thor_ctx {
   int spill_below = 0;      // warps with fewer live lanes hand them to the next launch (0 = off)
   int max_phases = 24;      // launches at most
   int final_below = 256;    // run to completion once this few packets are left
-  int core_lanes = 32;      // warps with at most this many live packets run pipelined events (0 = never)
-  int burst_lanes = 1;      // ... and, with at most this many, core bursts (0 = never)
+  int core_lanes = 32;      // warps with at most this many live packets run core events in rounds (0 = never)
+  int burst_lanes = 1;      // ... and, with at most this many, up to 32 of them between general events
   int share_tail = 1;       // work sharing in the tail of a one-launch shell run
   Buf b_share;
   // event-based grid loop (0 slots = the one-kernel loop throughout)

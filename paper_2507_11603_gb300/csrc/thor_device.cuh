@@ -523,13 +523,24 @@ __device__ __forceinline__ float P_hg(float mu, float g) {
   return 0.5f * (1.0f - g * g) * rsqrtf(d * d * d);
 }
 
+// a b + c, rounded once -- or twice in the grid loop's translation unit, which is compiled
+// without contraction (THOR_SEPARATE_ROUNDING) so that its two execution modes agree.  The
+// direction update is written with it, so that every place that evaluates an event rounds
+// alike whatever the code around it.
+__device__ __forceinline__ float mul_add(float a, float b, float c) {
+#ifdef THOR_SEPARATE_ROUNDING
+  return __fadd_rn(__fmul_rn(a, b), c);
+#else
+  return __fmaf_rn(a, b, c);
+#endif
+}
 // Orthonormal basis perpendicular to unit k (Duff et al. 2017, JCGT 6(1)).
 __device__ __forceinline__ void basis(float kx, float ky, float kz, float3& e1, float3& e2) {
   const float s = copysignf(1.0f, kz);
-  const float a = __fdividef(-1.0f, s + kz);
-  const float b = kx * ky * a;
-  e1 = make_float3(1.0f + s * kx * kx * a, s * b, -s * kx);
-  e2 = make_float3(b, s + ky * ky * a, -ky);
+  const float a = __fdividef(-1.0f, __fadd_rn(s, kz));
+  const float b = __fmul_rn(__fmul_rn(kx, ky), a);
+  e1 = make_float3(mul_add(__fmul_rn(__fmul_rn(s, kx), kx), a, 1.0f), __fmul_rn(s, b), -__fmul_rn(s, kx));
+  e2 = make_float3(b, mul_add(__fmul_rn(ky, ky), a, s), -ky);
 }
 
 struct AtomFrame {  // what peeling-off needs from a resonant scattering
@@ -546,24 +557,39 @@ struct AtomFrame {  // what peeling-off needs from a resonant scattering
 // they are formed before the rejection sampler and overlap with it; only the mixed phase
 // function's isotropic branch (core scatterings, Sec. 2.3.1) needs u_par and redoes the
 // direction afterwards.
+// Which product of each sum is fused is part of a history's bits: kForm fixes it (bit 0-2:
+// the second product of the inner sum for x, y, z; bit 3-5: of the outer sum; bit 6: x^2
+// instead of y^2 in the norm).  The forms in use:
+enum : int { kTurnShell = 0x21, kTurnShellIso = 0x79, kTurnPower = 0x41 };
+template <int kForm>
 __device__ __forceinline__ float3 turn(const float3& k, const float3& e1, const float3& e2, float mu, float st,
                                        float cp, float sp) {
+  auto sum = [](bool second, float a, float b, float c, float d) {  // a b + c d
+    return second ? mul_add(c, d, __fmul_rn(a, b)) : mul_add(a, b, __fmul_rn(c, d));
+  };
   float3 ko;
-  ko.x = mu * k.x + st * (cp * e1.x + sp * e2.x);
-  ko.y = mu * k.y + st * (cp * e1.y + sp * e2.y);
-  ko.z = mu * k.z + st * (cp * e1.z + sp * e2.z);
-  const float inv = rsqrtf(ko.x * ko.x + ko.y * ko.y + ko.z * ko.z);
-  return make_float3(ko.x * inv, ko.y * inv, ko.z * inv);
+  ko.x = sum(kForm & 8, mu, k.x, st, sum(kForm & 1, cp, e1.x, sp, e2.x));
+  ko.y = sum(kForm & 16, mu, k.y, st, sum(kForm & 2, cp, e1.y, sp, e2.y));
+  ko.z = sum(kForm & 32, mu, k.z, st, sum(kForm & 4, cp, e1.z, sp, e2.z));
+  const float inv = rsqrtf(mul_add(ko.z, ko.z, sum(!(kForm & 64), ko.x, ko.x, ko.y, ko.y)));
+  return make_float3(__fmul_rn(ko.x, inv), __fmul_rn(ko.y, inv), __fmul_rn(ko.z, inv));
 }
 
 // Eq. 7 without recoil: x_out = x - u_par + u . k_out, u . k_out = u_par mu + st (u1 cos phi
-// + u2 sin phi) (shared by scatter_resonant and the core bursts).
-__device__ __forceinline__ float x_after_scatter(float x, float upar, float mu, float st, float u1, float u2,
-                                                 float cp, float sp) {
-  const float perp = __fmul_rn(st, __fmaf_rn(u1, cp, __fmul_rn(u2, sp)));
+// + u2 sin phi); the perpendicular term does not depend on the frequency (shared by
+// scatter_resonant and the shell loop's core events).
+__device__ __forceinline__ float scatter_perp(float st, float u1, float u2, float cp, float sp) {
+  return __fmul_rn(st, __fmaf_rn(u1, cp, __fmul_rn(u2, sp)));
+}
+__device__ __forceinline__ float x_after_perp(float x, float upar, float mu, float perp) {
   return __fadd_rn(__fsub_rn(x, upar), __fmaf_rn(upar, mu, perp));
 }
+__device__ __forceinline__ float x_after_scatter(float x, float upar, float mu, float st, float u1, float u2,
+                                                 float cp, float sp) {
+  return x_after_perp(x, upar, mu, scatter_perp(st, u1, u2, cp, sp));
+}
 
+template <int kForm = kTurnPower, int kFormIso = kTurnPower>
 __device__ __forceinline__ float scatter_resonant(float x, float a, int phase, float3& k, const Rng& rng,
                                                   uint32_t& iters, AtomFrame* af, float xcrit = 0.0f) {
   const float xc = (fabsf(x) < xcrit) ? xcrit : 0.0f;
@@ -578,13 +604,13 @@ __device__ __forceinline__ float scatter_resonant(float x, float a, int phase, f
   float3 e1, e2;
   basis(k.x, k.y, k.z, e1, e2);
   float st = sqrt_approx(fmaxf(0.0f, __fmaf_rn(-mu, mu, 1.0f)));
-  float3 ko = turn(k, e1, e2, mu, st, cp, sp);
+  float3 ko = turn<kForm>(k, e1, e2, mu, st, cp, sp);
   const float upar = sample_upar(x, a, rng, iters);
   const bool core = fabsf(x - upar) < 0.2f;
   if (phase == PH_MIXED && core && rng.u(W_MIXED) < (1.0f / 3.0f)) {
     mu = __fmaf_rn(2.0f, Rm, -1.0f);
     st = sqrt_approx(fmaxf(0.0f, 1.0f - mu * mu));
-    ko = turn(k, e1, e2, mu, st, cp, sp);
+    ko = turn<kFormIso>(k, e1, e2, mu, st, cp, sp);
   }
   if (af) { af->upar = upar; af->u1 = u1; af->u2 = u2; af->e1 = e1; af->e2 = e2; af->core = core; }
   k = ko;
@@ -598,12 +624,7 @@ __device__ __forceinline__ void scatter_dust(float g, float3& k, const Rng& rng)
   float3 e1, e2;
   basis(k.x, k.y, k.z, e1, e2);
   const float st = sqrtf(fmaxf(0.0f, 1.0f - mu * mu));
-  float3 ko;
-  ko.x = mu * k.x + st * (cp * e1.x + sp * e2.x);
-  ko.y = mu * k.y + st * (cp * e1.y + sp * e2.y);
-  ko.z = mu * k.z + st * (cp * e1.z + sp * e2.z);
-  const float inv = rsqrtf(ko.x * ko.x + ko.y * ko.y + ko.z * ko.z);
-  k = make_float3(ko.x * inv, ko.y * inv, ko.z * inv);
+  k = turn<kTurnShell>(k, e1, e2, mu, st, cp, sp);
 }
 
 __device__ __forceinline__ float3 iso_dir(float Rmu, float Rphi) {

@@ -1,6 +1,7 @@
 // thor_grid.cu -- photon-packet loop on a uniform Cartesian grid (THOR Sec. 3.3-3.4.1):
 // field packing, emission CDF, DDA propagation with zeroth-order cells, interaction,
 // and peeling-off to three axis-aligned observers.
+#define THOR_SEPARATE_ROUNDING  // as this file's -fmad=false
 #include "thor_device.cuh"
 #include "thor_internal.h"
 

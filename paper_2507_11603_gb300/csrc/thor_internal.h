@@ -111,8 +111,8 @@ struct Compact {  // every field defaults to off / empty
   unsigned long long* n_spill = nullptr;
   int32_t spill_below = 0;  // 0: run to completion
   int32_t per_warp = 32;    // lanes per warp that take packets (1..32): few packets spread over all schedulers
-  int32_t core_lanes = 32;  // warps with at most this many live packets run pipelined events (0 = never)
-  int32_t burst_lanes = 1;  // ... and, with at most this many, core bursts (0 = never)
+  int32_t core_lanes = 32;  // warps with at most this many live packets run core events in rounds (0 = never)
+  int32_t burst_lanes = 1;  // ... and, with at most this many, up to 32 of them between general events
   // Work sharing in the tail of a one-launch run (pool = NULL: off).  Once the queue is
   // drained, a warp whose lanes are all done waits for a packet that a warp with several
   // live packets gives away, and runs it alone.

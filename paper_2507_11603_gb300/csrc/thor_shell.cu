@@ -16,8 +16,6 @@ namespace thor {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kServedPipeLanes = 32;  // served rounds: pipelined events in every warp
-constexpr int kServedBurstLanes = 1;  // served rounds: core bursts for lone packets
 constexpr uint32_t kLongLived = 1u << 14;
 constexpr uint32_t kPriBudget = 16;  // served rounds: budget multiple of a priority warp (one packet)  // served rounds: packets past this many events run one per warp
 
@@ -92,7 +90,7 @@ __device__ __forceinline__ float safe_distance(const ShellModel& m, const Photon
   return fmaxf(__double2float_rd(d) * 0.999999f, 0.0f);
 }
 
-// The start of a step, shared by shell_event's fast paths and the core bursts (one
+// The start of a step, shared by shell_event's fast paths and the core events in rounds (one
 // definition, so both evaluate an event bit for bit alike): H(a, x) from the table-free
 // polynomial in the core (|x| <= 2), else from the table; kH = kap0 H; the crossing at the
 // start-point rate s = tau / (kH + kapd); dust is chosen when R (kH + kapd) >= kH (the
@@ -244,7 +242,7 @@ __device__ int shell_event_words(const ShellModel& m, Photon& ph, const float* _
     return 0;
   }
   // Eq. 7: the gas-frame frequency after the scattering, at the same point
-  ph.x = scatter_resonant(x_site, m.a, m.phase, ph.k, ph.rng, ph.iters, nullptr, m.xcrit);
+  ph.x = scatter_resonant<kTurnShell, kTurnShellIso>(x_site, m.a, m.phase, ph.k, ph.rng, ph.iters, nullptr, m.xcrit);
   ++ph.nscat;
   if (m.max_scat && ph.nscat >= m.max_scat) {
     anchor(ph);
@@ -260,65 +258,81 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
   return shell_event_words(m, ph, Ktab, draw_tau(ph.rng));  // Eq. 3: tau ~ Exp(1)
 }
 
-// ---- pipelined events (homologous shells) -------------------------------------------
+// ---- core events in rounds (homologous shells) ---------------------------------------
 // A packet trapped in the line core spends its life in one kind of event: the crossing lies
 // within ds/16 of the start (start-point rate, Sec. 5.1 step limiter) inside the safety
 // ball, the interaction is a resonant scattering at |x| <= 2 (Sec. 3.4), and the u_par
 // sampler (Eq. 10) accepts within two trials.  In such an event only the frequency
-// chain x -> H(a,x) -> s -> x_site -> u_par -> x_out depends on the packet's state; the next
-// event's Philox blocks and optical depth, the perpendicular atom velocity (Eq. 5), mu and
-// the outgoing direction depend only on random words and the incoming direction.
-// shell_event_pipe evaluates that kind of event in one basic block, with the next event's
-// words formed beside the chain (a lone lane issues in order and would otherwise wait on
-// each link), and commits it only if the event is of that kind; otherwise it runs the
-// general event from the same words.  The general event evaluates these events with the
-// same helpers (voigt_start, start_step, dust_channel, u0_core, upar_q / atan_small,
-// region1, x_after_scatter), so both paths give bit-identical results.
-// In this mode ph.rng holds the words of the event about to run ("prepared"), and
-// tau_next its optical depth; pipe_prepare / pipe_unprepare switch between the modes.
-__device__ __forceinline__ void pipe_prepare(const ShellModel& m, Photon& ph, float& tau_next) {
-  ph.rng.next_event(shell_blocks(m));
-  tau_next = draw_tau(ph.rng);
-}
-__device__ __forceinline__ void pipe_unprepare(Photon& ph) { ph.rng.event -= 1u; }
-
-// The line-core form of the prepared event.  Always forms the next event's words and
-// optical depth (r2, tau2).  Returns 0 if the event is not of the core kind (the packet is
-// unchanged), 1 if it was committed, 3 if committed and the scattering cap was reached (the
-// packet is then finished as shell_event_words finishes it).  On commit the packet is
-// prepared for the next event.
-__device__ __forceinline__ int core_event_with(const ShellModel& m, Photon& ph, const float* __restrict__ Ktab,
-                                               float& tau_next, const Rng& r2, float tau2);
-__device__ __forceinline__ int core_event(const ShellModel& m, Photon& ph, const float* __restrict__ Ktab,
-                                          float& tau_next, Rng& r2, float& tau2) {
-  r2 = ph.rng;
-  r2.next_event(shell_blocks(m));
-  tau2 = draw_tau(r2);
-  return core_event_with(m, ph, Ktab, tau_next, r2, tau2);
-}
-// The core form of the prepared event, evaluated (nothing committed): the frequency chain,
-// the u_par sampler's first trial (and its second, when the first is rejected) and, beside
-// them, the perpendicular velocity, mu and the outgoing direction.  ok: the event is of the
-// core kind.
-struct CoreEval {
-  float s0, xs, upar, mu, st, u1, u2, cp, sp;
-  float3 ko;
-  uint32_t trials;  // u_par trials (one or two)
-  bool ok;
+// chain x -> H(a,x) -> s -> x_site -> u_par -> x_out depends on the packet's state; the
+// optical depth, the sampler's uniforms, the perpendicular atom velocity (Eq. 5), mu and the
+// azimuth are functions of the event's random words, which depend on nothing but the key,
+// the photon id and the event number.
+//
+// What bounds it: a run lasts as long as its longest photon (1e6 to 1e7 core events one after
+// another), so the time of one event in a warp with few packets is what counts, and that is
+// its instructions at the issue rate of a lone warp.  So the events run in rounds: all 32
+// lanes first evaluate everything that depends on words alone, one event of one packet
+// per lane, for the next D events of the warp's P packets (P D <= kChainSlots), into shared
+// memory; then the P lanes that own the packets run D events of the chain, each from one
+// 48-byte slot.  The general event evaluates these events with the same helpers
+// (start_step, dust_channel, u0_core, upar_q / atan_small, upar_trial, x_after_scatter) on
+// the same words, so both paths give bit-identical results.
+// Measured (GB300, 2070 MHz): a photon alone in a static sphere 0.36 us per event (0.47 us
+// when its own lane formed the directions' angles and the words came by shuffle); the
+// expanding shell of 1e5 photons at N_HI = 1e20 3.29 s (5.35 s).  The general events run for
+// all the packets that wait for one, at most once per `depth` core events: a general event
+// costs several core events, and one lane in sixty needs one at any time.
+constexpr int kChainSlots = 128;      // events per warp and round
+constexpr uint32_t kChainDepth = 32;  // ... and per packet, in warps with few packets
+constexpr uint32_t kCrowdDepth = 16;  // ... and per packet, in the others (kept until a general event runs)
+constexpr uint32_t kVoteEvents = 4;   // core events between two votes on whether any packet goes on
+struct ChainBuf {                     // one per warp
+  float4 a[kChainSlots];              // tau, R1, R2, R3
+  float4 b[kChainSlots];              // mu, st, perpendicular term (plain), channel uniform
+  float4 c[kChainSlots];              // cos phi, sin phi, perpendicular term (core-skipping), -
+  uint4 own[32];                      // photon id, last completed event, needs (owners in lane order)
+  uint4 key[32];                      // stream key, phase function, core-skipping threshold
 };
-// live = false: a lane of a cooperative burst without a packet in it; it evaluates at line
-// centre and skips the rare second trial, so that it takes the owners' branches.
-__device__ __forceinline__ CoreEval core_eval(const ShellModel& m, const Photon& ph, const float* __restrict__ Ktab,
-                                              float tau, bool live = true) {
-  const Rng& r = ph.rng;
-  CoreEval e;
+
+// A slot: what event e of photon (p0, p1) takes from its words (as start_event, draw_tau,
+// scatter_resonant and x_after_scatter form them).
+__device__ __forceinline__ void chain_slot(ChainBuf& cb, int s, const uint4& own, const uint4& key, uint32_t e) {
+  Rng r;
+  r.k0 = key.x; r.k1 = key.y; r.p0 = own.x; r.p1 = own.y;
+  r.start_event(e, (own.w & 1u) ? 3u : 2u);
+  float sp1, cp1, sp, cp;
+  __sincosf(2.0f * kPiF * r.u(W_BM_PHI), &sp1, &cp1);
+  __sincosf(2.0f * kPiF * r.u(W_PHI), &sp, &cp);
+  const float lr = __logf(r.u(W_BM_R));
+  const float Rm = r.u(W_MU);
+  const float mu = ((int)key.z == PH_ISO) ? __fmaf_rn(2.0f, Rm, -1.0f) : mu_dipole(Rm);
+  const float st = sqrt_approx(fmaxf(0.0f, __fmaf_rn(-mu, mu, 1.0f)));
+  auto perp = [&](float xc) {
+    const float rr = sqrt_approx(__fmaf_rn(xc, xc, -lr));
+    return scatter_perp(st, __fmul_rn(rr, cp1), __fmul_rn(rr, sp1), cp, sp);
+  };
+  cb.a[s] = make_float4(draw_tau(r), r.u(W_UPAR0), r.u(W_UPAR0 + 1), r.u(W_UPAR0 + 2));
+  cb.b[s] = make_float4(mu, st, perp(0.0f), (own.w & 1u) ? r.u(W_CHANNEL) : 0.0f);
+  cb.c[s] = make_float4(cp, sp, perp(__uint_as_float(key.w)), 0.0f);
+}
+
+// Whether the packet's next event may be of the core kind (the cheap part of the test).
+__device__ __forceinline__ bool chain_kind(const ShellModel& m, const Photon& ph) {
+  return !ph.region && m.phase != PH_MIXED && fabsf(ph.x) <= THOR_VCORE_X && (m.gam == 0.0f || ph.safe >= m.ds_core);
+}
+
+// One core event from its slot, committed where `go` holds and the event is of the core kind
+// (by selects: a loop body of one basic block but for the rare second trial).  Returns
+// whether it was committed.
+__device__ __forceinline__ bool chain_event(const ShellModel& m, Photon& ph, const float4& wa, const float4& wb,
+                                            const float4& wc, uint32_t e, bool go, uint32_t& second) {
   // ---- the frequency chain: rate at the start, crossing, gas-frame frequency at the site
-  const float x0 = live ? ph.x : 0.0f;
-  const StartStep st0 = start_step(m, voigt_start(m.a, x0, Ktab), tau);
+  const float x0 = go ? ph.x : 0.0f;  // lanes without a packet in the round take the owners' branches
+  const StartStep st0 = start_step(m, voigt_core_poly(m.a, x0), wa.x);
   const float s0 = st0.s;
   const bool in_ball = (m.gam == 0.0f) ? (s0 <= ph.safe) : (ph.safe >= m.ds_core && s0 <= 0.0625f * m.ds_core);
   const float xs = (m.gam == 0.0f) ? x0 : __fmaf_rn(-m.gam, s0, x0);
-  const bool dust = (m.kapd > 0.0f) && dust_channel(m, st0.kH, r.u(W_CHANNEL));
+  const bool dust = (m.kapd > 0.0f) && dust_channel(m, st0.kH, wb.w);
   // ---- u_par, first trial of the two-piece comparison function (as sample_upar)
   const float sgn = (xs < 0.0f) ? -1.0f : 1.0f;
   const float xr = fabsf(xs);
@@ -332,163 +346,101 @@ __device__ __forceinline__ CoreEval core_eval(const ShellModel& m, const Photon&
   const float mass = envelope_mass(w1, exp_fast(-u02));
   const float w1p = __fmul_rn(w1, 1.0f / kPiF);
   float u;
-  bool accepted = upar_trial(xr, m.a, w1, w1p, mass, u02, r.u(W_UPAR0), r.u(W_UPAR0 + 1), r.u(W_UPAR0 + 2), u);
-  e.trials = 1u;
-  if (!accepted && live) {  // rare: the second trial, from block 3 of the event as sample_upar takes it
+  bool accepted = upar_trial(xr, m.a, w1, w1p, mass, u02, wa.y, wa.z, wa.w, u);
+  const bool kind = go && fabsf(x0) <= THOR_VCORE_X && in_ball && !dust && xr <= 2.0f &&
+                    (split ? q <= 0.05f : m.a <= 0.05f * xr);
+  if (!accepted && kind) {  // rare: the second trial, from block 3 of the event as sample_upar takes it
+    Rng r = ph.rng;
+    r.event = e;
     uint32_t b0, b1, b2, b3;
     r.block(3u, b0, b1, b2, b3);
     accepted = upar_trial(xr, m.a, w1, w1p, mass, u02, uni32(b0), uni32(b1), uni32(b2), u);
-    e.trials = 2u;
+    second += accepted ? 1u : 0u;
   }
-  // ---- beside the chain: perpendicular velocity, mu, outgoing direction (as scatter_resonant)
-  const float xc = (xr < m.xcrit) ? m.xcrit : 0.0f;
-  const float rr = sqrt_approx(__fmaf_rn(xc, xc, -__logf(r.u(W_BM_R))));
-  float sp1, cp1;
-  __sincosf(2.0f * kPiF * r.u(W_BM_PHI), &sp1, &cp1);
-  e.u1 = __fmul_rn(rr, cp1);
-  e.u2 = __fmul_rn(rr, sp1);
-  const float Rm = r.u(W_MU);
-  e.mu = (m.phase == PH_ISO) ? __fmaf_rn(2.0f, Rm, -1.0f) : mu_dipole(Rm);
-  __sincosf(2.0f * kPiF * r.u(W_PHI), &e.sp, &e.cp);
+  const bool ok = kind && accepted;
+  // ---- beside the chain: the outgoing direction (as scatter_resonant)
   float3 e1, e2;
   basis(ph.k.x, ph.k.y, ph.k.z, e1, e2);
-  e.st = sqrt_approx(fmaxf(0.0f, __fmaf_rn(-e.mu, e.mu, 1.0f)));
-  e.ko = turn(ph.k, e1, e2, e.mu, e.st, e.cp, e.sp);
-  e.s0 = s0;
-  e.xs = xs;
-  e.upar = sgn * u;
-  e.ok = !ph.region && m.phase != PH_MIXED && in_ball && !dust && xr <= 2.0f &&
-         (split ? q <= 0.05f : m.a <= 0.05f * xr) && accepted;
-  return e;
-}
-// Commit an evaluated core event where `ok` (selects, no branch), as shell_event_words and
-// scatter_resonant do: the packet is then prepared with the next event's words r2 and
-// optical depth tau2.
-__device__ __forceinline__ void core_commit(Photon& ph, const CoreEval& e, bool ok, const Rng& r2, float tau2,
-                                            float& tau_next) {
-  ph.steps += ok ? 1u : 0u;
-  ph.ox = ok ? __fmaf_rn(e.s0, ph.k.x, ph.ox) : ph.ox;  // advance(ph, s0)
-  ph.oy = ok ? __fmaf_rn(e.s0, ph.k.y, ph.oy) : ph.oy;
-  ph.oz = ok ? __fmaf_rn(e.s0, ph.k.z, ph.oz) : ph.oz;
-  ph.safe = ok ? __fmaf_rd(-e.s0, 1.000001f, ph.safe) : ph.safe;
-  ph.x = ok ? x_after_scatter(e.xs, e.upar, e.mu, e.st, e.u1, e.u2, e.cp, e.sp) : ph.x;
-  ph.k.x = ok ? e.ko.x : ph.k.x;
-  ph.k.y = ok ? e.ko.y : ph.k.y;
-  ph.k.z = ok ? e.ko.z : ph.k.z;
-  ph.iters += ok ? e.trials : 0u;
-  ph.nscat += ok ? 1u : 0u;
-  ph.rng.event = ok ? r2.event : ph.rng.event;
-#pragma unroll
-  for (int j = 0; j < 12; ++j) ph.rng.v[j] = ok ? r2.v[j] : ph.rng.v[j];
-  tau_next = ok ? tau2 : tau_next;
-}
-// The same event with the next event's words (r2) and optical depth (tau2) given.
-__device__ __forceinline__ int core_event_with(const ShellModel& m, Photon& ph, const float* __restrict__ Ktab,
-                                               float& tau_next, const Rng& r2, float tau2) {
-  const CoreEval e = core_eval(m, ph, Ktab, tau_next);
-  if (!e.ok) return 0;
-  core_commit(ph, e, true, r2, tau2, tau_next);
-  if (m.max_scat && ph.nscat >= m.max_scat) {
-    anchor(ph);
-    const float b = (float)(ph.px * ph.k.x + ph.py * ph.k.y + ph.pz * ph.k.z);
-    ph.X = __fmaf_rn(ph.x, m.vth, m.vgrad * b);
-    return 3;
-  }
-  return 1;
+  const float3 ko = turn<kTurnShell>(ph.k, e1, e2, wb.x, wb.y, wc.x, wc.y);
+  // ---- commit
+  ph.ox = ok ? __fmaf_rn(s0, ph.k.x, ph.ox) : ph.ox;  // advance(ph, s0)
+  ph.oy = ok ? __fmaf_rn(s0, ph.k.y, ph.oy) : ph.oy;
+  ph.oz = ok ? __fmaf_rn(s0, ph.k.z, ph.oz) : ph.oz;
+  ph.safe = ok ? __fmaf_rd(-s0, 1.000001f, ph.safe) : ph.safe;
+  ph.x = ok ? x_after_perp(xs, sgn * u, wb.x, (xr < m.xcrit) ? wc.z : wb.z) : ph.x;
+  ph.k.x = ok ? ko.x : ph.k.x;
+  ph.k.y = ok ? ko.y : ph.k.y;
+  ph.k.z = ok ? ko.z : ph.k.z;
+  return ok;
 }
 
-// One prepared event: its core form if it is of that kind, else the general event from the
-// same words; the packet is then prepared for the next event.  Returns as shell_event.
-__device__ __forceinline__ int shell_event_pipe(const ShellModel& m, Photon& ph, const float* __restrict__ Ktab,
-                                                float& tau_next) {
-  Rng r2;
-  float tau2;
-  const int c = core_event(m, ph, Ktab, tau_next, r2, tau2);
-  if (c == 1) return 0;
-  if (c == 3) return 3;
-  const int status = shell_event_words(m, ph, Ktab, tau_next);
-  ph.rng = r2;
-  tau_next = tau2;
-  return status;
-}
-
-// A burst: core events of a prepared packet back to back, in one loop whose body is one
-// basic block (no vote or exchange between events), until an event is not of the core kind
-// (it is left prepared, for shell_event_pipe) or kCoreBurst events are done.  For warps with
-// few live packets, where a lone lane's latency is what counts.  Returns 3 if the cap was
-// reached, else 0.
-constexpr uint32_t kCoreBurst = 32;
-__device__ __forceinline__ int core_burst(const ShellModel& m, Photon& ph, const float* __restrict__ Ktab,
-                                          float& tau_next) {
-  for (uint32_t n = 0; n < kCoreBurst; ++n) {
-    Rng r2;
-    float tau2;
-    const int c = core_event(m, ph, Ktab, tau_next, r2, tau2);
-    if (c != 1) return c;  // 0: not a core event (still prepared); 3: capped
-  }
-  return 0;
-}
-
-// A cooperative burst, for warps with at most kCoopOwners packets in bursts.  Called by all
-// 32 lanes, converged; `mine` marks the lanes whose (prepared) packets burst.  In a core
-// event the next event's three Philox blocks are about half a lone lane's instructions, and
-// they depend on nothing but the key, the photon id and the event number.  So every lane
-// computes one block ahead -- for owner o, event d ahead, block b: D = 32 / (3 owners)
-// events deep -- and the owners take their words by shuffle, D events per round of blocks.
-// The words are the ones Rng::start_event forms, so the packets' histories are those of
-// core_burst, bit for bit.  Returns 0: a packet leaves the burst prepared, before its first
-// event that is not of the core kind, or one scattering short of the cap.
-constexpr int kCoopOwners = 10;
-__device__ __forceinline__ int core_burst_coop(const ShellModel& m, Photon& ph, const float* __restrict__ Ktab,
-                                               float& tau_next, bool mine) {
+// A round: up to `depth` core events of every packet in `mine` lanes (with its random words
+// formed by all lanes).  Called by all 32 lanes, converged.  Returns the events done; `stuck`
+// tells the lanes whose packet stopped before an event that is not of the core kind, or one
+// scattering short of the cap (shell_event runs that one).
+__device__ __forceinline__ uint32_t chain_round(const ShellModel& m, Photon& ph, ChainBuf& cb, bool mine,
+                                                uint32_t depth, bool& stuck) {
   const int lane = (int)(threadIdx.x & 31u);
   const unsigned owners = __ballot_sync(kFull, mine);
-  const int n_own = __popc(owners);
-  if (n_own == 0) return 0;
-  if (n_own > kCoopOwners) return mine ? core_burst(m, ph, Ktab, tau_next) : 0;
-  const int D = 32 / (3 * n_own);  // >= 1
-  const int span = 3 * D;
-  // as a block computer: owner rank oi (its lane src), event offset d, block b
-  const int oi = lane / span, rem = lane - oi * span;
-  const int d = rem / 3, b = rem - 3 * d;
-  unsigned o = owners;
-#pragma unroll
-  for (int k = 0; k < kCoopOwners - 1; ++k)
-    if (k < oi) o &= o - 1u;
-  const int src = o ? __ffs(o) - 1 : 0;  // lanes past the owners' spans compute a spare block
-  // as an owner: the first lane of its span
-  const int base = mine ? __popc(owners & ((1u << lane) - 1u)) * span : 0;
-  const bool b3 = shell_blocks(m) > 2u;  // else words 8..11 stay as start_event leaves them
-  // a burst stops one scattering short of the cap: the event that reaches it runs as
-  // shell_event_pipe (which finishes the packet)
-  const uint32_t room = m.max_scat ? (m.max_scat > ph.nscat + 1u ? m.max_scat - ph.nscat - 1u : 0u) : kCoreBurst;
-  bool go = mine && room > 0u;
-  for (uint32_t n = 0; n < kCoreBurst; n += (uint32_t)D) {
-    // a round of blocks: events e+1 .. e+D of each owner (e = its prepared event now)
-    const uint32_t k0 = __shfl_sync(kFull, ph.rng.k0, src), k1 = __shfl_sync(kFull, ph.rng.k1, src);
-    uint32_t h0 = __shfl_sync(kFull, ph.rng.p0, src), h1 = __shfl_sync(kFull, ph.rng.p1, src);
-    uint32_t h2 = __shfl_sync(kFull, ph.rng.event, src) + 1u + (uint32_t)d, h3 = (uint32_t)b;
-    philox10(h0, h1, h2, h3, k0, k1);
-    for (int i = 0; i < D && n + (uint32_t)i < kCoreBurst; ++i) {
-      const int s0 = base + 3 * i;
-      Rng r2 = ph.rng;
-      r2.event = ph.rng.event + 1u;
-      r2.v[0] = __shfl_sync(kFull, h0, s0); r2.v[1] = __shfl_sync(kFull, h1, s0);
-      r2.v[2] = __shfl_sync(kFull, h2, s0); r2.v[3] = __shfl_sync(kFull, h3, s0);
-      r2.v[4] = __shfl_sync(kFull, h0, s0 + 1); r2.v[5] = __shfl_sync(kFull, h1, s0 + 1);
-      r2.v[6] = __shfl_sync(kFull, h2, s0 + 1); r2.v[7] = __shfl_sync(kFull, h3, s0 + 1);
-      const uint32_t w8 = __shfl_sync(kFull, h0, s0 + 2), w9 = __shfl_sync(kFull, h1, s0 + 2);
-      const uint32_t w10 = __shfl_sync(kFull, h2, s0 + 2), w11 = __shfl_sync(kFull, h3, s0 + 2);
-      if (b3) { r2.v[8] = w8; r2.v[9] = w9; r2.v[10] = w10; r2.v[11] = w11; }
-      // every lane evaluates (the owners' events; garbage elsewhere, never committed) and
-      // commits by select: the loop body is one basic block
-      const CoreEval e = core_eval(m, ph, Ktab, tau_next, go);
-      go = go && e.ok && n + (uint32_t)i < room;
-      core_commit(ph, e, go, r2, draw_tau(r2), tau_next);
-      if (!__any_sync(kFull, go)) return 0;
-    }
+  const int P = __popc(owners);
+  const int rank = mine ? __popc(owners & ((1u << lane) - 1u)) : 0;
+  const int D = min((int)depth, kChainSlots / P);
+  if (mine) {
+    cb.own[rank] = make_uint4(ph.rng.p0, ph.rng.p1, ph.rng.event, m.kapd > 0.0f ? 1u : 0u);
+    cb.key[rank] = make_uint4(ph.rng.k0, ph.rng.k1, (uint32_t)m.phase, __float_as_uint(m.xcrit));
   }
-  return 0;
+  __syncwarp();
+  for (int s = lane; s < P * D; s += 32) {  // slot d P + r: event d of the owner of rank r
+    const int d = s / P, r = s - d * P;
+    const uint4 own = cb.own[r];
+    chain_slot(cb, s, own, cb.key[r], own.z + 1u + (uint32_t)d);
+  }
+  __syncwarp();
+  const uint32_t left = m.max_scat ? (m.max_scat > ph.nscat + 1u ? m.max_scat - ph.nscat - 1u : 0u) : (uint32_t)D;
+  const int lim = (int)min(left, (uint32_t)D);
+  bool go = mine;
+  uint32_t n = 0, second = 0;
+  int d = 0;
+  while (d < D) {
+    const int end = min(D, d + (int)kVoteEvents);
+#pragma unroll 1
+    for (; d < end; ++d) {
+      const int s = d * P + rank;
+      go = chain_event(m, ph, cb.a[s], cb.b[s], cb.c[s], ph.rng.event + 1u + (uint32_t)d, go && d < lim, second);
+      n += go ? 1u : 0u;
+    }
+    if (!__any_sync(kFull, go)) break;
+  }
+  __syncwarp();
+  if (mine) {
+    ph.rng.event += n;
+    ph.nscat += n;
+    ph.steps += n;
+    ph.iters += n + second;
+  }
+  stuck = mine && !go;
+  return n;
+}
+
+// Core events of a warp's packets until `depth` of them ran or the packet needs a general
+// event (`general` then stays set).  Several rounds where the slots of one do not reach
+// (P > kChainSlots / depth): the general events, which run for a few lanes at a time, come
+// once per `depth` events.  Returns this lane's events.
+__device__ __forceinline__ uint32_t core_events(const ShellModel& m, Photon& ph, ChainBuf& cb, bool active,
+                                                uint32_t depth, bool& general) {
+  uint32_t n = 0;
+  bool go = active && chain_kind(m, ph);
+  for (uint32_t d = 0; d < depth; ) {
+    const int P = __popc(__ballot_sync(kFull, go));
+    if (P == 0) break;
+    const uint32_t D = min(depth - d, (uint32_t)(kChainSlots / P));
+    bool stuck = false;
+    n += chain_round(m, ph, cb, go, D, stuck);
+    go = go && !stuck;
+    d += D;
+  }
+  general = active && !go;
+  return n;
 }
 
 // ---- power-law shells (Sec. 5.1) ---------------------------------------------------
@@ -728,6 +680,8 @@ __global__ void __launch_bounds__(256, 1) shell_run_kernel(const ShellModel* __r
                                                         Compact c, const float* __restrict__ gK) {
   __shared__ __align__(16) float sK[THOR_VOIGT_NINT * THOR_VOIGT_NCOEF];
   __shared__ ShellModel sm;
+  extern __shared__ __align__(16) unsigned char dyn[];
+  ChainBuf& cb = reinterpret_cast<ChainBuf*>(dyn)[kProfile ? 0 : threadIdx.x >> 5];  // not touched on power laws
   load_ktab(sK, gK);
   if (threadIdx.x == 0) sm = models[q.model[0]];
   __syncthreads();
@@ -736,8 +690,6 @@ __global__ void __launch_bounds__(256, 1) shell_run_kernel(const ShellModel* __r
   Photon ph;
   bool active = false, done = (int)lane >= c.per_warp;  // lanes above per_warp stay idle
   bool drained = false;  // warp-uniform: a refill found the photon queue exhausted
-  bool prepared = false;  // ph.rng holds the words of the next event (pipelined mode)
-  float tau_next = 0.0f;
   LaneTally lt;
   for (;;) {
     unsigned need = __ballot_sync(kFull, !active && !done);
@@ -748,7 +700,7 @@ __global__ void __launch_bounds__(256, 1) shell_run_kernel(const ShellModel* __r
       base = __shfl_sync(kFull, base, leader);
       if (!active && !done) {
         const unsigned long long g = base + __popc(need & ((1u << lane) - 1u));
-        if (g < c.n_resume) { load_rec(m, c.resume[g], ph); active = true; prepared = false; }
+        if (g < c.n_resume) { load_rec(m, c.resume[g], ph); active = true; }
       }
       need = __ballot_sync(kFull, !active && !done);
     }
@@ -765,7 +717,6 @@ __global__ void __launch_bounds__(256, 1) shell_run_kernel(const ShellModel* __r
           ph.pid = q.first_id[0] + g;
           shell_emit(m, ph);
           active = true;
-          prepared = false;
         } else {
           done = true;
         }
@@ -779,7 +730,6 @@ __global__ void __launch_bounds__(256, 1) shell_run_kernel(const ShellModel* __r
           unsigned long long base = 0;
           if ((int)lane == leader) base = atomicAdd(c.n_spill, (unsigned long long)__popc(live));
           base = __shfl_sync(kFull, base, leader);
-          if (active && prepared) pipe_unprepare(ph);
           if (active) save_rec(ph, c.spill[base + __popc(live & ((1u << lane) - 1u))]);
         }
         active = false;
@@ -793,7 +743,7 @@ __global__ void __launch_bounds__(256, 1) shell_run_kernel(const ShellModel* __r
         if (lane == 0) got = share_take(c);
         got = __shfl_sync(kFull, got, 0);
         if (got < 0) break;
-        if (lane == 0) { load_rec(m, c.pool[got], ph); active = true; prepared = false; }
+        if (lane == 0) { load_rec(m, c.pool[got], ph); active = true; }
         continue;
       }
       if (__popc(live) >= 2) {  // give packets away while empty warps wait, keeping the lowest lane's
@@ -810,7 +760,6 @@ __global__ void __launch_bounds__(256, 1) shell_run_kernel(const ShellModel* __r
           base = __shfl_sync(kFull, base, leader);
           if (giver) {
             const unsigned long long j = base + (unsigned long long)from_top;
-            if (prepared) { pipe_unprepare(ph); prepared = false; }
             save_rec(ph, c.pool[j]);
             __threadfence();
             *(volatile uint32_t*)&c.ready[j] = 1u;
@@ -820,45 +769,41 @@ __global__ void __launch_bounds__(256, 1) shell_run_kernel(const ShellModel* __r
       }
     }
     if (__all_sync(kFull, !active)) break;
-    // pipelined events in warps with at most core_lanes live packets (homologous shells),
-    // and core bursts in warps with at most burst_lanes
     const int n_live = __popc(__ballot_sync(kFull, active));
     const bool check_share = c.pool && drained && n_live >= 2;
+    const bool chain = kProfile == 0 && n_live <= c.core_lanes;
+    const uint32_t depth = n_live <= c.burst_lanes || n_live <= kChainSlots / (int)kChainDepth ? kChainDepth : kCrowdDepth;
     uint32_t n_ev = 0;
-    const bool pipe = kProfile == 0 && n_live <= c.core_lanes;
-    const bool burst = pipe && n_live <= c.burst_lanes;
-    // events until some lane of the warp finishes its packet: one vote per event, the
-    // refill and spill checks above run only when the set of live lanes changed
-    // (bursts are cooperative up to kCoopOwners live packets: all lanes, converged)
+    // events until some lane of the warp finishes its packet: the refill and spill checks
+    // above run only when the set of live lanes changed
     bool fin;
     do {
       fin = false;
-      int st = 0;
-      if (burst) {
-        if (active && !prepared) { pipe_prepare(m, ph, tau_next); prepared = true; }
-        st = core_burst_coop(m, ph, sK, tau_next, active);
-      }
-      if (active) {
-        if (pipe) {
-          if (!prepared) { pipe_prepare(m, ph, tau_next); prepared = true; }
-          if (!st) st = shell_event_pipe(m, ph, sK, tau_next);
-        } else {
-          if (prepared) { pipe_unprepare(ph); prepared = false; }
-          st = kProfile ? shell_event_pl(m, ph, sK) : shell_event(m, ph, sK);
+      bool general = active;  // lanes whose next event is a general one
+      if (chain) core_events(m, ph, cb, active, depth, general);
+      // packets whose next event is not of the core kind take general events: one, and more
+      // while at least half of the warp's packets need them
+      uint32_t n_gen = 0;
+      do {
+        if (general) {
+          const int st = kProfile ? shell_event_pl(m, ph, sK) : shell_event(m, ph, sK);
+          if (st) {
+            if (st == 1) { ++lt.esc; tally_spectrum(m, ph.X); }
+            else if (st == 2) ++lt.abs;
+            else ++lt.cap;
+            lt.scat += ph.nscat; lt.dust += ph.ndust; lt.iters += ph.iters; lt.steps += ph.steps; ++lt.done;
+            lt.scat2 += (double)ph.nscat * (double)ph.nscat;
+            write_raw(m, ph, st);
+            if (c.pool) atomicAdd(&c.share[3], 1ull);
+            active = false;
+            fin = true;
+          }
+          general = active && !(chain && chain_kind(m, ph));
         }
-        if (st) {
-          if (st == 1) { ++lt.esc; tally_spectrum(m, ph.X); }
-          else if (st == 2) ++lt.abs;
-          else ++lt.cap;
-          lt.scat += ph.nscat; lt.dust += ph.ndust; lt.iters += ph.iters; lt.steps += ph.steps; ++lt.done;
-          lt.scat2 += (double)ph.nscat * (double)ph.nscat;
-          write_raw(m, ph, st);
-          if (c.pool) atomicAdd(&c.share[3], 1ull);
-          active = false;
-          fin = true;
-        }
-      }
-    } while (!__any_sync(kFull, fin) && !(check_share && ++n_ev >= kShareEvents));
+      } while (!__any_sync(kFull, fin) && ++n_gen < kCrowdDepth &&
+               2 * __popc(__ballot_sync(kFull, general)) >= n_live);
+      n_ev += chain ? depth : n_gen;
+    } while (!__any_sync(kFull, fin) && !(check_share && n_ev >= kShareEvents));
   }
   // flush lane tallies: warp reduce, one atomic per warp and field
   const unsigned long long e = warp_sum(lt.esc), a = warp_sum(lt.abs), cp = warp_sum(lt.cap),
@@ -891,6 +836,8 @@ __global__ void __launch_bounds__(256, 1) shell_slice_kernel(const ShellModel* _
                                                           SlotState in, SlotState out, uint32_t budget,
                                                           const float* __restrict__ gK) {
   __shared__ __align__(16) float sK[THOR_VOIGT_NINT * THOR_VOIGT_NCOEF];
+  extern __shared__ __align__(16) unsigned char dyn[];
+  ChainBuf& cb = reinterpret_cast<ChainBuf*>(dyn)[threadIdx.x >> 5];
   load_ktab(sK, gK);
   int per_warp = 32;  // at most this many live packets per warp after a refill
   if (q.hdr) {
@@ -932,8 +879,6 @@ __global__ void __launch_bounds__(256, 1) shell_slice_kernel(const ShellModel* _
   }
   Photon ph;
   bool active = false, done = false;
-  bool prepared = false;  // ph.rng holds the words of the next event (pipelined mode)
-  float tau_next = 0.0f;
   const SlotState& st = in;
   if (slot >= 0) {
     ph.model = st.model[slot];
@@ -972,7 +917,6 @@ __global__ void __launch_bounds__(256, 1) shell_slice_kernel(const ShellModel* _
           ph.pid = q.first_id[e] + (g - q.prefix[e]);
           shell_emit(models[ph.model], ph);
           active = true;
-          prepared = false;
         } else {
           done = true;
         }
@@ -990,39 +934,31 @@ __global__ void __launch_bounds__(256, 1) shell_slice_kernel(const ShellModel* _
     }
     if (__any_sync(kFull, dropped)) { ++ev; continue; }  // refill the dropped lanes first
     const ShellModel mr = *mp;  // by value: the fields the event loop reads stay in registers
-    // events until some lane finishes its packet or the budget is used: one vote per event;
-    // homologous shells run pipelined events in warps with at most kServedPipeLanes live
-    // packets
+    // events until some lane finishes its packet or the budget is used (a warp is charged the
+    // events of the lane that ran most of them)
     const int n_live = __popc(__ballot_sync(kFull, active));
-    const bool pipe = n_live <= kServedPipeLanes;
-    const bool burst = n_live <= kServedBurstLanes;
+    const bool chain = !(kMixed && mr.profile);  // this lane's packet runs core events in rounds
     bool fin;
     do {
       fin = false;
-      uint32_t nb = 0;
-      int r = 0;
-      const bool pl = pipe && !(kMixed && mr.profile);  // this lane's packet runs pipelined events
-      if (burst && budget - ev > kCoreBurst) {  // cooperative burst: all lanes, converged
-        if (active && pl && !prepared) { pipe_prepare(mr, ph, tau_next); prepared = true; }
-        const uint32_t before = ph.nscat;
-        r = core_burst_coop(mr, ph, sK, tau_next, active && pl);
-        if (active && pl) nb = ph.nscat - before;
-      }
-      if (active) {
-        if (pl) {
-          if (!prepared) { pipe_prepare(mr, ph, tau_next); prepared = true; }
-          if (!r) r = shell_event_pipe(mr, ph, sK, tau_next);
-        } else {
-          if (prepared) { pipe_unprepare(ph); prepared = false; }
-          r = (kMixed && mr.profile) ? shell_event_pl(mr, ph, sK) : shell_event(mr, ph, sK);
+      bool general = active;
+      const uint32_t depth = min(n_live <= kChainSlots / (int)kChainDepth ? kChainDepth : kCrowdDepth, budget - ev);
+      uint32_t n = core_events(mr, ph, cb, active && chain, depth, general);
+      if (kMixed) general = general || (active && !chain);
+      uint32_t n_gen = 0;
+      do {
+        if (general) {
+          const int r = (kMixed && mr.profile) ? shell_event_pl(mr, ph, sK) : shell_event(mr, ph, sK);
+          ++n;
+          if (r) { finish_global(mr, ph, r); active = false; fin = true; }
+          general = active && !(chain && chain_kind(mr, ph));
         }
-        if (r) { finish_global(mr, ph, r); active = false; fin = true; }
-      }
-      ev += 1u + __reduce_max_sync(kFull, nb);  // a burst is charged its events
+      } while (!__any_sync(kFull, fin) && ++n_gen < kCrowdDepth && n_gen + depth < budget - ev &&
+               2 * __popc(__ballot_sync(kFull, general)) >= n_live);
+      ev += max(1u, __reduce_max_sync(kFull, n));
     } while (ev < budget && !__any_sync(kFull, fin) && !others_done());
   }
   if (!pri_warp && lane == 0) atomicAdd(&in.live[4], 1ull);  // this regular warp's round is over
-  if (active && prepared) pipe_unprepare(ph);  // saved packets hold their last completed event
   // append the packets still in flight to the next list (one atomic per warp and list):
   // priority packets from the back, the others from the front.  Priority: packets of the
   // requests the host marked (the oldest), and long-lived packets (more than kLongLived
@@ -1059,7 +995,7 @@ __global__ void __launch_bounds__(256, 1) shell_slice_kernel(const ShellModel* _
 // front list of `from` (from.live[1] packets) is copied into `to` by bucket -- line core
 // (|x| <= 2), near wing (|x| <= 5), far wing, empty cavity -- and the resume hands each warp
 // contiguous entries, so a warp's packets are of one kind (core packets then run the
-// pipelined core events in step, wing packets the general event).  The back (priority)
+// core events in step, wing packets the general event).  The back (priority)
 // list is copied in place.  cnt[0..3]: bucket sizes, cnt[4..7]: cursors, zero on entry.
 // The order inside a bucket does not matter: a packet's history does not depend on its
 // warp or lane.
@@ -1113,12 +1049,24 @@ cudaError_t launch_slot_presort(SlotState from, SlotState to, unsigned long long
   return cudaGetLastError();
 }
 
+// Shared memory of a block: one round buffer per warp (homologous shells).
+static size_t chain_bytes(int block) { return (size_t)(block / 32) * sizeof(ChainBuf); }
+template <class F>
+static cudaError_t allow_chain(F* f) {  // 57 KB for the largest block: above the default limit
+  return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chain_bytes(256));
+}
+
 int shell_grid(int block, int blocks_per_sm, bool sliced) {
   int dev = 0, sms = 0, occ = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (sliced) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, shell_slice_kernel<true>, block, 0);
-  else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, shell_run_kernel<true, 0>, block, 0);
+  allow_chain(shell_slice_kernel<true>);
+  allow_chain(shell_slice_kernel<false>);
+  allow_chain(shell_run_kernel<true, 0>);
+  allow_chain(shell_run_kernel<false, 0>);
+  const size_t smem = chain_bytes(block);
+  if (sliced) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, shell_slice_kernel<true>, block, smem);
+  else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, shell_run_kernel<true, 0>, block, smem);
   if (occ < 1) occ = 1;
   const int b = (blocks_per_sm > 0 && blocks_per_sm < occ) ? blocks_per_sm : occ;
   return sms * b;
@@ -1138,21 +1086,22 @@ cudaError_t launch_shell_run(const ShellModel* d_models, WorkQueue q, const floa
   none.core_lanes = core_lanes;
   none.burst_lanes = burst_lanes;
   if (profile) shell_run_kernel<false, 1><<<grid, block, 0, s>>>(d_models, q, none, d_ktab);
-  else shell_run_kernel<false, 0><<<grid, block, 0, s>>>(d_models, q, none, d_ktab);
+  else shell_run_kernel<false, 0><<<grid, block, chain_bytes(block), s>>>(d_models, q, none, d_ktab);
   return cudaGetLastError();
 }
 
 cudaError_t launch_shell_run_compact(const ShellModel* d_models, WorkQueue q, Compact c, const float* d_ktab,
                                      int grid, int block, int profile, cudaStream_t s) {
   if (profile) shell_run_kernel<true, 1><<<grid, block, 0, s>>>(d_models, q, c, d_ktab);
-  else shell_run_kernel<true, 0><<<grid, block, 0, s>>>(d_models, q, c, d_ktab);
+  else shell_run_kernel<true, 0><<<grid, block, chain_bytes(block), s>>>(d_models, q, c, d_ktab);
   return cudaGetLastError();
 }
 
 cudaError_t launch_shell_slice(const ShellModel* d_models, WorkQueue q, SlotState in, SlotState out, uint32_t budget,
                                const float* d_ktab, int grid, int block, bool mixed, cudaStream_t s) {
-  if (mixed) shell_slice_kernel<true><<<grid, block, 0, s>>>(d_models, q, in, out, budget, d_ktab);
-  else shell_slice_kernel<false><<<grid, block, 0, s>>>(d_models, q, in, out, budget, d_ktab);
+  const size_t smem = chain_bytes(block);
+  if (mixed) shell_slice_kernel<true><<<grid, block, smem, s>>>(d_models, q, in, out, budget, d_ktab);
+  else shell_slice_kernel<false><<<grid, block, smem, s>>>(d_models, q, in, out, budget, d_ktab);
   return cudaGetLastError();
 }
 

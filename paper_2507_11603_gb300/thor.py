@@ -280,9 +280,9 @@ class Context:
         self._check(self.L.thor_ctx_set_launch(self.h, block_size, blocks_per_sm))
 
     def set_bursts(self, pipe_lanes: int = 32, burst_lanes: int = 1):
-        """thor_ctx_set_bursts: pipelined events in warps with at most pipe_lanes live packets,
-        core bursts in warps with at most burst_lanes (0 = never); results do not depend on
-        them."""
+        """thor_ctx_set_bursts: core events in rounds in warps with at most pipe_lanes live
+        packets (0 = never), longer rounds in warps with at most burst_lanes; results do not
+        depend on them."""
         self._check(self.L.thor_ctx_set_bursts(self.h, pipe_lanes, burst_lanes))
 
     def set_grid_exec(self, slots: int = 0, handoff: int | None = None):
