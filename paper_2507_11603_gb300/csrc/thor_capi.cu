@@ -205,6 +205,7 @@ static int fill_power_law(ErrSink err, const thor_shell_params* p, ShellModel* m
   m->profile = THOR_PROFILE_POWER_LAW;
   m->R_in = ri;
   m->R_out = 1.0;
+  shell_record_radii(m);
   m->kapn = (float)(tau0 / F);
   m->kapdn = (float)(p->tau_dust / F);
   m->invF = (float)(1.0 / F);
@@ -275,6 +276,7 @@ int thor::shell_model_from_params(ErrSink err, const thor_shell_params* p, Shell
   std::memset(m, 0, sizeof(*m));
   m->R_in = p->R_in / p->R_out;
   m->R_out = 1.0;
+  shell_record_radii(m);
   m->kap0 = (float)(tau0 / L);
   m->kapd = (float)(p->tau_dust / L);
   const double vth = line_vth_kms(p->T);

@@ -106,16 +106,23 @@ __device__ __forceinline__ float uni32(uint32_t w) {
 // starts, at one uniform code point; they are read by constant index only, so they stay
 // in registers.  Later blocks (extra rejection iterations) are generated on demand.
 // The event index is the whole stream state between events.
-struct Rng {
+struct StreamKey {
   uint32_t k0, k1, p0, p1;  // key, photon id
   uint32_t event;           // current event
-  uint32_t v[12];           // words 0..11 of the current event (the preloaded blocks)
 
   __device__ __forceinline__ void block(uint32_t j, uint32_t& a, uint32_t& b, uint32_t& c, uint32_t& d) const {
     uint32_t c0 = p0, c1 = p1, c2 = event, c3 = j;
     philox10(c0, c1, c2, c3, k0, k1);
     a = c0; b = c1; c = c2; d = c3;
   }
+  __device__ __forceinline__ void keys(uint64_t seed, uint64_t pid) {
+    k0 = (uint32_t)seed; k1 = (uint32_t)(seed >> 32);
+    p0 = (uint32_t)pid; p1 = (uint32_t)(pid >> 32);
+  }
+};
+struct Rng : StreamKey {
+  uint32_t v[12];           // words 0..11 of the current event (the preloaded blocks)
+
   // nblk = 1, 2 or 3 blocks preloaded: 2 cover a resonant or dust event without the
   // channel, albedo and mixed-phase words
   __device__ __forceinline__ void start_event(uint32_t e, uint32_t nblk) {
@@ -123,10 +130,6 @@ struct Rng {
     block(0u, v[0], v[1], v[2], v[3]);
     if (nblk > 1u) block(1u, v[4], v[5], v[6], v[7]);
     if (nblk > 2u) block(2u, v[8], v[9], v[10], v[11]);
-  }
-  __device__ __forceinline__ void keys(uint64_t seed, uint64_t pid) {
-    k0 = (uint32_t)seed; k1 = (uint32_t)(seed >> 32);
-    p0 = (uint32_t)pid; p1 = (uint32_t)(pid >> 32);
   }
   __device__ __forceinline__ void init(uint64_t seed, uint64_t pid, uint32_t nblk) {
     keys(seed, pid);
@@ -434,7 +437,8 @@ __device__ __forceinline__ WingSplit wing_split(float xr, float a) {
   const float b2 = (top_mass(xr, a, b1, c1) <= top_mass(xr, a, b1, u)) ? c1 : u;
   return WingSplit{ub, b1, b2};
 }
-static __device__ __noinline__ UparDraw sample_upar_wing(float xr, float a, Rng rng) {
+static __device__ __noinline__ UparDraw sample_upar_wing(float xr, float a, float F1, float F2, float F3,
+                                                         StreamKey key) {
   uint32_t iters = 0;
   const WingSplit sp = wing_split(xr, a);
   const float ub = sp.ub, b1 = sp.b1, b2 = sp.b2;
@@ -449,8 +453,8 @@ static __device__ __noinline__ UparDraw sample_upar_wing(float xr, float a, Rng 
   const float mG = a * 1.7724538509f / gden, m1 = e1 * d1, m2 = e2 * d2, m3 = e3 * (kPiF - al2);
   const float c1 = mG + m1, c2 = c1 + m2, tot = c2 + m3;
   const float sub = ub * ub, sb1 = b1 * b1, sb2 = b2 * b2;
-  auto trial = [&](uint32_t r1, uint32_t r2, uint32_t r3, float& u) {
-    const float R1 = uni32(r1) * tot, R2 = uni32(r2), R3 = uni32(r3);
+  auto trial = [&](float q1, float R2, float R3, float& u) {
+    const float R1 = q1 * tot;
     ++iters;
     if (R1 < mG) {  // Gaussian piece
       u = erfinvf(__fmaf_rn(2.0f, R2, -1.0f));
@@ -466,20 +470,22 @@ static __device__ __noinline__ UparDraw sample_upar_wing(float xr, float a, Rng 
     return R3 <= __expf(sh - u * u);
   };
   float u;
-  if (!trial(rng.v[W_UPAR0], rng.v[W_UPAR0 + 1], rng.v[W_UPAR0 + 2], u)) {
+  if (!trial(F1, F2, F3, u)) {
     uint32_t r1, r2, r3, spare, blk = 3u;
     do {
-      rng.block(blk++, r1, r2, r3, spare);
-    } while (!trial(r1, r2, r3, u) && blk < 2u + kMaxUparTrials);
+      key.block(blk++, r1, r2, r3, spare);
+    } while (!trial(uni32(r1), uni32(r2), uni32(r3), u) && blk < 2u + kMaxUparTrials);
   }
   return UparDraw{u, iters};
 }
 
-__device__ __forceinline__ float sample_upar(float x, float a, const Rng& rng, uint32_t& iters) {
+// R1..R3: the uniforms of the first trial; further trials take theirs from `key`.
+__device__ __forceinline__ float sample_upar(float x, float a, float R1, float R2, float R3, const StreamKey& key,
+                                             uint32_t& iters) {
   const float sgn = (x < 0.0f) ? -1.0f : 1.0f;
   const float xr = fabsf(x);
   if (xr > kUparWing) {
-    const UparDraw d = sample_upar_wing(xr, a, rng);
+    const UparDraw d = sample_upar_wing(xr, a, R1, R2, R3, key);
     iters += d.trials;
     return sgn * d.u;
   }
@@ -491,18 +497,21 @@ __device__ __forceinline__ float sample_upar(float x, float a, const Rng& rng, u
   const float e0 = exp_fast(-u02);
   const float mass = envelope_mass(w1, e0);
   const float w1p = __fmul_rn(w1, 1.0f / kPiF);  // alpha in units of pi
-  auto trial = [&](uint32_t r1, uint32_t r2, uint32_t r3, float& u) {
+  auto trial = [&](float q1, float q2, float q3, float& u) {
     ++iters;
-    return upar_trial(xr, a, w1, w1p, mass, u02, uni32(r1), uni32(r2), uni32(r3), u);
+    return upar_trial(xr, a, w1, w1p, mass, u02, q1, q2, q3, u);
   };
   float u;
-  if (!trial(rng.v[W_UPAR0], rng.v[W_UPAR0 + 1], rng.v[W_UPAR0 + 2], u)) {
+  if (!trial(R1, R2, R3, u)) {
     uint32_t r1, r2, r3, spare, blk = 3u;
     do {
-      rng.block(blk++, r1, r2, r3, spare);
-    } while (!trial(r1, r2, r3, u) && blk < 2u + kMaxUparTrials);
+      key.block(blk++, r1, r2, r3, spare);
+    } while (!trial(uni32(r1), uni32(r2), uni32(r3), u) && blk < 2u + kMaxUparTrials);
   }
   return sgn * u;
+}
+__device__ __forceinline__ float sample_upar(float x, float a, const Rng& rng, uint32_t& iters) {
+  return sample_upar(x, a, rng.u(W_UPAR0), rng.u(W_UPAR0 + 1), rng.u(W_UPAR0 + 2), rng, iters);
 }
 
 // Phase functions (Sec. 2.3.1 resonant, Sec. 2.3.2 dust, Eq. 9): mu = k_in . k_out.
@@ -589,42 +598,71 @@ __device__ __forceinline__ float x_after_scatter(float x, float upar, float mu, 
   return x_after_perp(x, upar, mu, scatter_perp(st, u1, u2, cp, sp));
 }
 
+// What an event takes from its random words: functions of the words, the phase function and
+// the core-skipping threshold alone, so they can be formed ahead of the event and by any lane.
+struct EventWords {
+  float tau;                  // optical depth to the interaction (Eq. 3)
+  float R1, R2, R3;           // u_par sampler, first trial: region, angle, acceptance
+  float mu, st, cp, sp;       // dipole (or isotropic) mu, sqrt(1 - mu^2), azimuth
+  float u1, u2, v1, v2;       // perpendicular atom velocity, plain and truncated at xcrit
+  float Rm;                   // the uniform of mu
+  float channel, mixed, albedo;
+};
+// words of a resonant scattering (all but tau)
+__device__ __forceinline__ void scatter_words(EventWords& w, const Rng& rng, int phase, float xcrit) {
+  w.R1 = rng.u(W_UPAR0); w.R2 = rng.u(W_UPAR0 + 1); w.R3 = rng.u(W_UPAR0 + 2);
+  const float lr = __logf(rng.u(W_BM_R));
+  float s1, c1;
+  __sincosf(2.0f * kPiF * rng.u(W_BM_PHI), &s1, &c1);
+  const float r = sqrt_approx(-lr), rv = sqrt_approx(__fmaf_rn(xcrit, xcrit, -lr));
+  w.u1 = __fmul_rn(r, c1); w.u2 = __fmul_rn(r, s1);
+  w.v1 = __fmul_rn(rv, c1); w.v2 = __fmul_rn(rv, s1);
+  w.Rm = rng.u(W_MU);
+  w.mu = (phase == PH_ISO) ? __fmaf_rn(2.0f, w.Rm, -1.0f) : mu_dipole(w.Rm);
+  w.st = sqrt_approx(fmaxf(0.0f, __fmaf_rn(-w.mu, w.mu, 1.0f)));
+  __sincosf(2.0f * kPiF * rng.u(W_PHI), &w.sp, &w.cp);
+  w.mixed = rng.u(W_MIXED);
+}
+
 template <int kForm = kTurnPower, int kFormIso = kTurnPower>
-__device__ __forceinline__ float scatter_resonant(float x, float a, int phase, float3& k, const Rng& rng,
-                                                  uint32_t& iters, AtomFrame* af, float xcrit = 0.0f) {
-  const float xc = (fabsf(x) < xcrit) ? xcrit : 0.0f;
-  const float r = sqrt_approx(__fmaf_rn(xc, xc, -__logf(rng.u(W_BM_R))));
-  float sp1, cp1;
-  __sincosf(2.0f * kPiF * rng.u(W_BM_PHI), &sp1, &cp1);
-  const float u1 = __fmul_rn(r, cp1), u2 = __fmul_rn(r, sp1);
-  const float Rm = rng.u(W_MU);
-  float mu = (phase == PH_ISO) ? __fmaf_rn(2.0f, Rm, -1.0f) : mu_dipole(Rm);
-  float sp, cp;
-  __sincosf(2.0f * kPiF * rng.u(W_PHI), &sp, &cp);
+__device__ __forceinline__ float scatter_resonant(float x, float a, int phase, float3& k, const EventWords& w,
+                                                  const StreamKey& key, uint32_t& iters, AtomFrame* af,
+                                                  float xcrit = 0.0f) {
+  const bool skip = fabsf(x) < xcrit;
+  const float u1 = skip ? w.v1 : w.u1, u2 = skip ? w.v2 : w.u2;
+  float mu = w.mu, st = w.st;
   float3 e1, e2;
   basis(k.x, k.y, k.z, e1, e2);
-  float st = sqrt_approx(fmaxf(0.0f, __fmaf_rn(-mu, mu, 1.0f)));
-  float3 ko = turn<kForm>(k, e1, e2, mu, st, cp, sp);
-  const float upar = sample_upar(x, a, rng, iters);
+  float3 ko = turn<kForm>(k, e1, e2, mu, st, w.cp, w.sp);
+  const float upar = sample_upar(x, a, w.R1, w.R2, w.R3, key, iters);
   const bool core = fabsf(x - upar) < 0.2f;
-  if (phase == PH_MIXED && core && rng.u(W_MIXED) < (1.0f / 3.0f)) {
-    mu = __fmaf_rn(2.0f, Rm, -1.0f);
+  if (phase == PH_MIXED && core && w.mixed < (1.0f / 3.0f)) {
+    mu = __fmaf_rn(2.0f, w.Rm, -1.0f);
     st = sqrt_approx(fmaxf(0.0f, 1.0f - mu * mu));
-    ko = turn<kFormIso>(k, e1, e2, mu, st, cp, sp);
+    ko = turn<kFormIso>(k, e1, e2, mu, st, w.cp, w.sp);
   }
   if (af) { af->upar = upar; af->u1 = u1; af->u2 = u2; af->e1 = e1; af->e2 = e2; af->core = core; }
   k = ko;
-  return x_after_scatter(x, upar, mu, st, u1, u2, cp, sp);
+  return x_after_scatter(x, upar, mu, st, u1, u2, w.cp, w.sp);
+}
+__device__ __forceinline__ float scatter_resonant(float x, float a, int phase, float3& k, const Rng& rng,
+                                                  uint32_t& iters, AtomFrame* af) {
+  EventWords w;
+  scatter_words(w, rng, phase, 0.0f);
+  return scatter_resonant(x, a, phase, k, w, rng, iters, af);
 }
 
-__device__ __forceinline__ void scatter_dust(float g, float3& k, const Rng& rng) {
-  const float mu = mu_hg(rng.u(W_MU), g);
-  float sp, cp;
-  __sincosf(2.0f * kPiF * rng.u(W_PHI), &sp, &cp);
+__device__ __forceinline__ void scatter_dust(float g, float3& k, float Rm, float cp, float sp) {
+  const float mu = mu_hg(Rm, g);
   float3 e1, e2;
   basis(k.x, k.y, k.z, e1, e2);
   const float st = sqrtf(fmaxf(0.0f, 1.0f - mu * mu));
   k = turn<kTurnShell>(k, e1, e2, mu, st, cp, sp);
+}
+__device__ __forceinline__ void scatter_dust(float g, float3& k, const Rng& rng) {
+  float sp, cp;
+  __sincosf(2.0f * kPiF * rng.u(W_PHI), &sp, &cp);
+  scatter_dust(g, k, rng.u(W_MU), cp, sp);
 }
 
 __device__ __forceinline__ float3 iso_dir(float Rmu, float Rphi) {

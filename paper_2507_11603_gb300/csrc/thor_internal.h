@@ -20,6 +20,8 @@ struct Tally {
 // Gridless model (Sec. 3.3 spherical shell / sphere) as the kernels read it.
 struct ShellModel {
   double R_in, R_out;        // radii (R_out normalises lengths)
+  double R_in2;              // R_in^2, and from it in FP32 (segment bounds): R_out^2 - R_in^2,
+  float span, inv_in, inv_out;  // 1 / (2 R_in) (0 without a cavity), 1 / (R_out + R_in)
   float kap0;                // HI line-centre opacity per unit length
   float kapd;                // dust extinction per unit length
   float vth, inv_vth, a;     // km/s, s/km, Voigt parameter
@@ -54,6 +56,13 @@ struct ShellModel {
   float* raw_X0;             // optional per-photon emitted X and column
   float* raw_col;
 };
+
+inline void shell_record_radii(ShellModel* m) {
+  m->R_in2 = m->R_in * m->R_in;
+  m->span = (float)(m->R_out * m->R_out - m->R_in2);
+  m->inv_in = m->R_in > 0.0 ? (float)(0.5 / m->R_in) : 0.0f;
+  m->inv_out = (float)(1.0 / (m->R_out + m->R_in));
+}
 
 // Every FP32 parameter of a shell record is finite and the thermal speed and Voigt a are
 // positive (a parameter set whose opacities overflow FP32 is rejected, since a photon

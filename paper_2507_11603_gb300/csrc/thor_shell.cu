@@ -30,7 +30,7 @@ struct Photon {
   uint32_t nscat, ndust, iters, steps;
   float X0;              // emitted lab frequency
   float col_hi, col_lo;  // HI column traversed (power-law shells), two-level FP32 sum
-  Rng rng;
+  StreamKey key;  // key.event: last completed event
   int model;
   unsigned long long pid;
 };
@@ -48,15 +48,17 @@ __device__ __forceinline__ int find_entry(const WorkQueue& q, unsigned long long
 // with a continuum (Sec. 5.1) word 4 picks the line (probability p_line) or the flat
 // continuum, whose position is word 5.
 __device__ __forceinline__ void shell_emit(const ShellModel& m, Photon& ph) {
-  ph.rng.init(((uint64_t)m.seed_hi << 32) | m.seed_lo, ph.pid, m.cont_C > 0.0f ? 2u : 1u);
+  Rng rng;
+  rng.init(((uint64_t)m.seed_hi << 32) | m.seed_lo, ph.pid, m.cont_C > 0.0f ? 2u : 1u);
+  ph.key = rng;
   ph.px = 0.0; ph.py = 0.0; ph.pz = 0.0;
   ph.ox = 0.0f; ph.oy = 0.0f; ph.oz = 0.0f;
-  ph.k = iso_dir(ph.rng.u(0), ph.rng.u(1));
+  ph.k = iso_dir(rng.u(0), rng.u(1));
   float X = m.X0;
-  if (m.cont_C > 0.0f && ph.rng.u(4) > m.p_line) {
-    X = __fmaf_rn(m.cont_C, __fmaf_rn(2.0f, ph.rng.u(5), -1.0f), X);
+  if (m.cont_C > 0.0f && rng.u(4) > m.p_line) {
+    X = __fmaf_rn(m.cont_C, __fmaf_rn(2.0f, rng.u(5), -1.0f), X);
   } else if (m.line == 1) {
-    const float R1 = ph.rng.u(2), R2 = ph.rng.u(3);
+    const float R1 = rng.u(2), R2 = rng.u(3);
     X = __fmaf_rn(m.sigma * sqrtf(-2.0f * __logf(R1)), cospif(2.0f * R2), X);
   }
   ph.X = X;
@@ -78,6 +80,7 @@ __device__ __forceinline__ void advance(Photon& ph, float s) {
 }
 // Fold the offset into the FP64 anchor (before any use of the absolute position).
 __device__ __forceinline__ void anchor(Photon& ph) {
+  if (ph.ox == 0.0f && ph.oy == 0.0f && ph.oz == 0.0f) return;  // already folded (FP64 runs at 1/64 of FP32)
   ph.px += (double)ph.ox; ph.py += (double)ph.oy; ph.pz += (double)ph.oz;
   ph.ox = 0.0f; ph.oy = 0.0f; ph.oz = 0.0f;
 }
@@ -89,6 +92,46 @@ __device__ __forceinline__ float safe_distance(const ShellModel& m, const Photon
   if (m.R_in > 0.0) d = fmin(d, r - m.R_in);
   return fmaxf(__double2float_rd(d) * 0.999999f, 0.0f);
 }
+
+// The segment from p along k to the next boundary: b = p . k, pp = r^2.  FP64 runs at 1/64 of
+// the FP32 rate here and a dependent FP64 operation takes some 40 cycles, so the exact distance
+// is formed only for a sub-step that may end at the boundary.  `lower` is a lower bound of it:
+// r^2 - R_in^2 is taken in FP64 and rounded once, roots are formed without cancellation, and
+// the margins cover the FP32 rounding (relative 1e-6; absolute 1e-6 for R_out^2 - r^2).
+struct ShellSegment {
+  float lower, c_in, bf;  // bound, r^2 - R_in^2, b
+  __device__ __forceinline__ ShellSegment(const ShellModel& m, double b, double pp) {
+    bf = (float)b;
+    c_in = (float)(pp - m.R_in2);
+    const float b2 = bf * bf, disc = b2 - c_in, err = 1e-6f * (b2 + fabsf(c_in));
+    if (m.inv_in > 0.0f && bf < 0.0f && disc > -err) {  // may meet the inner sphere (before the outer one)
+      lower = 0.999f * c_in * rcp_approx(sqrt_approx(fmaxf(disc, 0.0f) + err) - bf);
+    } else {
+      const float c_out = fmaxf(m.span - c_in - 1e-6f, 0.0f), q = sqrt_approx(b2 + c_out);
+      lower = 0.999f * (bf >= 0.0f ? c_out * rcp_approx(q + bf + 1e-30f) : q - bf);
+    }
+  }
+  // the distance and what is met there (1 outside, 2 cavity)
+  static __device__ __forceinline__ double exact(const ShellModel& m, double b, double pp, int& next) {
+    next = 1;
+    if (m.R_in > 0.0 && b < 0.0) {
+      const double disc = b * b - (pp - m.R_in * m.R_in);
+      if (disc > 0.0) {  // nearer than the outer sphere: -b - sqrt(disc) < -b < its distance
+        next = 2;
+        return fmax(-b - sqrt(disc), 0.0);
+      }
+    }
+    return fmax(-b + sqrt(fmax(b * b - (pp - m.R_out * m.R_out), 0.0)), 0.0);
+  }
+  // Whether the point at s along the segment is certainly nearer than the sub-step to a
+  // boundary: r - R_in = (r^2 - R_in^2) / (r + R_in) <= (r^2 - R_in^2) / (2 R_in), likewise
+  // outside.
+  __device__ __forceinline__ bool near_edge(const ShellModel& m, float s) const {
+    const float t = __fmaf_rn(s, __fmaf_rn(2.0f, bf, s), c_in), e = 1e-6f;  // r'^2 - R_in^2
+    return (m.inv_in > 0.0f && (t + e) * m.inv_in < 0.99f * m.ds_core) ||
+           (m.span - t + e) * m.inv_out < 0.99f * m.ds_core;
+  }
+};
 
 // The start of a step, shared by shell_event's fast paths and the core events in rounds (one
 // definition, so both evaluate an event bit for bit alike): H(a, x) from the table-free
@@ -103,8 +146,6 @@ __device__ __forceinline__ StartStep start_step(const ShellModel& m, float H, fl
   const float kH = __fmul_rn(m.kap0, H);
   return StartStep{kH, __fmul_rn(tau, rcp_approx(__fadd_rn(kH, m.kapd)))};
 }
-// The optical depth to the next interaction, tau = -ln R (Eq. 3), shared likewise.
-__device__ __forceinline__ float draw_tau(const Rng& r) { return -ln_fast(r.u(W_TAU)); }
 __device__ __forceinline__ bool dust_channel(const ShellModel& m, float kH, float R) {
   return __fmul_rn(R, __fadd_rn(kH, m.kapd)) >= kH;
 }
@@ -115,12 +156,15 @@ __device__ __forceinline__ bool dust_channel(const ShellModel& m, float kH, floa
 // same point.  A conservative safety distance to the shell boundaries lets events whose
 // interaction lies inside the safety ball skip the FP64 ray-sphere geometry (the common
 // case for photons trapped in the line core).
-__device__ __forceinline__ uint32_t shell_blocks(const ShellModel& m) {
-  return (m.kapd > 0.0f || m.phase == PH_MIXED) ? 3u : 2u;
+// Blocks of words an event may take: the third holds the channel, albedo and mixed-phase words.
+__device__ __forceinline__ bool needs_block2(const ShellModel& m) {
+  return m.kapd > 0.0f || m.kapdn > 0.0f || m.phase == PH_MIXED || m.n_lines == 2;
 }
 
-// The event whose words ph.rng holds, with the optical depth tau_rem drawn from them.
-__device__ int shell_event_words(const ShellModel& m, Photon& ph, const float* __restrict__ Ktab, float tau_rem) {
+// The packet's next event, from what it takes of its random words.
+__device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restrict__ Ktab, const EventWords& w) {
+  ++ph.key.event;
+  float tau_rem = w.tau;
   float x_site, kH;
   for (;;) {
     if (ph.region) {  // empty cavity: straight to the inner sphere, lab X conserved
@@ -178,39 +222,83 @@ __device__ int shell_event_words(const ShellModel& m, Photon& ph, const float* _
       ph.x -= m.gam * ds;
       continue;
     }
-    // ---- general path: exact segment to the next boundary (FP64), then sub-steps
+    // ---- general path: sub-steps to the crossing or the next boundary, its distance exact
+    // (FP64) where it counts
     anchor(ph);
     const double kx = ph.k.x, ky = ph.k.y, kz = ph.k.z;
     const double b = ph.px * kx + ph.py * ky + ph.pz * kz;
     const double pp = ph.px * ph.px + ph.py * ph.py + ph.pz * ph.pz;
-    double S = -b + sqrt(fmax(b * b - (pp - m.R_out * m.R_out), 0.0));
-    int next = 1;  // 1 escape, 2 cavity
-    if (m.R_in > 0.0 && b < 0.0) {
-      const double disc = b * b - (pp - m.R_in * m.R_in);
-      if (disc > 0.0) {
-        const double s_in = -b - sqrt(disc);
-        if (s_in < S) { S = s_in; next = 2; }
-      }
-    }
-    S = fmax(S, 0.0);
-    const float Sf = (float)S;
+    const ShellSegment seg(m, b, pp);
     const float x0 = ph.x;
+    double S = 0.0;  // distance to the boundary, once needed (seg.exact), and what is there
+    float Sf = 0.0f;
+    int next = 1;
     float s_star = -1.0f;
     if (m.gam == 0.0f) {
+      S = seg.exact(m, b, pp, next);
+      Sf = (float)S;
       const float kap = kH + m.kapd;
       if (kap * Sf >= tau_rem) s_star = fminf(tau_rem / kap, Sf);
       else tau_rem -= kap * Sf;
     } else {
       float s = 0.0f;
-      while (s < Sf) {
-        const float s1 = fminf(Sf, s + m.ds_core);
+      bool have = false;
+      for (;;) {
+        float s1 = s + m.ds_core;
+        if (!have && !(s1 <= seg.lower)) {
+          S = seg.exact(m, b, pp, next);
+          Sf = (float)S;
+          have = true;
+        }
+        if (have) {
+          if (!(s < Sf)) break;
+          s1 = fminf(Sf, s1);
+        }
         const float xm = x0 - m.gam * 0.5f * (s + s1);
         const float kap = __fmaf_rn(m.kap0, voigt<false>(m.a, xm, Ktab), m.kapd);
         const float dtau = kap * (s1 - s);
         ++ph.steps;
-        if (dtau >= tau_rem) { s_star = fminf(s + tau_rem / kap, Sf); break; }
+        if (dtau >= tau_rem) {
+          s_star = s + tau_rem / kap;
+          if (have) s_star = fminf(s_star, Sf);
+          break;
+        }
         tau_rem -= dtau;
         s = s1;
+        // Free flight: sub-steps in the wing, four at a time.  Their opacities do not depend
+        // on one another (x drifts monotonically), so they are formed side by side and only
+        // the depth is summed in order.
+        while (s + 4.25f * m.ds_core <= (have ? Sf : seg.lower)) {
+          float e[5], kp[4];
+          e[0] = s;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) e[i + 1] = e[i] + m.ds_core;
+          const float xa = x0 - m.gam * 0.5f * (e[0] + e[1]), xb = x0 - m.gam * 0.5f * (e[3] + e[4]);
+          if (!(fminf(xa, xb) >= 6.0f || fmaxf(xa, xb) <= -6.0f)) break;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float ax = fabsf(x0 - m.gam * 0.5f * (e[i] + e[i + 1]));
+            kp[i] = __fmaf_rn(m.kap0, voigt_wing<false>(m.a, ax * ax), m.kapd);
+          }
+          bool cross = false;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float dt = kp[i] * (e[i + 1] - e[i]);
+            if (!cross) {
+              ++ph.steps;
+              if (dt >= tau_rem) {
+                cross = true;
+                s_star = e[i] + tau_rem / kp[i];
+                if (have) s_star = fminf(s_star, Sf);
+              } else {
+                tau_rem -= dt;
+                s = e[i + 1];
+              }
+            }
+          }
+          if (cross) break;
+        }
+        if (s_star >= 0.0f) break;
       }
     }
     if (s_star >= 0.0f) {
@@ -218,7 +306,10 @@ __device__ int shell_event_words(const ShellModel& m, Photon& ph, const float* _
       ph.px += sd * kx; ph.py += sd * ky; ph.pz += sd * kz;
       x_site = x0 - m.gam * s_star;
       if (m.gam != 0.0f) kH = m.kap0 * voigt<false>(m.a, x_site, Ktab);
-      ph.safe = safe_distance(m, ph);
+      // the safety distance counts only from ds on: where it is certainly shorter (photons
+      // trapped at the shell's edge, which come here event after event) its FP64 square root
+      // is left out
+      ph.safe = (m.gam != 0.0f && seg.near_edge(m, s_star)) ? 0.0f : safe_distance(m, ph);
       break;
     }
     ph.px += S * kx; ph.py += S * ky; ph.pz += S * kz;
@@ -230,19 +321,20 @@ __device__ int shell_event_words(const ShellModel& m, Photon& ph, const float* _
   ph.x = x_site;
   // Interaction (Sec. 3.4): channel i with probability tau_i / sum_i tau_i.
   bool dust = false;
-  if (m.kapd > 0.0f) dust = dust_channel(m, kH, ph.rng.u(W_CHANNEL));
+  if (m.kapd > 0.0f) dust = dust_channel(m, kH, w.channel);
   if (dust) {
     bool scat;
     if (m.albedo <= 0.0f) scat = false;
     else if (m.albedo >= 1.0f) scat = true;
-    else scat = ph.rng.u(W_ALBEDO) < m.albedo;
+    else scat = w.albedo < m.albedo;
     if (!scat) return 2;
-    scatter_dust(m.g_hg, ph.k, ph.rng);  // gas-frame frequency unchanged
+    scatter_dust(m.g_hg, ph.k, w.Rm, w.cp, w.sp);  // gas-frame frequency unchanged
     ++ph.ndust;
     return 0;
   }
   // Eq. 7: the gas-frame frequency after the scattering, at the same point
-  ph.x = scatter_resonant<kTurnShell, kTurnShellIso>(x_site, m.a, m.phase, ph.k, ph.rng, ph.iters, nullptr, m.xcrit);
+  ph.x = scatter_resonant<kTurnShell, kTurnShellIso>(x_site, m.a, m.phase, ph.k, w, ph.key, ph.iters, nullptr,
+                                                     m.xcrit);
   ++ph.nscat;
   if (m.max_scat && ph.nscat >= m.max_scat) {
     anchor(ph);
@@ -251,11 +343,6 @@ __device__ int shell_event_words(const ShellModel& m, Photon& ph, const float* _
     return 3;
   }
   return 0;
-}
-
-__device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restrict__ Ktab) {
-  ph.rng.next_event(shell_blocks(m));
-  return shell_event_words(m, ph, Ktab, draw_tau(ph.rng));  // Eq. 3: tau ~ Exp(1)
 }
 
 // ---- core events in rounds (homologous shells) ---------------------------------------
@@ -274,7 +361,7 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
 // lanes first evaluate everything that depends on words alone, one event of one packet
 // per lane, for the next D events of the warp's P packets (P D <= kChainSlots), into shared
 // memory; then the P lanes that own the packets run D events of the chain, each from one
-// 48-byte slot.  The general event evaluates these events with the same helpers
+// 64-byte slot.  The general event evaluates these events with the same helpers
 // (start_step, dust_channel, u0_core, upar_q / atan_small, upar_trial, x_after_scatter) on
 // the same words, so both paths give bit-identical results.
 // Measured (GB300, 2070 MHz): a photon alone in a static sphere 0.36 us per event (0.47 us
@@ -286,34 +373,53 @@ constexpr int kChainSlots = 128;      // events per warp and round
 constexpr uint32_t kChainDepth = 32;  // ... and per packet, in warps with few packets
 constexpr uint32_t kCrowdDepth = 16;  // ... and per packet, in the others (kept until a general event runs)
 constexpr uint32_t kVoteEvents = 4;   // core events between two votes on whether any packet goes on
-struct ChainBuf {                     // one per warp
+struct WordBuf {                      // one per warp
   float4 a[kChainSlots];              // tau, R1, R2, R3
-  float4 b[kChainSlots];              // mu, st, perpendicular term (plain), channel uniform
-  float4 c[kChainSlots];              // cos phi, sin phi, perpendicular term (core-skipping), -
-  uint4 own[32];                      // photon id, last completed event, needs (owners in lane order)
+  float4 b[kChainSlots];              // mu, st, cos phi, sin phi
+  float4 c[kChainSlots];              // u1, u2, v1, v2
+  float4 d[kChainSlots];              // Rm, channel, mixed, albedo
+  uint4 own[32];                      // photon id, last completed event, flags (owners in lane order)
   uint4 key[32];                      // stream key, phase function, core-skipping threshold
 };
+// Where a lane's slots lie: slot (cur P + rank) holds its next event while cur < D.
+struct WordPos {
+  int P = 1, D = 0, rank = 0, cur = 0;
+};
 
-// A slot: what event e of photon (p0, p1) takes from its words (as start_event, draw_tau,
-// scatter_resonant and x_after_scatter form them).
-__device__ __forceinline__ void chain_slot(ChainBuf& cb, int s, const uint4& own, const uint4& key, uint32_t e) {
-  Rng r;
-  r.k0 = key.x; r.k1 = key.y; r.p0 = own.x; r.p1 = own.y;
-  r.start_event(e, (own.w & 1u) ? 3u : 2u);
-  float sp1, cp1, sp, cp;
-  __sincosf(2.0f * kPiF * r.u(W_BM_PHI), &sp1, &cp1);
-  __sincosf(2.0f * kPiF * r.u(W_PHI), &sp, &cp);
-  const float lr = __logf(r.u(W_BM_R));
-  const float Rm = r.u(W_MU);
-  const float mu = ((int)key.z == PH_ISO) ? __fmaf_rn(2.0f, Rm, -1.0f) : mu_dipole(Rm);
-  const float st = sqrt_approx(fmaxf(0.0f, __fmaf_rn(-mu, mu, 1.0f)));
-  auto perp = [&](float xc) {
-    const float rr = sqrt_approx(__fmaf_rn(xc, xc, -lr));
-    return scatter_perp(st, __fmul_rn(rr, cp1), __fmul_rn(rr, sp1), cp, sp);
-  };
-  cb.a[s] = make_float4(draw_tau(r), r.u(W_UPAR0), r.u(W_UPAR0 + 1), r.u(W_UPAR0 + 2));
-  cb.b[s] = make_float4(mu, st, perp(0.0f), (own.w & 1u) ? r.u(W_CHANNEL) : 0.0f);
-  cb.c[s] = make_float4(cp, sp, perp(__uint_as_float(key.w)), 0.0f);
+// Forms the next D events' words of every packet in `mine` lanes, one slot per lane at a
+// time (P D <= kChainSlots).  Called by all 32 lanes, converged.
+__device__ __forceinline__ void form_words(const ShellModel& m, const Photon& ph, WordBuf& wb, bool mine, int D,
+                                           WordPos& at) {
+  const int lane = (int)(threadIdx.x & 31u);
+  const unsigned owners = __ballot_sync(kFull, mine);
+  const int P = __popc(owners);
+  at.P = P; at.D = mine ? D : 0; at.cur = 0;
+  at.rank = mine ? __popc(owners & ((1u << lane) - 1u)) : 0;
+  if (mine) {
+    wb.own[at.rank] = make_uint4(ph.key.p0, ph.key.p1, ph.key.event, (needs_block2(m) ? 1u : 0u) | (m.profile ? 2u : 0u));
+    wb.key[at.rank] = make_uint4(ph.key.k0, ph.key.k1, (uint32_t)m.phase, __float_as_uint(m.xcrit));
+  }
+  __syncwarp();
+  for (int s = lane; s < P * D; s += 32) {  // slot d P + r: event d of the owner of rank r
+    const int d = s / P, r = s - d * P;
+    const uint4 own = wb.own[r], key = wb.key[r];
+    Rng q;
+    q.k0 = key.x; q.k1 = key.y; q.p0 = own.x; q.p1 = own.y;
+    q.v[8] = q.v[9] = q.v[10] = 0u;  // not drawn: not used
+    q.start_event(own.z + 1u + (uint32_t)d, (own.w & 1u) ? 3u : 2u);
+    EventWords w;
+    scatter_words(w, q, (int)key.z, __uint_as_float(key.w));
+    const float t = q.u(W_TAU);
+    wb.a[s] = make_float4((own.w & 2u) ? -__logf(t) : -ln_fast(t), w.R1, w.R2, w.R3);
+    wb.b[s] = make_float4(w.mu, w.st, w.cp, w.sp);
+    wb.c[s] = make_float4(w.u1, w.u2, w.v1, w.v2);
+    wb.d[s] = make_float4(w.Rm, q.u(W_CHANNEL), w.mixed, q.u(W_ALBEDO));
+  }
+  __syncwarp();
+}
+__device__ __forceinline__ EventWords read_words(const WordBuf& wb, int s) {
+  const float4 a = wb.a[s], b = wb.b[s], c = wb.c[s], d = wb.d[s];
+  return EventWords{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w, d.x, d.y, d.z, d.w};
 }
 
 // Whether the packet's next event may be of the core kind (the cheap part of the test).
@@ -325,14 +431,14 @@ __device__ __forceinline__ bool chain_kind(const ShellModel& m, const Photon& ph
 // (by selects: a loop body of one basic block but for the rare second trial).  Returns
 // whether it was committed.
 __device__ __forceinline__ bool chain_event(const ShellModel& m, Photon& ph, const float4& wa, const float4& wb,
-                                            const float4& wc, uint32_t e, bool go, uint32_t& second) {
+                                            const float4& wc, float channel, uint32_t e, bool go, uint32_t& second) {
   // ---- the frequency chain: rate at the start, crossing, gas-frame frequency at the site
   const float x0 = go ? ph.x : 0.0f;  // lanes without a packet in the round take the owners' branches
   const StartStep st0 = start_step(m, voigt_core_poly(m.a, x0), wa.x);
   const float s0 = st0.s;
   const bool in_ball = (m.gam == 0.0f) ? (s0 <= ph.safe) : (ph.safe >= m.ds_core && s0 <= 0.0625f * m.ds_core);
   const float xs = (m.gam == 0.0f) ? x0 : __fmaf_rn(-m.gam, s0, x0);
-  const bool dust = (m.kapd > 0.0f) && dust_channel(m, st0.kH, wb.w);
+  const bool dust = (m.kapd > 0.0f) && dust_channel(m, st0.kH, channel);
   // ---- u_par, first trial of the two-piece comparison function (as sample_upar)
   const float sgn = (xs < 0.0f) ? -1.0f : 1.0f;
   const float xr = fabsf(xs);
@@ -350,7 +456,7 @@ __device__ __forceinline__ bool chain_event(const ShellModel& m, Photon& ph, con
   const bool kind = go && fabsf(x0) <= THOR_VCORE_X && in_ball && !dust && xr <= 2.0f &&
                     (split ? q <= 0.05f : m.a <= 0.05f * xr);
   if (!accepted && kind) {  // rare: the second trial, from block 3 of the event as sample_upar takes it
-    Rng r = ph.rng;
+    StreamKey r = ph.key;
     r.event = e;
     uint32_t b0, b1, b2, b3;
     r.block(3u, b0, b1, b2, b3);
@@ -361,41 +467,28 @@ __device__ __forceinline__ bool chain_event(const ShellModel& m, Photon& ph, con
   // ---- beside the chain: the outgoing direction (as scatter_resonant)
   float3 e1, e2;
   basis(ph.k.x, ph.k.y, ph.k.z, e1, e2);
-  const float3 ko = turn<kTurnShell>(ph.k, e1, e2, wb.x, wb.y, wc.x, wc.y);
+  const float3 ko = turn<kTurnShell>(ph.k, e1, e2, wb.x, wb.y, wb.z, wb.w);
   // ---- commit
   ph.ox = ok ? __fmaf_rn(s0, ph.k.x, ph.ox) : ph.ox;  // advance(ph, s0)
   ph.oy = ok ? __fmaf_rn(s0, ph.k.y, ph.oy) : ph.oy;
   ph.oz = ok ? __fmaf_rn(s0, ph.k.z, ph.oz) : ph.oz;
   ph.safe = ok ? __fmaf_rd(-s0, 1.000001f, ph.safe) : ph.safe;
-  ph.x = ok ? x_after_perp(xs, sgn * u, wb.x, (xr < m.xcrit) ? wc.z : wb.z) : ph.x;
+  const bool skip = xr < m.xcrit;
+  const float perp = scatter_perp(wb.y, skip ? wc.z : wc.x, skip ? wc.w : wc.y, wb.z, wb.w);
+  ph.x = ok ? x_after_perp(xs, sgn * u, wb.x, perp) : ph.x;
   ph.k.x = ok ? ko.x : ph.k.x;
   ph.k.y = ok ? ko.y : ph.k.y;
   ph.k.z = ok ? ko.z : ph.k.z;
   return ok;
 }
 
-// A round: up to `depth` core events of every packet in `mine` lanes (with its random words
-// formed by all lanes).  Called by all 32 lanes, converged.  Returns the events done; `stuck`
-// tells the lanes whose packet stopped before an event that is not of the core kind, or one
-// scattering short of the cap (shell_event runs that one).
-__device__ __forceinline__ uint32_t chain_round(const ShellModel& m, Photon& ph, ChainBuf& cb, bool mine,
-                                                uint32_t depth, bool& stuck) {
-  const int lane = (int)(threadIdx.x & 31u);
-  const unsigned owners = __ballot_sync(kFull, mine);
-  const int P = __popc(owners);
-  const int rank = mine ? __popc(owners & ((1u << lane) - 1u)) : 0;
-  const int D = min((int)depth, kChainSlots / P);
-  if (mine) {
-    cb.own[rank] = make_uint4(ph.rng.p0, ph.rng.p1, ph.rng.event, m.kapd > 0.0f ? 1u : 0u);
-    cb.key[rank] = make_uint4(ph.rng.k0, ph.rng.k1, (uint32_t)m.phase, __float_as_uint(m.xcrit));
-  }
-  __syncwarp();
-  for (int s = lane; s < P * D; s += 32) {  // slot d P + r: event d of the owner of rank r
-    const int d = s / P, r = s - d * P;
-    const uint4 own = cb.own[r];
-    chain_slot(cb, s, own, cb.key[r], own.z + 1u + (uint32_t)d);
-  }
-  __syncwarp();
+// A round: up to D core events of every packet in `mine` lanes.  Called by all 32 lanes,
+// converged.  `stuck` tells the lanes whose packet stopped before an event that is not of the
+// core kind, or one scattering short of the cap (the general event runs that one, from slot
+// at.cur).  Returns the events done.
+__device__ __forceinline__ uint32_t chain_round(const ShellModel& m, Photon& ph, WordBuf& wb, bool mine, int D,
+                                                WordPos& at, bool& stuck) {
+  form_words(m, ph, wb, mine, D, at);
   const uint32_t left = m.max_scat ? (m.max_scat > ph.nscat + 1u ? m.max_scat - ph.nscat - 1u : 0u) : (uint32_t)D;
   const int lim = (int)min(left, (uint32_t)D);
   bool go = mine;
@@ -405,18 +498,18 @@ __device__ __forceinline__ uint32_t chain_round(const ShellModel& m, Photon& ph,
     const int end = min(D, d + (int)kVoteEvents);
 #pragma unroll 1
     for (; d < end; ++d) {
-      const int s = d * P + rank;
-      go = chain_event(m, ph, cb.a[s], cb.b[s], cb.c[s], ph.rng.event + 1u + (uint32_t)d, go && d < lim, second);
+      const int s = d * at.P + at.rank;
+      go = chain_event(m, ph, wb.a[s], wb.b[s], wb.c[s], wb.d[s].y, ph.key.event + 1u + (uint32_t)d, go && d < lim, second);
       n += go ? 1u : 0u;
     }
     if (!__any_sync(kFull, go)) break;
   }
-  __syncwarp();
   if (mine) {
-    ph.rng.event += n;
+    ph.key.event += n;
     ph.nscat += n;
     ph.steps += n;
     ph.iters += n + second;
+    at.cur = (int)n;
   }
   stuck = mine && !go;
   return n;
@@ -425,9 +518,10 @@ __device__ __forceinline__ uint32_t chain_round(const ShellModel& m, Photon& ph,
 // Core events of a warp's packets until `depth` of them ran or the packet needs a general
 // event (`general` then stays set).  Several rounds where the slots of one do not reach
 // (P > kChainSlots / depth): the general events, which run for a few lanes at a time, come
-// once per `depth` events.  Returns this lane's events.
-__device__ __forceinline__ uint32_t core_events(const ShellModel& m, Photon& ph, ChainBuf& cb, bool active,
-                                                uint32_t depth, bool& general) {
+// once per `depth` events.  Returns this lane's events; `at`: the slots of its last round, if
+// no other round has overwritten them.
+__device__ __forceinline__ uint32_t core_events(const ShellModel& m, Photon& ph, WordBuf& wb, bool active,
+                                                uint32_t depth, bool& general, WordPos& at) {
   uint32_t n = 0;
   bool go = active && chain_kind(m, ph);
   for (uint32_t d = 0; d < depth; ) {
@@ -435,12 +529,22 @@ __device__ __forceinline__ uint32_t core_events(const ShellModel& m, Photon& ph,
     if (P == 0) break;
     const uint32_t D = min(depth - d, (uint32_t)(kChainSlots / P));
     bool stuck = false;
-    n += chain_round(m, ph, cb, go, D, stuck);
+    __syncwarp();  // the round before is read
+    n += chain_round(m, ph, wb, go, (int)D, at, stuck);
     go = go && !stuck;
     d += D;
   }
   general = active && !go;
   return n;
+}
+
+// Slots for the next general event of the lanes in `general`, formed where they are not there
+// yet: as many events ahead as one pass of the 32 lanes yields (at most kCrowdDepth).
+__device__ __forceinline__ void general_words(const ShellModel& m, const Photon& ph, WordBuf& wb, bool general,
+                                              WordPos& at) {
+  if (!__any_sync(kFull, general && at.cur >= at.D)) return;
+  const int P = __popc(__ballot_sync(kFull, general));
+  form_words(m, ph, wb, general, min((int)kCrowdDepth, 32 / P), at);
 }
 
 // ---- power-law shells (Sec. 5.1) ---------------------------------------------------
@@ -477,9 +581,9 @@ __device__ __forceinline__ float from_line2(const ShellModel& m, float X2) {
   return __fmaf_rn(-__fdividef(m.eps2, 1.0f + m.eps2), kCkms + X2, X2);
 }
 
-__device__ int shell_event_pl(const ShellModel& m, Photon& ph, const float* __restrict__ Ktab) {
-  ph.rng.next_event((m.kapdn > 0.0f || m.phase == PH_MIXED || m.n_lines == 2) ? 3u : 2u);
-  float tau_rem = -__logf(ph.rng.u(W_TAU));  // Eq. 3
+__device__ int shell_event_pl(const ShellModel& m, Photon& ph, const float* __restrict__ Ktab, const EventWords& w) {
+  ++ph.key.event;
+  float tau_rem = w.tau;
   float kH, kH2 = 0.0f, kD;
   PLState site;
   for (;;) {
@@ -513,47 +617,101 @@ __device__ int shell_event_pl(const ShellModel& m, Photon& ph, const float* __re
         break;
       }
     }
-    // general path: exact segment to the next boundary (FP64), sub-steps of <= ds
+    // general path: sub-steps of <= ds to the crossing or the next boundary, its distance
+    // exact (FP64) where it counts
     anchor(ph);
     const double kx = ph.k.x, ky = ph.k.y, kz = ph.k.z;
     const double b = ph.px * kx + ph.py * ky + ph.pz * kz;
     const double pp = ph.px * ph.px + ph.py * ph.py + ph.pz * ph.pz;
-    double S = -b + sqrt(fmax(b * b - (pp - m.R_out * m.R_out), 0.0));
-    int next = 1;  // 1 escape, 2 cavity
-    if (b < 0.0) {
-      const double disc = b * b - (pp - m.R_in * m.R_in);
-      if (disc > 0.0) {
-        const double s_in = -b - sqrt(disc);
-        if (s_in < S) { S = s_in; next = 2; }
-      }
-    }
-    S = fmax(S, 0.0);
-    const float Sf = (float)S;
+    const ShellSegment seg(m, b, pp);
+    double S = 0.0;
+    float Sf = 0.0f;
+    int next = 1;
+    bool have = false;
     const float p0x = (float)ph.px, p0y = (float)ph.py, p0z = (float)ph.pz;
     float s = 0.0f, s_star = -1.0f;
-    while (s < Sf) {
-      const float s1 = fminf(Sf, s + m.ds_core);
-      const float sm = 0.5f * (s + s1);
-      const PLState st = pl_state(m, __fmaf_rn(sm, ph.k.x, p0x), __fmaf_rn(sm, ph.k.y, p0y),
-                                  __fmaf_rn(sm, ph.k.z, p0z), ph.k);
-      const float x = (ph.X - st.v * st.mur) * m.inv_vth;
-      const float H = voigt<false>(m.a, x, Ktab);
-      const float H2 = (m.n_lines == 2) ? voigt<false>(m.a2, (to_line2(m, ph.X) - st.v * st.mur) * m.inv_vth, Ktab)
-                                         : 0.0f;
-      const float kap = st.nr * __fmaf_rn(m.kapn, H, __fmaf_rn(m.kapn2, H2, m.kapdn));
+    // one sub-step of opacity kap, density nr, [s, s1]: true where the crossing lies in it
+    auto sub_step = [&](float s1, float kap, float nr) {
       const float dtau = kap * (s1 - s);
       ++ph.steps;
       if (dtau >= tau_rem) {
-        s_star = fminf(s + __fdividef(tau_rem, kap), Sf);
-        col_add(ph, st.nr * m.invF * (s_star - s));
-        kH = m.kapn * st.nr * H;
-        kH2 = m.kapn2 * st.nr * H2;
-        kD = m.kapdn * st.nr;
-        break;
+        s_star = s + __fdividef(tau_rem, kap);
+        if (have) s_star = fminf(s_star, Sf);
+        col_add(ph, nr * m.invF * (s_star - s));
+        return true;
       }
-      col_add(ph, st.nr * m.invF * (s1 - s));
+      col_add(ph, nr * m.invF * (s1 - s));
       tau_rem -= dtau;
       s = s1;
+      return false;
+    };
+    for (;;) {
+      float s1 = s + m.ds_core;
+      if (!have && !(s1 <= seg.lower)) {
+        S = seg.exact(m, b, pp, next);
+        Sf = (float)S;
+        have = true;
+      }
+      if (have) {
+        if (!(s < Sf)) break;
+        s1 = fminf(Sf, s1);
+      }
+      {
+        const float sm = 0.5f * (s + s1);
+        const PLState st = pl_state(m, __fmaf_rn(sm, ph.k.x, p0x), __fmaf_rn(sm, ph.k.y, p0y),
+                                    __fmaf_rn(sm, ph.k.z, p0z), ph.k);
+        const float x = (ph.X - st.v * st.mur) * m.inv_vth;
+        const float H = voigt<false>(m.a, x, Ktab);
+        const float H2 = (m.n_lines == 2) ? voigt<false>(m.a2, (to_line2(m, ph.X) - st.v * st.mur) * m.inv_vth, Ktab)
+                                           : 0.0f;
+        const float kap = st.nr * __fmaf_rn(m.kapn, H, __fmaf_rn(m.kapn2, H2, m.kapdn));
+        if (sub_step(s1, kap, st.nr)) {
+          kH = m.kapn * st.nr * H;
+          kH2 = m.kapn2 * st.nr * H2;
+          kD = m.kapdn * st.nr;
+          break;
+        }
+      }
+      // Free flight: four sub-steps at a time while all of them lie in the lines' wings.  Their
+      // opacities do not depend on one another, so they are formed side by side (a photon's
+      // flight is a chain of some 100 dependent instructions per sub-step otherwise); depth
+      // and column are summed in order.
+      bool cross = false;
+      while (s + 4.25f * m.ds_core <= (have ? Sf : seg.lower)) {
+        float e[5], H[4], H2[4], nr[4];
+        e[0] = s;
+        bool wing = true;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          e[i + 1] = e[i] + m.ds_core;
+          const float sm = 0.5f * (e[i] + e[i + 1]);
+          const PLState st = pl_state(m, __fmaf_rn(sm, ph.k.x, p0x), __fmaf_rn(sm, ph.k.y, p0y),
+                                      __fmaf_rn(sm, ph.k.z, p0z), ph.k);
+          nr[i] = st.nr;
+          const float ax = fabsf((ph.X - st.v * st.mur) * m.inv_vth);
+          H[i] = voigt_wing<false>(m.a, ax * ax);
+          wing = wing && ax >= 6.0f;
+          H2[i] = 0.0f;
+          if (m.n_lines == 2) {
+            const float ax2 = fabsf((to_line2(m, ph.X) - st.v * st.mur) * m.inv_vth);
+            H2[i] = voigt_wing<false>(m.a2, ax2 * ax2);
+            wing = wing && ax2 >= 6.0f;
+          }
+        }
+        if (!wing) break;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float kap = nr[i] * __fmaf_rn(m.kapn, H[i], __fmaf_rn(m.kapn2, H2[i], m.kapdn));
+          if (!cross && sub_step(e[i + 1], kap, nr[i])) {
+            cross = true;
+            kH = m.kapn * nr[i] * H[i];
+            kH2 = m.kapn2 * nr[i] * H2[i];
+            kD = m.kapdn * nr[i];
+          }
+        }
+        if (cross) break;
+      }
+      if (cross) break;
     }
     if (s_star >= 0.0f) {
       const double sd = s_star;
@@ -570,17 +728,20 @@ __device__ int shell_event_pl(const ShellModel& m, Photon& ph, const float* __re
   // opacities (one uniform); dust absorbs.
   int ch = 0;
   if (kD > 0.0f || m.n_lines == 2) {
-    const float u = ph.rng.u(W_CHANNEL), kt = kH + kH2 + kD;
+    const float u = w.channel, kt = kH + kH2 + kD;
     ch = (u < __fdividef(kH, kt)) ? 0 : ((u < __fdividef(kH + kH2, kt)) ? 1 : 2);
   }
   if (ch == 2) return 2;
   const float qx = (float)ph.px + ph.ox, qy = (float)ph.py + ph.oy, qz = (float)ph.pz + ph.oz;
   float xo;
   if (ch == 0) {
-    xo = scatter_resonant((ph.X - site.v * site.mur) * m.inv_vth, m.a, m.phase, ph.k, ph.rng, ph.iters, nullptr,
+    xo = scatter_resonant((ph.X - site.v * site.mur) * m.inv_vth, m.a, m.phase, ph.k, w, ph.key, ph.iters, nullptr,
                           m.xcrit);
   } else {  // second transition: J = 1/2 upper level, isotropic
-    xo = scatter_resonant((to_line2(m, ph.X) - site.v * site.mur) * m.inv_vth, m.a2, PH_ISO, ph.k, ph.rng,
+    EventWords wi = w;
+    wi.mu = __fmaf_rn(2.0f, w.Rm, -1.0f);
+    wi.st = sqrt_approx(fmaxf(0.0f, __fmaf_rn(-wi.mu, wi.mu, 1.0f)));
+    xo = scatter_resonant((to_line2(m, ph.X) - site.v * site.mur) * m.inv_vth, m.a2, PH_ISO, ph.k, wi, ph.key,
                           ph.iters, nullptr, 0.0f);
   }
   // back to the lab frame with the new direction: X = x v_th + v(r) r_hat . k_out
@@ -651,7 +812,7 @@ __device__ __forceinline__ void save_rec(const Photon& ph, PhotonRec& r) {
   r.x = ph.x; r.X = ph.X; r.safe = ph.safe;
   r.region = ph.region;
   r.nscat = ph.nscat; r.ndust = ph.ndust; r.iters = ph.iters; r.steps = ph.steps;
-  r.event = ph.rng.event;
+  r.event = ph.key.event;
   r.pid = ph.pid;
 }
 
@@ -664,8 +825,8 @@ __device__ __forceinline__ void load_rec(const ShellModel& m, const PhotonRec& r
   ph.region = r.region;
   ph.nscat = r.nscat; ph.ndust = r.ndust; ph.iters = r.iters; ph.steps = r.steps;
   ph.pid = r.pid;
-  ph.rng.keys(((uint64_t)m.seed_hi << 32) | m.seed_lo, ph.pid);
-  ph.rng.event = r.event;
+  ph.key.keys(((uint64_t)m.seed_hi << 32) | m.seed_lo, ph.pid);
+  ph.key.event = r.event;
 }
 
 // ---- work sharing in the tail of a one-launch run (pool_take in thor_device.cuh) ----------
@@ -681,7 +842,7 @@ __global__ void __launch_bounds__(256, 1) shell_run_kernel(const ShellModel* __r
   __shared__ __align__(16) float sK[THOR_VOIGT_NINT * THOR_VOIGT_NCOEF];
   __shared__ ShellModel sm;
   extern __shared__ __align__(16) unsigned char dyn[];
-  ChainBuf& cb = reinterpret_cast<ChainBuf*>(dyn)[kProfile ? 0 : threadIdx.x >> 5];  // not touched on power laws
+  WordBuf& wb = reinterpret_cast<WordBuf*>(dyn)[threadIdx.x >> 5];
   load_ktab(sK, gK);
   if (threadIdx.x == 0) sm = models[q.model[0]];
   __syncthreads();
@@ -780,13 +941,16 @@ __global__ void __launch_bounds__(256, 1) shell_run_kernel(const ShellModel* __r
     do {
       fin = false;
       bool general = active;  // lanes whose next event is a general one
-      if (chain) core_events(m, ph, cb, active, depth, general);
+      WordPos at;
+      if (chain) core_events(m, ph, wb, active, depth, general, at);
       // packets whose next event is not of the core kind take general events: one, and more
       // while at least half of the warp's packets need them
       uint32_t n_gen = 0;
       do {
+        general_words(m, ph, wb, general, at);
         if (general) {
-          const int st = kProfile ? shell_event_pl(m, ph, sK) : shell_event(m, ph, sK);
+          const EventWords w = read_words(wb, at.cur++ * at.P + at.rank);
+          const int st = kProfile ? shell_event_pl(m, ph, sK, w) : shell_event(m, ph, sK, w);
           if (st) {
             if (st == 1) { ++lt.esc; tally_spectrum(m, ph.X); }
             else if (st == 2) ++lt.abs;
@@ -837,7 +1001,7 @@ __global__ void __launch_bounds__(256, 1) shell_slice_kernel(const ShellModel* _
                                                           const float* __restrict__ gK) {
   __shared__ __align__(16) float sK[THOR_VOIGT_NINT * THOR_VOIGT_NCOEF];
   extern __shared__ __align__(16) unsigned char dyn[];
-  ChainBuf& cb = reinterpret_cast<ChainBuf*>(dyn)[threadIdx.x >> 5];
+  WordBuf& wb = reinterpret_cast<WordBuf*>(dyn)[threadIdx.x >> 5];
   load_ktab(sK, gK);
   int per_warp = 32;  // at most this many live packets per warp after a refill
   if (q.hdr) {
@@ -884,8 +1048,8 @@ __global__ void __launch_bounds__(256, 1) shell_slice_kernel(const ShellModel* _
     ph.model = st.model[slot];
     const ShellModel& m = models[ph.model];
     ph.pid = st.pid[slot];
-    ph.rng.keys(((uint64_t)m.seed_hi << 32) | m.seed_lo, ph.pid);
-    ph.rng.event = st.event[slot];
+    ph.key.keys(((uint64_t)m.seed_hi << 32) | m.seed_lo, ph.pid);
+    ph.key.event = st.event[slot];
     ph.px = st.px[slot]; ph.py = st.py[slot]; ph.pz = st.pz[slot];
     ph.ox = st.ox[slot]; ph.oy = st.oy[slot]; ph.oz = st.oz[slot];
     ph.k = make_float3(st.kx[slot], st.ky[slot], st.kz[slot]);
@@ -943,12 +1107,15 @@ __global__ void __launch_bounds__(256, 1) shell_slice_kernel(const ShellModel* _
       fin = false;
       bool general = active;
       const uint32_t depth = min(n_live <= kChainSlots / (int)kChainDepth ? kChainDepth : kCrowdDepth, budget - ev);
-      uint32_t n = core_events(mr, ph, cb, active && chain, depth, general);
+      WordPos at;
+      uint32_t n = core_events(mr, ph, wb, active && chain, depth, general, at);
       if (kMixed) general = general || (active && !chain);
       uint32_t n_gen = 0;
       do {
+        general_words(mr, ph, wb, general, at);
         if (general) {
-          const int r = (kMixed && mr.profile) ? shell_event_pl(mr, ph, sK) : shell_event(mr, ph, sK);
+          const EventWords w = read_words(wb, at.cur++ * at.P + at.rank);
+          const int r = (kMixed && mr.profile) ? shell_event_pl(mr, ph, sK, w) : shell_event(mr, ph, sK, w);
           ++n;
           if (r) { finish_global(mr, ph, r); active = false; fin = true; }
           general = active && !(chain && chain_kind(mr, ph));
@@ -979,7 +1146,7 @@ __global__ void __launch_bounds__(256, 1) shell_slice_kernel(const ShellModel* _
       const unsigned long long j = pri ? (unsigned long long)(out.n_slots - 1) - r : r;
       SlotState& o = out;
       o.model[j] = ph.model; o.pid[j] = ph.pid;
-      o.event[j] = ph.rng.event;
+      o.event[j] = ph.key.event;
       o.px[j] = ph.px; o.py[j] = ph.py; o.pz[j] = ph.pz;
       o.ox[j] = ph.ox; o.oy[j] = ph.oy; o.oz[j] = ph.oz; o.safe[j] = ph.safe;
       o.kx[j] = ph.k.x; o.ky[j] = ph.k.y; o.kz[j] = ph.k.z;
@@ -1049,10 +1216,10 @@ cudaError_t launch_slot_presort(SlotState from, SlotState to, unsigned long long
   return cudaGetLastError();
 }
 
-// Shared memory of a block: one round buffer per warp (homologous shells).
-static size_t chain_bytes(int block) { return (size_t)(block / 32) * sizeof(ChainBuf); }
+// Shared memory of a block: one buffer of event words per warp.
+static size_t chain_bytes(int block) { return (size_t)(block / 32) * sizeof(WordBuf); }
 template <class F>
-static cudaError_t allow_chain(F* f) {  // 57 KB for the largest block: above the default limit
+static cudaError_t allow_chain(F* f) {  // 73 KB for the largest block: above the default limit
   return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chain_bytes(256));
 }
 
@@ -1064,6 +1231,8 @@ int shell_grid(int block, int blocks_per_sm, bool sliced) {
   allow_chain(shell_slice_kernel<false>);
   allow_chain(shell_run_kernel<true, 0>);
   allow_chain(shell_run_kernel<false, 0>);
+  allow_chain(shell_run_kernel<true, 1>);
+  allow_chain(shell_run_kernel<false, 1>);
   const size_t smem = chain_bytes(block);
   if (sliced) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, shell_slice_kernel<true>, block, smem);
   else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, shell_run_kernel<true, 0>, block, smem);
@@ -1085,14 +1254,14 @@ cudaError_t launch_shell_run(const ShellModel* d_models, WorkQueue q, const floa
   none.per_warp = per_warp;
   none.core_lanes = core_lanes;
   none.burst_lanes = burst_lanes;
-  if (profile) shell_run_kernel<false, 1><<<grid, block, 0, s>>>(d_models, q, none, d_ktab);
+  if (profile) shell_run_kernel<false, 1><<<grid, block, chain_bytes(block), s>>>(d_models, q, none, d_ktab);
   else shell_run_kernel<false, 0><<<grid, block, chain_bytes(block), s>>>(d_models, q, none, d_ktab);
   return cudaGetLastError();
 }
 
 cudaError_t launch_shell_run_compact(const ShellModel* d_models, WorkQueue q, Compact c, const float* d_ktab,
                                      int grid, int block, int profile, cudaStream_t s) {
-  if (profile) shell_run_kernel<true, 1><<<grid, block, 0, s>>>(d_models, q, c, d_ktab);
+  if (profile) shell_run_kernel<true, 1><<<grid, block, chain_bytes(block), s>>>(d_models, q, c, d_ktab);
   else shell_run_kernel<true, 0><<<grid, block, chain_bytes(block), s>>>(d_models, q, c, d_ktab);
   return cudaGetLastError();
 }
