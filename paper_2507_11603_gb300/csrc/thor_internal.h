@@ -102,6 +102,7 @@ struct PhotonRec {
   float ox, oy, oz;   // FP32 offset from the anchor (saved as is: resuming is bit-exact)
   float X0, col_hi, col_lo;  // emitted X, HI column traversed (two-level sum)
   float kx, ky, kz, x, X, safe;
+  float fly, fly_tau;  // event interrupted in flight
   int32_t region;
   uint32_t nscat, ndust, iters, steps, event;
   unsigned long long pid;
@@ -137,6 +138,7 @@ struct SlotState {
   double *px, *py, *pz;              // FP64 anchor
   float *ox, *oy, *oz, *safe;        // FP32 offset, safety distance (saved as is)
   float *kx, *ky, *kz, *X, *x;
+  float *fly, *fly_tau;              // event interrupted in flight
   uint32_t* event;                   // RNG position: events done
   uint32_t *nscat, *ndust, *iters, *steps;
   int32_t* model;

@@ -331,7 +331,7 @@ extern "C" int thor_server_create(thor_ctx_t ctx, const thor_server_config* cfg,
   s->active.assign(R, nullptr);
   const size_t spec_bytes = (size_t)R * (s->max_bins + 2) * 8;
   const int64_t n = s->n_slots;
-  const size_t slot_bytes = (size_t)n * (3 * 8 + 4 * 4 + 5 * 4 + 4 + 4 * 4 + 4 + 8 + 1) + 24 * 256;
+  const size_t slot_bytes = (size_t)n * (3 * 8 + 4 * 4 + 7 * 4 + 4 + 4 * 4 + 4 + 8 + 1) + 26 * 256;
   s->slot_bytes = slot_bytes;
   bool ok = cudaMallocHost(&s->h_queue, queue_bytes(R)) == cudaSuccess &&
             cudaMallocHost(&s->h_out, 8 + sizeof(Tally) * R) == cudaSuccess &&
@@ -355,6 +355,7 @@ extern "C" int thor_server_create(thor_ctx_t ctx, const thor_server_config* cfg,
     st.safe = (float*)take(n * 4);
     st.kx = (float*)take(n * 4); st.ky = (float*)take(n * 4); st.kz = (float*)take(n * 4); st.X = (float*)take(n * 4);
     st.x = (float*)take(n * 4);
+    st.fly = (float*)take(n * 4); st.fly_tau = (float*)take(n * 4);
     st.event = (uint32_t*)take(n * 4);
     st.nscat = (uint32_t*)take(n * 4); st.ndust = (uint32_t*)take(n * 4); st.iters = (uint32_t*)take(n * 4);
     st.steps = (uint32_t*)take(n * 4);

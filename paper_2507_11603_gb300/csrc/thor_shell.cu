@@ -16,6 +16,14 @@ namespace thor {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
+// A flight of many sub-steps (thin gas: hundreds to thousands per event) is interrupted after
+// kFlySteps of them, and the packet's next turn resumes it: a warp's iteration is one event
+// per lane, and lanes with short events would wait for the longest flight of each (Mg II
+// sphere, 8500 sub-steps per photon: 5.4 of 32 lanes were active).  Photon::fly: kFlyNone, or
+// the distance along the segment, or kFlyBall inside the safety ball (the packet's own
+// position then holds the progress).
+constexpr int kFlySteps = 128;
+constexpr float kFlyNone = -1.0f, kFlyBall = -2.0f;
 constexpr uint32_t kLongLived = 1u << 14;
 constexpr uint32_t kPriBudget = 16;  // served rounds: budget multiple of a priority warp (one packet)  // served rounds: packets past this many events run one per warp
 
@@ -28,6 +36,7 @@ struct Photon {
   float safe;  // lower bound on the distance from p to any shell boundary (0 = unknown)
   int region;  // 1 = inside the empty cavity
   uint32_t nscat, ndust, iters, steps;
+  float fly, fly_tau;    // an event interrupted in flight (kFly*): where, and the depth left
   float X0;              // emitted lab frequency
   float col_hi, col_lo;  // HI column traversed (power-law shells), two-level FP32 sum
   StreamKey key;  // key.event: last completed event
@@ -68,6 +77,7 @@ __device__ __forceinline__ void shell_emit(const ShellModel& m, Photon& ph) {
   ph.region = (m.R_in > 0.0) ? 1 : 0;
   ph.safe = (float)m.R_out;
   ph.nscat = 0; ph.ndust = 0; ph.iters = 0; ph.steps = 0;
+  ph.fly = kFlyNone; ph.fly_tau = 0.0f;
 }
 
 // Move by s along k inside the safety ball: FP32 offset only.  The moves since the last
@@ -150,7 +160,8 @@ __device__ __forceinline__ bool dust_channel(const ShellModel& m, float kH, floa
   return __fmul_rn(R, __fadd_rn(kH, m.kapd)) >= kH;
 }
 
-// One event.  Returns 0 = continues, 1 = escaped, 2 = absorbed by dust, 3 = capped.
+// One event.  Returns 0 = continues, 1 = escaped, 2 = absorbed by dust, 3 = capped, -1 =
+// interrupted in flight (the same event goes on with the next call).
 // The gas-frame frequency x is carried along the ray: in the homologous flow it drifts
 // as x(s) = x0 - gam s in every direction, and a scattering leaves it at x_out at the
 // same point.  A conservative safety distance to the shell boundaries lets events whose
@@ -163,8 +174,11 @@ __device__ __forceinline__ bool needs_block2(const ShellModel& m) {
 
 // The packet's next event, from what it takes of its random words.
 __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restrict__ Ktab, const EventWords& w) {
-  ++ph.key.event;
-  float tau_rem = w.tau;
+  const bool resumed = ph.fly != kFlyNone;
+  float tau_rem = resumed ? ph.fly_tau : w.tau;
+  float s_seg = ph.fly;  // >= 0: resumed in a segment, there
+  ph.fly = kFlyNone;
+  int turn_steps = kFlySteps;
   float x_site, kH;
   for (;;) {
     if (ph.region) {  // empty cavity: straight to the inner sphere, lab X conserved
@@ -179,7 +193,9 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
       ph.safe = 0.0f;
     }
     // ---- fast path: the next (sub-)step lies inside the safety ball
-    if (m.gam == 0.0f) {
+    if (s_seg >= 0.0f) {
+      // resumed below
+    } else if (m.gam == 0.0f) {
       const StartStep st0 = start_step(m, voigt_start(m.a, ph.x, Ktab), tau_rem);
       kH = st0.kH;
       const float s = st0.s;
@@ -220,6 +236,10 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
       advance(ph, ds);
       ph.safe = __fmaf_rd(-ds, 1.000001f, ph.safe);
       ph.x -= m.gam * ds;
+      if (--turn_steps <= 0) {
+        ph.fly = kFlyBall; ph.fly_tau = tau_rem;
+        return -1;
+      }
       continue;
     }
     // ---- general path: sub-steps to the crossing or the next boundary, its distance exact
@@ -241,9 +261,15 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
       if (kap * Sf >= tau_rem) s_star = fminf(tau_rem / kap, Sf);
       else tau_rem -= kap * Sf;
     } else {
-      float s = 0.0f;
+      float s = fmaxf(s_seg, 0.0f);
+      s_seg = kFlyNone;
       bool have = false;
       for (;;) {
+        if (turn_steps <= 0) {
+          ph.fly = s; ph.fly_tau = tau_rem;
+          return -1;
+        }
+        --turn_steps;
         float s1 = s + m.ds_core;
         if (!have && !(s1 <= seg.lower)) {
           S = seg.exact(m, b, pp, next);
@@ -268,7 +294,8 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
         // Free flight: sub-steps in the wing, four at a time.  Their opacities do not depend
         // on one another (x drifts monotonically), so they are formed side by side and only
         // the depth is summed in order.
-        while (s + 4.25f * m.ds_core <= (have ? Sf : seg.lower)) {
+        while (turn_steps > 0 && s + 4.25f * m.ds_core <= (have ? Sf : seg.lower)) {
+          turn_steps -= 4;
           float e[5], kp[4];
           e[0] = s;
 #pragma unroll
@@ -318,6 +345,7 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
     if (next == 1) return 1;
     ph.region = 1;
   }
+  ++ph.key.event;
   ph.x = x_site;
   // Interaction (Sec. 3.4): channel i with probability tau_i / sum_i tau_i.
   bool dust = false;
@@ -424,7 +452,7 @@ __device__ __forceinline__ EventWords read_words(const WordBuf& wb, int s) {
 
 // Whether the packet's next event may be of the core kind (the cheap part of the test).
 __device__ __forceinline__ bool chain_kind(const ShellModel& m, const Photon& ph) {
-  return !ph.region && m.phase != PH_MIXED && fabsf(ph.x) <= THOR_VCORE_X && (m.gam == 0.0f || ph.safe >= m.ds_core);
+  return ph.fly == kFlyNone && !ph.region && m.phase != PH_MIXED && fabsf(ph.x) <= THOR_VCORE_X && (m.gam == 0.0f || ph.safe >= m.ds_core);
 }
 
 // One core event from its slot, committed where `go` holds and the event is of the core kind
@@ -582,8 +610,11 @@ __device__ __forceinline__ float from_line2(const ShellModel& m, float X2) {
 }
 
 __device__ int shell_event_pl(const ShellModel& m, Photon& ph, const float* __restrict__ Ktab, const EventWords& w) {
-  ++ph.key.event;
-  float tau_rem = w.tau;
+  const bool resumed = ph.fly != kFlyNone;
+  float tau_rem = resumed ? ph.fly_tau : w.tau;
+  float s_seg = ph.fly;
+  ph.fly = kFlyNone;
+  int turn_steps = kFlySteps;
   float kH, kH2 = 0.0f, kD;
   PLState site;
   for (;;) {
@@ -597,7 +628,7 @@ __device__ int shell_event_pl(const ShellModel& m, Photon& ph, const float* __re
       ph.region = 0;
       ph.safe = 0.0f;
     }
-    {  // short step with the rate at the current point
+    if (!(s_seg >= 0.0f)) {  // short step with the rate at the current point
       const PLState st = pl_state(m, (float)ph.px + ph.ox, (float)ph.py + ph.oy, (float)ph.pz + ph.oz, ph.k);
       const float x = (ph.X - st.v * st.mur) * m.inv_vth;
       const float H = voigt<false>(m.a, x, Ktab);
@@ -629,7 +660,8 @@ __device__ int shell_event_pl(const ShellModel& m, Photon& ph, const float* __re
     int next = 1;
     bool have = false;
     const float p0x = (float)ph.px, p0y = (float)ph.py, p0z = (float)ph.pz;
-    float s = 0.0f, s_star = -1.0f;
+    float s = fmaxf(s_seg, 0.0f), s_star = -1.0f;
+    s_seg = kFlyNone;
     // one sub-step of opacity kap, density nr, [s, s1]: true where the crossing lies in it
     auto sub_step = [&](float s1, float kap, float nr) {
       const float dtau = kap * (s1 - s);
@@ -646,6 +678,11 @@ __device__ int shell_event_pl(const ShellModel& m, Photon& ph, const float* __re
       return false;
     };
     for (;;) {
+      if (turn_steps <= 0) {
+        ph.fly = s; ph.fly_tau = tau_rem;
+        return -1;
+      }
+      --turn_steps;
       float s1 = s + m.ds_core;
       if (!have && !(s1 <= seg.lower)) {
         S = seg.exact(m, b, pp, next);
@@ -677,7 +714,8 @@ __device__ int shell_event_pl(const ShellModel& m, Photon& ph, const float* __re
       // flight is a chain of some 100 dependent instructions per sub-step otherwise); depth
       // and column are summed in order.
       bool cross = false;
-      while (s + 4.25f * m.ds_core <= (have ? Sf : seg.lower)) {
+      while (turn_steps > 0 && s + 4.25f * m.ds_core <= (have ? Sf : seg.lower)) {
+        turn_steps -= 4;
         float e[5], H[4], H2[4], nr[4];
         e[0] = s;
         bool wing = true;
@@ -724,6 +762,7 @@ __device__ int shell_event_pl(const ShellModel& m, Photon& ph, const float* __re
     if (next == 1) return 1;  // escapes with its lab X
     ph.region = 1;
   }
+  ++ph.key.event;
   // Interaction (Sec. 3.4): transition 1, transition 2 or dust in proportion to their
   // opacities (one uniform); dust absorbs.
   int ch = 0;
@@ -809,6 +848,7 @@ __device__ __forceinline__ void save_rec(const Photon& ph, PhotonRec& r) {
   r.ox = ph.ox; r.oy = ph.oy; r.oz = ph.oz;
   r.X0 = ph.X0; r.col_hi = ph.col_hi; r.col_lo = ph.col_lo;
   r.kx = ph.k.x; r.ky = ph.k.y; r.kz = ph.k.z;
+  r.fly = ph.fly; r.fly_tau = ph.fly_tau;
   r.x = ph.x; r.X = ph.X; r.safe = ph.safe;
   r.region = ph.region;
   r.nscat = ph.nscat; r.ndust = ph.ndust; r.iters = ph.iters; r.steps = ph.steps;
@@ -821,6 +861,7 @@ __device__ __forceinline__ void load_rec(const ShellModel& m, const PhotonRec& r
   ph.ox = r.ox; ph.oy = r.oy; ph.oz = r.oz;
   ph.X0 = r.X0; ph.col_hi = r.col_hi; ph.col_lo = r.col_lo;
   ph.k = make_float3(r.kx, r.ky, r.kz);
+  ph.fly = r.fly; ph.fly_tau = r.fly_tau;
   ph.x = r.x; ph.X = r.X; ph.safe = r.safe;
   ph.region = r.region;
   ph.nscat = r.nscat; ph.ndust = r.ndust; ph.iters = r.iters; ph.steps = r.steps;
@@ -949,9 +990,10 @@ __global__ void __launch_bounds__(256, 1) shell_run_kernel(const ShellModel* __r
       do {
         general_words(m, ph, wb, general, at);
         if (general) {
-          const EventWords w = read_words(wb, at.cur++ * at.P + at.rank);
+          const EventWords w = read_words(wb, at.cur * at.P + at.rank);
           const int st = kProfile ? shell_event_pl(m, ph, sK, w) : shell_event(m, ph, sK, w);
-          if (st) {
+          if (st >= 0) ++at.cur;
+          if (st > 0) {
             if (st == 1) { ++lt.esc; tally_spectrum(m, ph.X); }
             else if (st == 2) ++lt.abs;
             else ++lt.cap;
@@ -1058,6 +1100,7 @@ __global__ void __launch_bounds__(256, 1) shell_slice_kernel(const ShellModel* _
     ph.safe = st.safe[slot];
     ph.X0 = 0.0f; ph.col_hi = 0.0f; ph.col_lo = 0.0f;  // raw records are not served
     ph.region = st.region[slot];
+    ph.fly = st.fly[slot]; ph.fly_tau = st.fly_tau[slot];
     ph.nscat = st.nscat[slot]; ph.ndust = st.ndust[slot]; ph.iters = st.iters[slot]; ph.steps = st.steps[slot];
     active = true;
   }
@@ -1114,10 +1157,11 @@ __global__ void __launch_bounds__(256, 1) shell_slice_kernel(const ShellModel* _
       do {
         general_words(mr, ph, wb, general, at);
         if (general) {
-          const EventWords w = read_words(wb, at.cur++ * at.P + at.rank);
+          const EventWords w = read_words(wb, at.cur * at.P + at.rank);
           const int r = (kMixed && mr.profile) ? shell_event_pl(mr, ph, sK, w) : shell_event(mr, ph, sK, w);
+          if (r >= 0) ++at.cur;
           ++n;
-          if (r) { finish_global(mr, ph, r); active = false; fin = true; }
+          if (r > 0) { finish_global(mr, ph, r); active = false; fin = true; }
           general = active && !(chain && chain_kind(mr, ph));
         }
       } while (!__any_sync(kFull, fin) && ++n_gen < kCrowdDepth && n_gen + depth < budget - ev &&
@@ -1151,6 +1195,7 @@ __global__ void __launch_bounds__(256, 1) shell_slice_kernel(const ShellModel* _
       o.ox[j] = ph.ox; o.oy[j] = ph.oy; o.oz[j] = ph.oz; o.safe[j] = ph.safe;
       o.kx[j] = ph.k.x; o.ky[j] = ph.k.y; o.kz[j] = ph.k.z;
       o.X[j] = ph.X; o.x[j] = ph.x; o.region[j] = (uint8_t)ph.region;
+      o.fly[j] = ph.fly; o.fly_tau[j] = ph.fly_tau;
       o.nscat[j] = ph.nscat; o.ndust[j] = ph.ndust; o.iters[j] = ph.iters; o.steps[j] = ph.steps;
     }
   }
@@ -1176,6 +1221,7 @@ __device__ __forceinline__ void copy_slot(const SlotState& a, int64_t i, const S
   b.ox[j] = a.ox[i]; b.oy[j] = a.oy[i]; b.oz[j] = a.oz[i]; b.safe[j] = a.safe[i];
   b.kx[j] = a.kx[i]; b.ky[j] = a.ky[i]; b.kz[j] = a.kz[i]; b.X[j] = a.X[i]; b.x[j] = a.x[i];
   b.event[j] = a.event[i];
+  b.fly[j] = a.fly[i]; b.fly_tau[j] = a.fly_tau[i];
   b.nscat[j] = a.nscat[i]; b.ndust[j] = a.ndust[i]; b.iters[j] = a.iters[i]; b.steps[j] = a.steps[i];
   b.model[j] = a.model[i]; b.pid[j] = a.pid[i]; b.region[j] = a.region[i];
 }
