@@ -3,23 +3,41 @@
 // sightlines parallel to z, v_k = (k + 1/2) dv_cell + v_los,k, v_b = (b + 1/2) dv_bin,
 // nearest periodic image in a box of width V = nz dv_cell = n_bins dv_bin.
 //
-// One CTA per sightline.  The sightline's cells are staged in shared memory (velocity,
-// 1/v_th, a, a^2, amplitudes); every thread owns n_bins / blockDim bins and sweeps all
-// cells, so each Voigt evaluation costs one shared-memory broadcast read and no global
-// traffic.  Velocities are 32-bit fixed point with the period V mapped onto 2^32
-// (unit V / 2^32, about 5e-7 km/s here): v_b - v_k wraps modulo 2^32, which is the
+// One CTA per sightline (several where there are few).  The sightline's cells are staged in
+// shared memory (velocity, 1/v_th, a, a^2, amplitudes).  Velocities are 32-bit fixed point with
+// the period V mapped onto 2^32 (unit V / 2^32): v_b - v_k wraps modulo 2^32, which is the
 // nearest periodic image when read as a signed integer, exactly and without a branch.
-// FP32 accumulation in two levels (blocks of 32 cells, then the running total) keeps
-// the summation error below 1e-6 relative for positive terms.
+//
+// Evaluating every cell at every bin is bound by instruction issue (0.97 of the issue peak:
+// 22 lane instructions per pair, 5.5 ms for 4096 sightlines of 1024 cells x 2048 bins), and most
+// pairs lie far out in the Lorentzian wing, where a cell's profile is smooth on the scale of
+// many bins.  So the spectrum is cut into intervals of at most 64 bins and 8 coarse ones:
+//   far    a cell whose line centre is at least kFar half-widths from an interval's centre, with
+//          the interval outside |x| < 6, contributes at the interval's 16 Chebyshev nodes instead
+//          of at its bins -- on the coarse intervals where it is far from one, else on the fine
+//          ones.  With the pole of 1/x^2 at kFar = 2.25 half-widths the interpolation error is
+//          below (kFar + sqrt(kFar^2 - 1))^-16 x 68 = 7e-9 of the contribution, under FP32's own
+//          rounding; all contributions are positive, so it is the same for the sum;
+//   near   the other cells (the core |x| < 6, the wing next to it, and the cells opposite the
+//          interval, where the nearest image changes side) are evaluated at each bin.
+// The node sums become Chebyshev coefficients once per interval and each bin evaluates them.
+// FP32 accumulation in two levels (blocks of 32 cells, then the running total).
 #include "thor_device.cuh"
 #include "thor_internal.h"
 
 namespace thor {
 namespace {
 
+constexpr unsigned kFull = 0xffffffffu;
 constexpr int kForestThreads = 256;
-constexpr int kMaxBinsPerThread = 8;  // n_bins <= 2048 per pass
-constexpr int kCellChunk = 1024;    // cells staged per pass
+constexpr int kForestWarps = kForestThreads / 32;
+constexpr int kCellChunk = 1024;  // cells staged per pass
+constexpr int kMaxBins = 2048;
+constexpr int kIvBins = 64;       // bins per interval at most (two per lane)
+constexpr int kMaxIv = kMaxBins / kIvBins;
+constexpr int kCoarse = 8;        // coarse intervals
+constexpr int kNodes = 16;        // Chebyshev nodes per interval
+constexpr float kFar = 2.25f;
 
 // Wing (|x| >= 6) without the a/sqrt(pi) factor: t g(t), t = 1/(x^2 + a^2), g the
 // degree-4 fit of thor_device.cuh (one polynomial for the whole wing, no branch).  MUFU
@@ -29,73 +47,216 @@ __device__ __forceinline__ float wing_tP(float a2, float x2) {
   return t * wing_g(t);
 }
 
-// kBinsPerThread bins per thread per pass (1, 2, 4 or 8, the smallest that covers n_bins
-// in one pass, so short spectra do not evaluate bins that do not exist)
-template <int kBinsPerThread>
+struct ForestCells {
+  float4 p[kCellChunk];        // (v as fixed point bits, unit / v_th, a, a^2)
+  float2 amp[kCellChunk];      // (n sigma_0 ds, n sigma_0 ds a / sqrt(pi))
+  uint32_t core[kCellChunk];   // |x| = 6 in fixed point, rounded up; 2^32 - 1: always near
+};
+
+// A cell's line centre d from an interval's centre (fixed point, wrapped), half-width h: far?
+// The interval must also lie on one side of the cell's antipode (nearest image).
+__device__ __forceinline__ bool is_far(uint32_t d, uint32_t h, uint32_t core) {
+  const uint32_t ad = (d & 0x80000000u) ? 0u - d : d;
+  const uint32_t lim = max((uint32_t)(kFar * (float)h), core + min(h, ~core));
+  return ad >= lim && ad <= 0x80000000u - h - 2u;
+}
+
+// One wing term at a node or bin at fixed-point velocity v.
+__device__ __forceinline__ float wing_at(uint32_t v, const float4& c, float ampw) {
+  const float x = (float)(int32_t)(v - __float_as_uint(c.x)) * c.y;
+  return ampw * wing_tP(c.w, x * x);
+}
+__device__ __forceinline__ float profile_at(uint32_t v, const float4& c, const float2& am, const float* sK, float sum) {
+  const float x = (float)(int32_t)(v - __float_as_uint(c.x)) * c.y;  // nearest image, in Doppler widths
+  const float x2 = x * x;
+  if (x2 >= 36.0f) return __fmaf_rn(am.y, wing_tP(c.w, x2), sum);
+  return __fmaf_rn(am.x, voigt_core<true>(c.z, fabsf(x), x2, sK), sum);
+}
+
+// Cells of the mask (bit k: cell j0 + k) at the interval's nodes, two cells at a time: lanes
+// 0-15 and 16-31 hold the 16 nodes each.
+__device__ __forceinline__ float node_terms(const ForestCells& sc, int j0, unsigned mask, uint32_t vnode, float sum) {
+  const bool upper = (threadIdx.x & 16u) != 0u;
+  while (mask) {
+    int k = __ffs(mask) - 1;
+    mask &= mask - 1u;
+    bool on = true;
+    if (upper) {
+      on = mask != 0u;
+      k = on ? __ffs(mask) - 1 : k;
+    }
+    mask &= mask - 1u;  // 0 stays 0
+    const float w = wing_at(vnode, sc.p[j0 + k], sc.amp[j0 + k].y);
+    sum += on ? w : 0.0f;
+  }
+  return sum;
+}
+
+// Chebyshev coefficient k of node values f: (2/16) sum_n f_n cos(k pi (n + 1/2) / 16).
+__device__ __forceinline__ float cheb_coef(const float* f, int k, const float* cosT) {
+  float s = 0.0f;
+#pragma unroll
+  for (int n = 0; n < kNodes; ++n) s = __fmaf_rn(f[n], cosT[(k * (2 * n + 1)) & 63], s);
+  return s * (2.0f / kNodes);
+}
+__device__ __forceinline__ float cheb_eval(const float* c, float xi) {  // Clenshaw
+  const float x2 = 2.0f * xi;
+  float b1 = 0.0f, b2 = 0.0f;
+#pragma unroll
+  for (int k = kNodes - 1; k >= 1; --k) {
+    const float b = __fmaf_rn(x2, b1, c[k] - b2);
+    b2 = b1;
+    b1 = b;
+  }
+  return __fmaf_rn(xi, b1, __fmaf_rn(0.5f, c[0], -b2));
+}
+
+// n_iv = 2^iv_log2 intervals; the CTA's blockIdx.y takes the iv_cta intervals from iv_cta
+// blockIdx.y on; `splits` warps share an interval's cells where there are fewer intervals
+// than warps.
 __global__ void __launch_bounds__(kForestThreads, 4) forest_kernel(
     const float* __restrict__ nHI, const float* __restrict__ T, const float* __restrict__ vlos, int nx, int ny,
-    int nz, int64_t first, double ds_cm, double dv_cell, int n_bins, double dv_bin, float* __restrict__ tau,
-    const float* __restrict__ gK) {
+    int nz, int64_t first, double ds_cm, double dv_cell, int n_bins, double dv_bin, int iv_log2, int iv_cta,
+    float* __restrict__ tau, const float* __restrict__ gK) {
   __shared__ __align__(16) float sK[THOR_VOIGT_NINT * THOR_VOIGT_NCOEF];
-  __shared__ float4 sCell[kCellChunk];  // (v as fixed point bits, unit / v_th, a, a^2)
-  __shared__ float2 sAmp[kCellChunk];   // (n sigma_0 ds, n sigma_0 ds a / sqrt(pi))
+  __shared__ ForestCells sc;
+  __shared__ float sAcc[kMaxIv * kIvBins];       // direct sums: task, bin of the interval
+  __shared__ float sFine[kMaxIv * kNodes];       // node sums per task, then coefficients per interval
+  __shared__ float sCoarse[kCoarse][kNodes];     // node sums, then coefficients
+  __shared__ float sCos[64];                     // cos(pi m / 32)
   load_ktab(sK, gK);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t sl = first + blockIdx.x;
   const int ix = (int)(sl % nx), iy = (int)(sl / nx);
   const double V = (double)nz * dv_cell;
   const double to_fix = 4294967296.0 / V;  // fixed-point units per km/s
+  const double to_x = 1.0 / (THOR_VTH1 * to_fix);
+  const double amp1 = THOR_SIG1 * ds_cm;
   const int64_t plane = (int64_t)nx * ny;
+  const int n_iv = 1 << iv_log2, iv0 = blockIdx.y * iv_cta;
+  const int splits = iv_cta >= kForestWarps ? 1 : kForestWarps / iv_cta, n_task = iv_cta * splits;
+  const uint32_t h = iv_log2 ? 1u << (31 - iv_log2) : 0x80000000u;  // half-width of an interval
+  const bool far_on = iv_log2 >= 3, coarse_on = iv_log2 >= 4;
+  constexpr uint32_t hc = 0x80000000u / kCoarse;
+  const int coarse_shift = iv_log2 - 3;
+  if (tid < 64) sCos[tid] = cospif((float)tid / 32.0f);
+  for (int j = tid; j < kMaxIv * kIvBins; j += kForestThreads) sAcc[j] = 0.0f;
+  for (int j = tid; j < kMaxIv * kNodes; j += kForestThreads) sFine[j] = 0.0f;
+  if (tid < kCoarse * kNodes) sCoarse[tid / kNodes][tid % kNodes] = 0.0f;
+  __syncthreads();
+  const float xi_node = sCos[2 * (lane & 15) + 1];
+  const int32_t off_fine = __float2int_rn(xi_node * (float)h), off_coarse = __float2int_rn(xi_node * (float)hc);
+  auto first_bin = [&](int iv) { return (2 * iv * n_bins + n_iv - 1) >> (iv_log2 + 1); };  // centre at or after its start
+  auto bin_fix = [&](int b) {
+    return (uint32_t)(unsigned long long)llrint(((double)b + 0.5) * dv_bin * to_fix);
+  };
 
-  for (int b0 = 0; b0 < n_bins; b0 += kForestThreads * kBinsPerThread) {
-    // bin q of this thread sits q * blockDim bins after its first bin
-    uint32_t vb[kBinsPerThread];
-    float acc[kBinsPerThread], part[kBinsPerThread];
-#pragma unroll
-    for (int q = 0; q < kBinsPerThread; ++q) {
-      const double v = ((double)(b0 + threadIdx.x + q * kForestThreads) + 0.5) * dv_bin;
-      vb[q] = (uint32_t)(unsigned long long)llrint(fmod(v, V) * to_fix);
-      acc[q] = 0.0f;
-      part[q] = 0.0f;
+  for (int k0 = 0; k0 < nz; k0 += kCellChunk) {
+    const int nk = min(kCellChunk, nz - k0);
+    __syncthreads();
+    for (int j = tid; j < nk; j += kForestThreads) {
+      const int64_t c = (int64_t)(k0 + j) * plane + (int64_t)iy * nx + ix;
+      const double rT = rsqrt((double)__ldg(T + c));
+      const double vk = ((double)(k0 + j) + 0.5) * dv_cell + (double)__ldg(vlos + c);
+      const uint32_t vfix = (uint32_t)(unsigned long long)llrint(vk * to_fix);  // modulo the period
+      const double amp = (double)__ldg(nHI + c) * amp1 * rT;
+      const double a = THOR_A1 * rT;
+      const float iv = (float)(rT * to_x), ampw = (float)(amp * a * 0.5641895835477563);
+      sc.p[j] = make_float4(__uint_as_float(vfix), iv, (float)a, (float)(a * a));
+      sc.amp[j] = make_float2((float)amp, ampw);
+      // cells that are not finite (or near overflow) stay near everywhere: each bin then gets
+      // the plain sum
+      const float w = __fdividef(6.00002f, iv);
+      sc.core[j] = (w < 2.0e9f && w > 0.0f && fabsf(ampw) < 1e30f) ? (uint32_t)w + 2u : 0xffffffffu;
     }
-    for (int k0 = 0; k0 < nz; k0 += kCellChunk) {
-      const int nk = min(kCellChunk, nz - k0);
-      __syncthreads();
-      for (int j = threadIdx.x; j < nk; j += kForestThreads) {
-        const int64_t c = (int64_t)(k0 + j) * plane + (int64_t)iy * nx + ix;
-        const double Tc = (double)__ldg(T + c);
-        const double rT = 1.0 / sqrt(Tc);
-        double vk = ((double)(k0 + j) + 0.5) * dv_cell + (double)__ldg(vlos + c);
-        vk -= V * floor(vk / V);  // into [0, V)
-        const uint32_t vfix = (uint32_t)(unsigned long long)llrint(vk * to_fix);  // 2^32 wraps to 0
-        const double amp = (double)__ldg(nHI + c) * THOR_SIG1 * rT * ds_cm;
-        const double a = THOR_A1 * rT;
-        sCell[j] = make_float4(__uint_as_float(vfix), (float)(rT / (THOR_VTH1 * to_fix)), (float)a, (float)(a * a));
-        sAmp[j] = make_float2((float)amp, (float)(amp * a * 0.5641895835477563));
-      }
-      __syncthreads();
-      for (int j = 0; j < nk; ++j) {
-        const float4 cv = sCell[j];
-        const float2 am = sAmp[j];
-        const uint32_t vk = __float_as_uint(cv.x);
-#pragma unroll
-        for (int q = 0; q < kBinsPerThread; ++q) {
-          const float x = (float)(int32_t)(vb[q] - vk) * cv.y;  // nearest image, in Doppler widths
-          const float x2 = x * x;
-          if (x2 >= 36.0f) part[q] = __fmaf_rn(am.y, wing_tP(cv.w, x2), part[q]);
-          else part[q] = __fmaf_rn(am.x, voigt_core<true>(cv.z, fabsf(x), x2, sK), part[q]);
+    __syncthreads();
+    if (coarse_on) {  // one coarse interval per warp
+      const int c = warp;
+      if ((((c + 1) << coarse_shift) > iv0) && ((c << coarse_shift) < iv0 + iv_cta)) {
+        const uint32_t vc = (uint32_t)c * (2u * hc) + hc;
+        float sum = 0.0f;
+        for (int j0 = 0; j0 < nk; j0 += 32) {
+          const int j = j0 + lane;
+          bool far = false;
+          if (j < nk) far = is_far(vc - __float_as_uint(sc.p[j].x), hc, sc.core[j]);
+          sum += node_terms(sc, j0, __ballot_sync(kFull, far), vc + (uint32_t)off_coarse, 0.0f);
         }
-        if ((j & 31) == 31) {
-#pragma unroll
-          for (int q = 0; q < kBinsPerThread; ++q) { acc[q] += part[q]; part[q] = 0.0f; }
-        }
+        sum += __shfl_down_sync(kFull, sum, 16);
+        if (lane < kNodes) sCoarse[c][lane] += sum;
       }
-#pragma unroll
-      for (int q = 0; q < kBinsPerThread; ++q) { acc[q] += part[q]; part[q] = 0.0f; }
     }
-#pragma unroll
-    for (int q = 0; q < kBinsPerThread; ++q) {
-      const int b = b0 + threadIdx.x + q * kForestThreads;
-      if (b < n_bins) tau[(size_t)blockIdx.x * n_bins + b] = acc[q];
+    for (int task = warp; task < n_task; task += kForestWarps) {
+      const int iv = iv0 + task / splits, split = task % splits;
+      const uint32_t vc = (uint32_t)iv * (2u * h) + h;  // interval centre
+      const uint32_t vcc = (uint32_t)(iv >> (coarse_on ? coarse_shift : 0)) * (2u * hc) + hc;
+      const int b0 = first_bin(iv), nb = first_bin(iv + 1) - b0;
+      const uint32_t v0 = bin_fix(b0 + lane), v1 = bin_fix(b0 + lane + 32);
+      const bool two = nb > 32;
+      float acc0 = 0.0f, acc1 = 0.0f, sum = 0.0f;
+      for (int j0 = 32 * split; j0 < nk; j0 += 32 * splits) {
+        const int j = j0 + lane;
+        bool near = false, fine = false;
+        if (j < nk) {
+          const uint32_t vk = __float_as_uint(sc.p[j].x), core = sc.core[j];
+          const bool coarse = coarse_on && is_far(vcc - vk, hc, core);
+          fine = far_on && !coarse && is_far(vc - vk, h, core);
+          near = !fine && !coarse;
+        }
+        unsigned mask = __ballot_sync(kFull, near);
+        sum += node_terms(sc, j0, __ballot_sync(kFull, fine), vc + (uint32_t)off_fine, 0.0f);
+        float p0 = 0.0f, p1 = 0.0f;
+        while (mask) {
+          const int k = j0 + __ffs(mask) - 1;
+          mask &= mask - 1u;
+          const float4 c = sc.p[k];
+          const float2 am = sc.amp[k];
+          p0 = profile_at(v0, c, am, sK, p0);
+          if (two) p1 = profile_at(v1, c, am, sK, p1);
+        }
+        acc0 += p0;
+        acc1 += p1;
+      }
+      sum += __shfl_down_sync(kFull, sum, 16);
+      if (lane < kNodes) sFine[task * kNodes + lane] += sum;
+      sAcc[task * kIvBins + lane] += acc0;
+      sAcc[task * kIvBins + lane + 32] += acc1;
+    }
+  }
+  __syncthreads();
+  // node sums to coefficients: coarse first, then each interval's own nodes plus the coarse sum there
+  if (coarse_on) {
+    const float c = cheb_coef(sCoarse[warp], lane & 15, sCos);
+    __syncwarp();
+    if (lane < kNodes) sCoarse[warp][lane] = c;
+  }
+  __syncthreads();
+  for (int i = warp; i < iv_cta; i += kForestWarps) {
+    const int iv = iv0 + i;
+    if (far_on) {
+      float f = 0.0f;
+      for (int s = 0; s < splits; ++s) f += sFine[(i * splits + s) * kNodes + (lane & 15)];
+      if (coarse_on) {
+        const int c = iv >> coarse_shift;
+        const uint32_t v = (uint32_t)iv * (2u * h) + h + (uint32_t)off_fine, vc = (uint32_t)c * (2u * hc) + hc;
+        f += cheb_eval(sCoarse[c], (float)(int32_t)(v - vc) * (1.0f / (float)hc));
+      }
+      __syncwarp();
+      float* row = sFine + i * splits * kNodes;
+      if (lane < kNodes) row[lane] = f;
+      __syncwarp();
+      const float c = cheb_coef(row, lane & 15, sCos);
+      __syncwarp();
+      if (lane < kNodes) row[lane] = c;
+      __syncwarp();
+    }
+    const int b0 = first_bin(iv), nb = first_bin(iv + 1) - b0;
+    const uint32_t vc = (uint32_t)iv * (2u * h) + h;
+    for (int q = lane; q < nb; q += 32) {
+      float t = 0.0f;
+      for (int s = 0; s < splits; ++s) t += sAcc[(i * splits + s) * kIvBins + q];
+      if (far_on)
+        t += cheb_eval(sFine + i * splits * kNodes, (float)(int32_t)(bin_fix(b0 + q) - vc) * (1.0f / (float)h));
+      tau[(size_t)blockIdx.x * n_bins + b0 + q] = t;
     }
   }
 }
@@ -105,23 +266,24 @@ __global__ void __launch_bounds__(kForestThreads, 4) forest_kernel(
 cudaError_t launch_forest(const float* nHI, const float* T, const float* vlos, int nx, int ny, int nz, int64_t first,
                           int64_t count, double ds_cm, double dv_cell, int n_bins, double dv_bin, float* tau,
                           const float* d_ktab, cudaStream_t s) {
+  // Intervals of at most 64 bins, a power of two of them.  From 8 on the far cells pay (a far
+  // cell costs 16 node terms per interval; up to 128 bins nearly every cell is near anyway).
+  int iv_log2 = 0;
+  while ((kIvBins << iv_log2) < n_bins) ++iv_log2;
+  if (n_bins > 128 && iv_log2 < 3) iv_log2 = 3;
+  // Few sightlines: several CTAs share one, each with some of its intervals (and its own copy of
+  // the cells), until there are two per SM.
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  int iv_cta = 1 << iv_log2;
+  while (iv_cta > 1 && count * ((1 << iv_log2) / iv_cta) < 2 * (int64_t)sms) iv_cta >>= 1;
   int64_t done = 0;
   while (done < count) {  // grid.x limit
     const int64_t n = count - done < (int64_t)0x7fffffff ? count - done : (int64_t)0x7fffffff;
-    float* out = tau + (size_t)done * n_bins;
-    const int64_t f = first + done;
-    if (n_bins <= kForestThreads)
-      forest_kernel<1><<<(unsigned)n, kForestThreads, 0, s>>>(nHI, T, vlos, nx, ny, nz, f, ds_cm, dv_cell, n_bins, dv_bin,
-                                                               out, d_ktab);
-    else if (n_bins <= 2 * kForestThreads)
-      forest_kernel<2><<<(unsigned)n, kForestThreads, 0, s>>>(nHI, T, vlos, nx, ny, nz, f, ds_cm, dv_cell, n_bins, dv_bin,
-                                                               out, d_ktab);
-    else if (n_bins <= 4 * kForestThreads)
-      forest_kernel<4><<<(unsigned)n, kForestThreads, 0, s>>>(nHI, T, vlos, nx, ny, nz, f, ds_cm, dv_cell, n_bins, dv_bin,
-                                                               out, d_ktab);
-    else
-      forest_kernel<kMaxBinsPerThread><<<(unsigned)n, kForestThreads, 0, s>>>(nHI, T, vlos, nx, ny, nz, f, ds_cm,
-                                                                              dv_cell, n_bins, dv_bin, out, d_ktab);
+    forest_kernel<<<dim3((unsigned)n, (unsigned)((1 << iv_log2) / iv_cta)), kForestThreads, 0, s>>>(
+        nHI, T, vlos, nx, ny, nz, first + done, ds_cm, dv_cell, n_bins, dv_bin, iv_log2, iv_cta,
+        tau + (size_t)done * n_bins, d_ktab);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     done += n;
