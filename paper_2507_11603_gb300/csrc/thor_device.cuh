@@ -141,47 +141,49 @@ struct Rng : StreamKey {
 };
 
 // ------------------------------------------------------------------------------
-// Work sharing in the tail of a one-launch photon loop (shell and grid): warps that ran
-// dry wait for packets that crowded warps give away.  share: [0] pool entries reserved,
-// [1] taken, [2] warps waiting, [3] photons finished, [4] a taken entry never became ready;
-// ready[i] is set (after a fence) once entry i is written.
-// Lane 0 of a warp whose lanes are all done (queue drained) takes the next pool entry
-// (compare-and-swap on the taken counter), or gives up once every photon of the run has
-// finished or after kPollMax polls (a packet still in the pool then is resumed by the
-// host).  Between polls it sleeps, backing off to 32 us, so that a thousand waiting warps
-// load the counters' cache lines little.  Returns the pool index, or -1.
+// Work sharing in the tail of a one-launch photon loop: warps that ran dry wait for packets
+// that crowded warps give away.  share: [0] pool entries reserved by givers, [1] tickets of
+// waiting warps (ticket i takes entry i), [3] photons finished.
+// ready[i]: 0, then 1 once entry i is written (after a fence), or 2 once ticket i gave up.
+// Each waiting warp polls its own entry's flag and sleeps in between, backing off to 32 us.
+// (With one counter that all waiting warps raced for by compare-and-swap, a thousand of them
+// held up runs of short histories: 5452 photons through a thin shell took 0.5 ms, 0.04 ms
+// without sharing.)  Lane 0 of a warp whose lanes are all done: returns its pool index, or -1
+// once every photon of the run has finished or after kPollMax polls (the giver then keeps the
+// packet; one written beyond the last ticket is resumed by the host).
 constexpr uint32_t kPollMax = 1u << 24;
 __device__ __forceinline__ unsigned long long vload(const unsigned long long* p) {
   return *(volatile const unsigned long long*)p;
 }
-static __device__ __noinline__ long long pool_take(unsigned long long* share, const uint32_t* ready,
+static __device__ __noinline__ long long pool_take(unsigned long long* share, uint32_t* ready,
                                                    unsigned long long n_total) {
-  atomicAdd(&share[2], 1ull);
-  long long got = -1;
+  if (vload(&share[3]) >= n_total) return -1;
+  const unsigned long long t = atomicAdd(&share[1], 1ull);
+  if (t >= n_total) return -1;  // no such entry: at most one per photon
   unsigned ns = 64;
   for (uint32_t it = 0; it < kPollMax; ++it) {
-    const unsigned long long t = vload(&share[1]), n = vload(&share[0]);
-    if (t < n) {
-      if (atomicCAS(&share[1], t, t + 1ull) == t) { got = (long long)t; break; }
-      continue;
+    if (*(volatile uint32_t*)&ready[t]) {
+      __threadfence();
+      return (long long)t;
     }
-    if (vload(&share[3]) >= n_total) break;
+    if (vload(&share[3]) >= n_total) return -1;
     __nanosleep(ns);
     ns = ns < 32768u ? 2u * ns : 32768u;
   }
-  atomicAdd(&share[2], ~0ull);  // -1
-  if (got >= 0) {  // the giver writes the record, then the flag: wait for the flag (short)
-    uint32_t it = 0;
-    while (*(volatile const uint32_t*)&ready[got] == 0u && ++it < kPollMax) __nanosleep(32);
-    if (it >= kPollMax) { atomicAdd(&share[4], 1ull); return -1; }
-    __threadfence();
-  }
-  return got;
+  if (atomicCAS(&ready[t], 0u, 2u) == 0u) return -1;
+  __threadfence();
+  return (long long)t;
 }
-// How many packets a warp with `live` packets gives away: all but one, up to the warps
-// waiting beyond the entries already in the pool.
+// The giver's half, after the record is written: false where ticket j gave up (the giver keeps
+// the packet).
+__device__ __forceinline__ bool pool_put(uint32_t* ready, unsigned long long j) {
+  __threadfence();
+  return atomicCAS(&ready[j], 0u, 1u) == 0u;
+}
+// How many packets a warp with `live` packets gives away: all but one, up to the tickets beyond
+// the entries already reserved.
 __device__ __forceinline__ long long pool_give_count(const unsigned long long* share, int live) {
-  const long long waiting = (long long)vload(&share[2]) - (long long)(vload(&share[0]) - vload(&share[1]));
+  const long long waiting = (long long)(vload(&share[1]) - vload(&share[0]));
   return min((long long)(live - 1), waiting);
 }
 
@@ -622,6 +624,62 @@ __device__ __forceinline__ void scatter_words(EventWords& w, const Rng& rng, int
   w.st = sqrt_approx(fmaxf(0.0f, __fmaf_rn(-w.mu, w.mu, 1.0f)));
   __sincosf(2.0f * kPiF * rng.u(W_PHI), &w.sp, &w.cp);
   w.mixed = rng.u(W_MIXED);
+}
+
+// ---- event words formed by a whole warp ----------------------------------------------
+// All 32 lanes form what the next D events of the warp's P packets take from their words, one
+// slot per lane at a time, into shared memory (P D <= kWordSlots): the random numbers are
+// about half of an event's instructions, and a warp with few packets would form them on one
+// lane each.  In a full warp the slots are formed D at a time by a loop of their own, which
+// keeps the event loop's code short.
+constexpr int kWordSlots = 128;
+constexpr uint32_t kWordBlock2 = 1u, kWordLog = 2u;  // the third block is drawn; tau by __logf
+struct WordBuf {         // one per warp
+  float4 a[kWordSlots];  // tau, R1, R2, R3
+  float4 b[kWordSlots];  // mu, st, cos phi, sin phi
+  float4 c[kWordSlots];  // u1, u2, v1, v2
+  float4 d[kWordSlots];  // Rm, channel, mixed, albedo
+  uint4 own[32];         // photon id, last completed event, flags (owners in lane order)
+  uint4 key[32];         // stream key, phase function, core-skipping threshold
+};
+// Where a lane's slots lie: slot (cur P + rank) holds its next event while cur < D.
+struct WordPos {
+  int P = 1, D = 0, rank = 0, cur = 0;
+};
+// The next D events of every packet in `mine` lanes; key.event is the packet's last event.
+// Called by all 32 lanes, converged.
+__device__ __forceinline__ void form_words(WordBuf& wb, const StreamKey& sk, uint32_t flags, int phase, float xcrit,
+                                           bool mine, int D, WordPos& at) {
+  const int lane = (int)(threadIdx.x & 31u);
+  const unsigned owners = __ballot_sync(0xffffffffu, mine);
+  const int P = __popc(owners);
+  at.P = P; at.D = mine ? D : 0; at.cur = 0;
+  at.rank = mine ? __popc(owners & ((1u << lane) - 1u)) : 0;
+  if (mine) {
+    wb.own[at.rank] = make_uint4(sk.p0, sk.p1, sk.event, flags);
+    wb.key[at.rank] = make_uint4(sk.k0, sk.k1, (uint32_t)phase, __float_as_uint(xcrit));
+  }
+  __syncwarp();
+  for (int s = lane; s < P * D; s += 32) {  // slot d P + r: event d of the owner of rank r
+    const int d = s / P, r = s - d * P;
+    const uint4 own = wb.own[r], key = wb.key[r];
+    Rng q;
+    q.k0 = key.x; q.k1 = key.y; q.p0 = own.x; q.p1 = own.y;
+    q.v[8] = q.v[9] = q.v[10] = 0u;  // not drawn: not used
+    q.start_event(own.z + 1u + (uint32_t)d, (own.w & kWordBlock2) ? 3u : 2u);
+    EventWords w;
+    scatter_words(w, q, (int)key.z, __uint_as_float(key.w));
+    const float t = q.u(W_TAU);
+    wb.a[s] = make_float4((own.w & kWordLog) ? -__logf(t) : -ln_fast(t), w.R1, w.R2, w.R3);
+    wb.b[s] = make_float4(w.mu, w.st, w.cp, w.sp);
+    wb.c[s] = make_float4(w.u1, w.u2, w.v1, w.v2);
+    wb.d[s] = make_float4(w.Rm, q.u(W_CHANNEL), w.mixed, q.u(W_ALBEDO));
+  }
+  __syncwarp();
+}
+__device__ __forceinline__ EventWords read_words(const WordBuf& wb, int s) {
+  const float4 a = wb.a[s], b = wb.b[s], c = wb.c[s], d = wb.d[s];
+  return EventWords{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w, d.x, d.y, d.z, d.w};
 }
 
 template <int kForm = kTurnPower, int kFormIso = kTurnPower>

@@ -112,7 +112,7 @@ struct GPhoton {
   float3 k;
   float X;
   uint32_t nscat, ndust, iters, steps;
-  Rng rng;
+  StreamKey key;  // key.event: the current event (the last one between events)
   unsigned long long pid;
 };
 
@@ -251,10 +251,12 @@ __device__ __forceinline__ void deposit(const GridModel& m, const double p[3], i
 // Emission (Sec. 2.1, 3.4): cell with probability n_HI^2 / sum, uniform position in it,
 // isotropic direction, thermal x ~ N(0, 1/2) in the cell frame; peel at emission.
 __device__ void grid_emit(const GridModel& m, GPhoton& ph, const float* Ktab, uint32_t& pr, uint32_t& pc) {
-  ph.rng.init(((uint64_t)m.seed_hi << 32) | m.seed_lo, ph.pid, 2u);
+  Rng rng;
+  rng.init(((uint64_t)m.seed_hi << 32) | m.seed_lo, ph.pid, 2u);
+  ph.key = rng;
   const int64_t n = (int64_t)m.nx * m.ny * m.nz;
   const double total = m.cdf[n - 1];
-  const double R = (double)ph.rng.u(0) * total;
+  const double R = (double)rng.u(0) * total;
   int64_t lo = 0, hi = n - 1;  // smallest c with cdf[c] > R
   while (lo < hi) {
     const int64_t mid = (lo + hi) >> 1;
@@ -262,9 +264,9 @@ __device__ void grid_emit(const GridModel& m, GPhoton& ph, const float* Ktab, ui
   }
   const int64_t c = lo;
   const int ix = (int)(c % m.nx), iy = (int)((c / m.nx) % m.ny), iz = (int)(c / ((int64_t)m.nx * m.ny));
-  ph.p[0] = ix + (double)ph.rng.u(1);
-  ph.p[1] = iy + (double)ph.rng.u(2);
-  ph.p[2] = iz + (double)ph.rng.u(3);
+  ph.p[0] = ix + (double)rng.u(1);
+  ph.p[1] = iy + (double)rng.u(2);
+  ph.p[2] = iz + (double)rng.u(3);
 #pragma unroll
   for (int a = 0; a < 3; ++a) {  // a uniform of exactly 1.0 would land on the next cell's face
     const double lim = (a == 0 ? ix : a == 1 ? iy : iz) + 1.0;
@@ -272,8 +274,8 @@ __device__ void grid_emit(const GridModel& m, GPhoton& ph, const float* Ktab, ui
   }
   ph.o[0] = 0.0f; ph.o[1] = 0.0f; ph.o[2] = 0.0f;
   ph.safe = 0.0f;
-  ph.k = iso_dir(ph.rng.u(4), ph.rng.u(5));
-  const float R1 = ph.rng.u(6), R2 = ph.rng.u(7);
+  ph.k = iso_dir(rng.u(4), rng.u(5));
+  const float R1 = rng.u(6), R2 = rng.u(7);
   const float xe = sqrtf(-__logf(R1)) * cospif(2.0f * R2);
   const GridCell g = load_cell(m.cells, c);
   ph.X = __fmaf_rn(xe, g.vth, v_dot_k(g, ph.k));
@@ -311,10 +313,17 @@ __device__ __forceinline__ void peel_from_cell(const GridModel& m, const GPhoton
   const float v = (ax == 0) ? g.vx : (ax == 1) ? g.vy : g.vz;
   const float x = (Xp - v) * g.inv_vth;
   const float d = (ax == 0) ? ph.fhi[0] - ph.o[0] : (ax == 1) ? ph.fhi[1] - ph.o[1] : ph.fhi[2] - ph.o[2];
-  float tau = __fmaf_rn(g.kap0, peel_voigt(g.a, x, Ktab), g.kd) * fmaxf(d, 0.0f);
   ++pr;
   ++pc;
-  if (tau > m.tau_cut) return;  // blocked inside the current cell: no FP64, no gather
+  // Blocked inside the current cell: no FP64, no gather.  In a thick cell nearly every ray is,
+  // and a lower bound of H shows it without the table: H >= e^{-x^2} (1 - a^2 |1 - 2 x^2|) -
+  // 2 a / sqrt(pi) (K >= -1), and H >= a / (sqrt(pi) x^2) for |x| >= 2 (K >= 1 / (2 x^2)); the
+  // constants take 2% off for the approximate exponential and the table's own error.
+  const float x2 = x * x;
+  const float low = (x2 < 4.0f) ? __fmaf_rn(0.98f, exp_fast(-x2), -1.2f * g.a) : 0.55f * g.a * rcp_approx(x2);
+  if (g.a < 0.02f && g.kap0 * low * d > m.tau_cut) return;
+  float tau = __fmaf_rn(g.kap0, peel_voigt(g.a, x, Ktab), g.kd) * fmaxf(d, 0.0f);
+  if (tau > m.tau_cut) return;
   const double p[3] = {ph.p[0] + (double)ph.o[0], ph.p[1] + (double)ph.o[1], ph.p[2] + (double)ph.o[2]};
   walk(p, ax, Xp, w0, tau);
 }
@@ -331,10 +340,9 @@ __device__ __forceinline__ void peel_from_cell(const GridModel& m, const GPhoton
 // any FP64 arithmetic (the common case for photons trapped in optically thick cells).
 // Otherwise the cell walk runs from the current position (FP64, the bit-reproducible
 // contract of Dda) and re-establishes the cell frame at the interaction point.
-__device__ __forceinline__ int grid_move(const GridModel& m, GPhoton& ph, const float* Ktab, float& x_out,
-                                         float& kH_out) {
-  ph.rng.next_event(3u);
-  float tau_rem = -__logf(ph.rng.u(W_TAU));
+__device__ __forceinline__ int grid_move(const GridModel& m, GPhoton& ph, const float* Ktab, float tau_rem,
+                                         float& x_out, float& kH_out) {
+  ++ph.key.event;
   float x = 0.0f, kH = 0.0f;
   bool fast = false;
   if (ph.safe > 0.0f) {
@@ -390,22 +398,22 @@ __device__ __forceinline__ int grid_move(const GridModel& m, GPhoton& ph, const 
 }
 
 // The interaction channel at the site (Sec. 3.4): dust with probability kd / (kH + kd).
-__device__ __forceinline__ bool grid_dust_channel(const GPhoton& ph, float kH) {
+__device__ __forceinline__ bool grid_dust_channel(const GPhoton& ph, float kH, float R) {
   const GridCell& g = ph.gc;
-  return g.kd > 0.0f && ph.rng.u(W_CHANNEL) >= __fdividef(kH, kH + g.kd);
+  return g.kd > 0.0f && R >= __fdividef(kH, kH + g.kd);
 }
 // A dust interaction: absorbed with probability 1 - albedo (returns 2), else scattered by the
 // Henyey-Greenstein phase function (Eq. 8-9) with its peel-off (returns 0).
 template <class Walk>
-__device__ __forceinline__ int grid_dust(const GridModel& m, GPhoton& ph, const float* Ktab, uint32_t& pr,
-                                         uint32_t& pc, const Walk& walk) {
+__device__ __forceinline__ int grid_dust(const GridModel& m, GPhoton& ph, const EventWords& w, const float* Ktab,
+                                         uint32_t& pr, uint32_t& pc, const Walk& walk) {
   const GridCell& g = ph.gc;
   const float vv[3] = {g.vx, g.vy, g.vz};
   const float vk_in = v_dot_k(g, ph.k);
   bool scat;
   if (m.albedo <= 0.0f) scat = false;
   else if (m.albedo >= 1.0f) scat = true;
-  else scat = ph.rng.u(W_ALBEDO) < m.albedo;
+  else scat = w.albedo < m.albedo;
   if (!scat) return 2;
   if (m.peel) {
     const float kin[3] = {ph.k.x, ph.k.y, ph.k.z};
@@ -415,7 +423,7 @@ __device__ __forceinline__ int grid_dust(const GridModel& m, GPhoton& ph, const 
       peel_from_cell(m, ph, ax, Xp, P_hg(kin[ax], m.g_hg) * (0.5f / kPiF), Ktab, pr, pc, walk);
     }
   }
-  scatter_dust(m.g_hg, ph.k, ph.rng);
+  scatter_dust(m.g_hg, ph.k, w.Rm, w.cp, w.sp);
   ph.X += v_dot_k(g, ph.k) - vk_in;
   ++ph.ndust;
   return 0;
@@ -423,13 +431,13 @@ __device__ __forceinline__ int grid_dust(const GridModel& m, GPhoton& ph, const 
 // A resonant scattering at gas-frame frequency x (Eq. 5-7) with its peel-off.  Returns 3
 // if it reached the scattering cap, else 0.
 template <class Walk>
-__device__ __forceinline__ int grid_resonant(const GridModel& m, GPhoton& ph, float x, const float* Ktab,
-                                             uint32_t& pr, uint32_t& pc, const Walk& walk) {
+__device__ __forceinline__ int grid_resonant(const GridModel& m, GPhoton& ph, const EventWords& w, float x,
+                                             const float* Ktab, uint32_t& pr, uint32_t& pc, const Walk& walk) {
   const GridCell& g = ph.gc;
   const float vv[3] = {g.vx, g.vy, g.vz};
   const float kin[3] = {ph.k.x, ph.k.y, ph.k.z};
   AtomFrame af;
-  const float xo = scatter_resonant(x, g.a, m.phase, ph.k, ph.rng, ph.iters, &af);
+  const float xo = scatter_resonant(x, g.a, m.phase, ph.k, w, ph.key, ph.iters, &af);
   if (m.peel) {
     const float e1[3] = {af.e1.x, af.e1.y, af.e1.z}, e2[3] = {af.e2.x, af.e2.y, af.e2.z};
 #pragma unroll
@@ -450,21 +458,29 @@ __device__ __forceinline__ int grid_resonant(const GridModel& m, GPhoton& ph, fl
   return 0;
 }
 
-// The interaction half, from the words of the current event: channel, then dust or
-// resonant scattering, each with its peel-off (Sec. 3.4.1).  Returns 0 continue,
-// 2 absorbed, 3 capped.
-template <class Walk>
-__device__ __forceinline__ int grid_interact(const GridModel& m, GPhoton& ph, float x, float kH, const float* Ktab,
-                                             uint32_t& pr, uint32_t& pc, const Walk& walk) {
-  if (grid_dust_channel(ph, kH)) return grid_dust(m, ph, Ktab, pr, pc, walk);
-  return grid_resonant(m, ph, x, Ktab, pr, pc, walk);
+// One event from what it takes of its words: the move, then the interaction (channel, dust or
+// resonant scattering, each with its peel-off, Sec. 3.4.1).  Returns 0 continue, 1 escaped, 2
+// absorbed, 3 capped.
+__device__ __forceinline__ int grid_event(const GridModel& m, GPhoton& ph, const EventWords& w, const float* Ktab,
+                                          uint32_t& pr, uint32_t& pc) {
+  float x, kH;
+  if (grid_move(m, ph, Ktab, w.tau, x, kH)) return 1;
+  const WalkHere walk{m, Ktab, pc};
+  if (grid_dust_channel(ph, kH, w.channel)) return grid_dust(m, ph, w, Ktab, pr, pc, walk);
+  return grid_resonant(m, ph, w, x, Ktab, pr, pc, walk);
 }
 
-// One event; returns 0 continue, 1 escaped, 2 absorbed, 3 capped.
-__device__ int grid_event(const GridModel& m, GPhoton& ph, const float* Ktab, uint32_t& pr, uint32_t& pc) {
-  float x, kH;
-  if (grid_move(m, ph, Ktab, x, kH)) return 1;
-  return grid_interact(m, ph, x, kH, Ktab, pr, pc, WalkHere{m, Ktab, pc});
+// What event e of a packet takes from its words, formed by its own lane (event-based loop).
+__device__ __forceinline__ EventWords grid_words(const GridModel& m, const StreamKey& key, uint32_t e) {
+  Rng r;
+  r.k0 = key.k0; r.k1 = key.k1; r.p0 = key.p0; r.p1 = key.p1;
+  r.start_event(e, 3u);
+  EventWords w;
+  scatter_words(w, r, m.phase, 0.0f);
+  w.tau = -__logf(r.u(W_TAU));
+  w.channel = r.u(W_CHANNEL);
+  w.albedo = r.u(W_ALBEDO);
+  return w;
 }
 
 // ---- event-based loop: packets in device memory between its kernels -----------------
@@ -477,7 +493,7 @@ __device__ __forceinline__ void slot_save(const GridSlots& S, int64_t i, const G
   S.safe[i] = ph.safe;
   S.kx[i] = ph.k.x; S.ky[i] = ph.k.y; S.kz[i] = ph.k.z; S.X[i] = ph.X;
   S.nscat[i] = ph.nscat; S.ndust[i] = ph.ndust; S.iters[i] = ph.iters; S.steps[i] = ph.steps;
-  S.event[i] = ph.rng.event;
+  S.event[i] = ph.key.event;
   S.pid[i] = ph.pid;
 }
 // with_cell: re-read the cell record (always for the interaction half; for the move only
@@ -492,8 +508,8 @@ __device__ __forceinline__ void slot_load(const GridModel& m, const GridSlots& S
   ph.X = S.X[i];
   ph.nscat = S.nscat[i]; ph.ndust = S.ndust[i]; ph.iters = S.iters[i]; ph.steps = S.steps[i];
   ph.pid = S.pid[i];
-  ph.rng.keys(((uint64_t)m.seed_hi << 32) | m.seed_lo, ph.pid);
-  ph.rng.event = S.event[i];
+  ph.key.keys(((uint64_t)m.seed_hi << 32) | m.seed_lo, ph.pid);
+  ph.key.event = S.event[i];
   if (with_cell || ph.safe > 0.0f)
     ph.gc = load_cell(m.cells, cell_index(m, (int)floor(ph.p[0]), (int)floor(ph.p[1]), (int)floor(ph.p[2])));
 }
@@ -681,7 +697,7 @@ __global__ void __launch_bounds__(256) grid_run_kernel(GridModel m, WorkQueue q,
     do {
       fin = false;
       if (active) {
-        const int st = grid_event(m, ph, sK, t.pr, t.pc);
+        const int st = grid_event(m, ph, grid_words(m, ph.key, ph.key.event + 1u), sK, t.pr, t.pc);
         if (st) {
           grid_finish(m, ph, st, t);
           active = false;
@@ -736,11 +752,12 @@ __global__ void __launch_bounds__(256) grid_move_kernel(GridModel m, WorkQueue q
     }
     if (!live) continue;
     float x, kH;
-    int st = grid_move(m, ph, sK, x, kH);
+    const EventWords w = grid_words(m, ph.key, ph.key.event + 1u);
+    int st = grid_move(m, ph, sK, w.tau, x, kH);
     bool queued = false;
     if (st == 0) {
-      if (grid_dust_channel(ph, kH)) {
-        st = grid_dust(m, ph, sK, t.pr, t.pc, walk);
+      if (grid_dust_channel(ph, kH, w.channel)) {
+        st = grid_dust(m, ph, w, sK, t.pr, t.pc, walk);
       } else {
         queued = true;
         S.xs[i] = x;
@@ -784,8 +801,7 @@ __global__ void __launch_bounds__(256) grid_scatter_kernel(GridModel m, GridSlot
     const int64_t i = S.rq[j];
     GPhoton ph;
     slot_load(m, S, i, ph, true);
-    ph.rng.start_event(ph.rng.event, 3u);
-    const int st = grid_resonant(m, ph, S.xs[i], sK, t.pr, t.pc, walk);
+    const int st = grid_resonant(m, ph, grid_words(m, ph.key, ph.key.event), S.xs[i], sK, t.pr, t.pc, walk);
     if (st) {
       grid_finish(m, ph, st, t);
       --dlive;

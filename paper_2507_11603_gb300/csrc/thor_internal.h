@@ -127,9 +127,8 @@ struct Compact {  // every field defaults to off / empty
   // drained, a warp whose lanes are all done waits for a packet that a warp with several
   // live packets gives away, and runs it alone.
   PhotonRec* pool = nullptr;            // given-away packets (one entry per photon at most)
-  uint32_t* ready = nullptr;            // pool entry i written (1), set after the record
-  unsigned long long* share = nullptr;  // [0] entries reserved, [1] taken, [2] empty warps waiting,
-                                        // [3] photons finished, [4] a taken entry never became ready
+  uint32_t* ready = nullptr;            // pool entry i: 1 once written, 2 once its ticket gave up
+  unsigned long long* share = nullptr;  // [0] entries reserved, [1] tickets taken, [3] photons finished
   unsigned long long n_total = 0;       // photons of the run
 };
 

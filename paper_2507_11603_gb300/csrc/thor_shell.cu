@@ -24,6 +24,7 @@ constexpr unsigned kFull = 0xffffffffu;
 // position then holds the progress).
 constexpr int kFlySteps = 128;
 constexpr float kFlyNone = -1.0f, kFlyBall = -2.0f;
+constexpr float kSafePending = -1.0f;  // Photon::safe: not formed yet (power laws; the offset is zero)
 constexpr uint32_t kLongLived = 1u << 14;
 constexpr uint32_t kPriBudget = 16;  // served rounds: budget multiple of a priority warp (one packet)  // served rounds: packets past this many events run one per warp
 
@@ -37,6 +38,8 @@ struct Photon {
   int region;  // 1 = inside the empty cavity
   uint32_t nscat, ndust, iters, steps;
   float fly, fly_tau;    // an event interrupted in flight (kFly*): where, and the depth left
+  // power law: position in FP32, r, 1 / r, density and speed there (pl_ir = 0: not formed)
+  float qx, qy, qz, pl_r, pl_ir, pl_nr, pl_v;
   float X0;              // emitted lab frequency
   float col_hi, col_lo;  // HI column traversed (power-law shells), two-level FP32 sum
   StreamKey key;  // key.event: last completed event
@@ -78,6 +81,7 @@ __device__ __forceinline__ void shell_emit(const ShellModel& m, Photon& ph) {
   ph.safe = (float)m.R_out;
   ph.nscat = 0; ph.ndust = 0; ph.iters = 0; ph.steps = 0;
   ph.fly = kFlyNone; ph.fly_tau = 0.0f;
+  ph.pl_ir = 0.0f;
 }
 
 // Move by s along k inside the safety ball: FP32 offset only.  The moves since the last
@@ -158,6 +162,43 @@ __device__ __forceinline__ StartStep start_step(const ShellModel& m, float H, fl
 }
 __device__ __forceinline__ bool dust_channel(const ShellModel& m, float kH, float R) {
   return __fmul_rn(R, __fadd_rn(kH, m.kapd)) >= kH;
+}
+
+// Free flight: sub-steps in the wing, four at a time while none of them ends the flight (the
+// caller takes that one).  Their opacities do not depend on one another (x drifts
+// monotonically), so they are formed side by side -- one at a time a flight is a chain of some
+// 100 dependent instructions per sub-step -- and only depth and column are summed in order.
+// (Out of line it took 14.0 instead of 11.7 ms on the Mg II sphere.)
+struct FlyOut {
+  float s, tau, col_hi, col_lo;
+  uint32_t n;  // sub-steps done
+};
+static __device__ __forceinline__ FlyOut fly_wing(float kap0, float kapd, float a, float gam, float x0, float ds, float s,
+                                               float bound, float tau, int most) {
+  FlyOut o{s, tau, 0.0f, 0.0f, 0u};
+  const float g = gam * 0.5f;
+  while ((int)o.n < most && o.s + 4.25f * ds <= bound) {
+    float e[5], kp[4];
+    e[0] = o.s;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) e[i + 1] = e[i] + ds;
+    const float xa = __fmaf_rn(-g, e[0] + e[1], x0), xb = __fmaf_rn(-g, e[3] + e[4], x0);
+    if (!(fminf(xa, xb) >= 6.0f || fmaxf(xa, xb) <= -6.0f)) break;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float x = __fmaf_rn(-g, e[i] + e[i + 1], x0);
+      kp[i] = __fmaf_rn(kap0, voigt_wing<false>(a, x * x), kapd);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float dt = __fmul_rn(kp[i], e[i + 1] - e[i]);
+      if (dt >= o.tau) return o;
+      o.tau = __fsub_rn(o.tau, dt);
+      o.s = e[i + 1];
+      ++o.n;
+    }
+  }
+  return o;
 }
 
 // One event.  Returns 0 = continues, 1 = escaped, 2 = absorbed by dust, 3 = capped, -1 =
@@ -291,41 +332,14 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
         }
         tau_rem -= dtau;
         s = s1;
-        // Free flight: sub-steps in the wing, four at a time.  Their opacities do not depend
-        // on one another (x drifts monotonically), so they are formed side by side and only
-        // the depth is summed in order.
-        while (turn_steps > 0 && s + 4.25f * m.ds_core <= (have ? Sf : seg.lower)) {
-          turn_steps -= 4;
-          float e[5], kp[4];
-          e[0] = s;
-#pragma unroll
-          for (int i = 0; i < 4; ++i) e[i + 1] = e[i] + m.ds_core;
-          const float xa = x0 - m.gam * 0.5f * (e[0] + e[1]), xb = x0 - m.gam * 0.5f * (e[3] + e[4]);
-          if (!(fminf(xa, xb) >= 6.0f || fmaxf(xa, xb) <= -6.0f)) break;
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float ax = fabsf(x0 - m.gam * 0.5f * (e[i] + e[i + 1]));
-            kp[i] = __fmaf_rn(m.kap0, voigt_wing<false>(m.a, ax * ax), m.kapd);
-          }
-          bool cross = false;
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float dt = kp[i] * (e[i + 1] - e[i]);
-            if (!cross) {
-              ++ph.steps;
-              if (dt >= tau_rem) {
-                cross = true;
-                s_star = e[i] + tau_rem / kp[i];
-                if (have) s_star = fminf(s_star, Sf);
-              } else {
-                tau_rem -= dt;
-                s = e[i + 1];
-              }
-            }
-          }
-          if (cross) break;
+        const float bound = have ? Sf : seg.lower;
+        if (turn_steps > 0 && s + 4.25f * m.ds_core <= bound && fabsf(xm) >= 6.0f) {
+          const FlyOut f = fly_wing(m.kap0, m.kapd, m.a, m.gam, x0, m.ds_core, s, bound, tau_rem, turn_steps);
+          s = f.s;
+          tau_rem = f.tau;
+          ph.steps += f.n;
+          turn_steps -= (int)f.n + 1;
         }
-        if (s_star >= 0.0f) break;
       }
     }
     if (s_star >= 0.0f) {
@@ -397,57 +411,15 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
 // expanding shell of 1e5 photons at N_HI = 1e20 3.29 s (5.35 s).  The general events run for
 // all the packets that wait for one, at most once per `depth` core events: a general event
 // costs several core events, and one lane in sixty needs one at any time.
-constexpr int kChainSlots = 128;      // events per warp and round
+constexpr int kChainSlots = kWordSlots;  // events per warp and round
 constexpr uint32_t kChainDepth = 32;  // ... and per packet, in warps with few packets
 constexpr uint32_t kCrowdDepth = 16;  // ... and per packet, in the others (kept until a general event runs)
+constexpr uint32_t kFirstDepth = 4;   // ... at first: doubled where a round runs full, halved where it mostly does not
 constexpr uint32_t kVoteEvents = 4;   // core events between two votes on whether any packet goes on
-struct WordBuf {                      // one per warp
-  float4 a[kChainSlots];              // tau, R1, R2, R3
-  float4 b[kChainSlots];              // mu, st, cos phi, sin phi
-  float4 c[kChainSlots];              // u1, u2, v1, v2
-  float4 d[kChainSlots];              // Rm, channel, mixed, albedo
-  uint4 own[32];                      // photon id, last completed event, flags (owners in lane order)
-  uint4 key[32];                      // stream key, phase function, core-skipping threshold
-};
-// Where a lane's slots lie: slot (cur P + rank) holds its next event while cur < D.
-struct WordPos {
-  int P = 1, D = 0, rank = 0, cur = 0;
-};
-
-// Forms the next D events' words of every packet in `mine` lanes, one slot per lane at a
-// time (P D <= kChainSlots).  Called by all 32 lanes, converged.
 __device__ __forceinline__ void form_words(const ShellModel& m, const Photon& ph, WordBuf& wb, bool mine, int D,
                                            WordPos& at) {
-  const int lane = (int)(threadIdx.x & 31u);
-  const unsigned owners = __ballot_sync(kFull, mine);
-  const int P = __popc(owners);
-  at.P = P; at.D = mine ? D : 0; at.cur = 0;
-  at.rank = mine ? __popc(owners & ((1u << lane) - 1u)) : 0;
-  if (mine) {
-    wb.own[at.rank] = make_uint4(ph.key.p0, ph.key.p1, ph.key.event, (needs_block2(m) ? 1u : 0u) | (m.profile ? 2u : 0u));
-    wb.key[at.rank] = make_uint4(ph.key.k0, ph.key.k1, (uint32_t)m.phase, __float_as_uint(m.xcrit));
-  }
-  __syncwarp();
-  for (int s = lane; s < P * D; s += 32) {  // slot d P + r: event d of the owner of rank r
-    const int d = s / P, r = s - d * P;
-    const uint4 own = wb.own[r], key = wb.key[r];
-    Rng q;
-    q.k0 = key.x; q.k1 = key.y; q.p0 = own.x; q.p1 = own.y;
-    q.v[8] = q.v[9] = q.v[10] = 0u;  // not drawn: not used
-    q.start_event(own.z + 1u + (uint32_t)d, (own.w & 1u) ? 3u : 2u);
-    EventWords w;
-    scatter_words(w, q, (int)key.z, __uint_as_float(key.w));
-    const float t = q.u(W_TAU);
-    wb.a[s] = make_float4((own.w & 2u) ? -__logf(t) : -ln_fast(t), w.R1, w.R2, w.R3);
-    wb.b[s] = make_float4(w.mu, w.st, w.cp, w.sp);
-    wb.c[s] = make_float4(w.u1, w.u2, w.v1, w.v2);
-    wb.d[s] = make_float4(w.Rm, q.u(W_CHANNEL), w.mixed, q.u(W_ALBEDO));
-  }
-  __syncwarp();
-}
-__device__ __forceinline__ EventWords read_words(const WordBuf& wb, int s) {
-  const float4 a = wb.a[s], b = wb.b[s], c = wb.c[s], d = wb.d[s];
-  return EventWords{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w, d.x, d.y, d.z, d.w};
+  form_words(wb, ph.key, (needs_block2(m) ? kWordBlock2 : 0u) | (m.profile ? kWordLog : 0u), m.phase, m.xcrit, mine, D,
+             at);
 }
 
 // Whether the packet's next event may be of the core kind (the cheap part of the test).
@@ -461,7 +433,7 @@ __device__ __forceinline__ bool chain_kind(const ShellModel& m, const Photon& ph
 __device__ __forceinline__ bool chain_event(const ShellModel& m, Photon& ph, const float4& wa, const float4& wb,
                                             const float4& wc, float channel, uint32_t e, bool go, uint32_t& second) {
   // ---- the frequency chain: rate at the start, crossing, gas-frame frequency at the site
-  const float x0 = go ? ph.x : 0.0f;  // lanes without a packet in the round take the owners' branches
+  const float x0 = ph.x;  // (lanes that are not going evaluate what they have, and commit nothing)
   const StartStep st0 = start_step(m, voigt_core_poly(m.a, x0), wa.x);
   const float s0 = st0.s;
   const bool in_ball = (m.gam == 0.0f) ? (s0 <= ph.safe) : (ph.safe >= m.ds_core && s0 <= 0.0625f * m.ds_core);
@@ -472,17 +444,17 @@ __device__ __forceinline__ bool chain_event(const ShellModel& m, Photon& ph, con
   const float xr = fabsf(xs);
   const float u0 = u0_core(xr, m.a);
   const float q = upar_q(xr, m.a);
-  // w1 = atan2(a, x - u0) as sample_upar forms it: the q form where u0 > 0, else (u0 = 0,
-  // within ~0.04 of line centre) the series in a / x
-  const bool split = u0 > 0.0f;
-  const float w1 = split ? atan_small(q) : atan2_series(m.a, xr);
+  // w1 = atan2(a, x - u0) as sample_upar forms it: from q where u0 > 0 and q is small, else the
+  // series in a / x, else (within 20 a of line centre, and in cold gas) atan2f itself
+  const bool split = u0 > 0.0f && q <= 0.05f, far = m.a <= 0.05f * (xr - u0);
+  float w1 = split ? atan_small(q) : atan2_series(m.a, xr - u0);
+  if (go && !split && !far) w1 = atan2f(m.a, xr - u0);
   const float u02 = __fmul_rn(u0, u0);
   const float mass = envelope_mass(w1, exp_fast(-u02));
   const float w1p = __fmul_rn(w1, 1.0f / kPiF);
   float u;
   bool accepted = upar_trial(xr, m.a, w1, w1p, mass, u02, wa.y, wa.z, wa.w, u);
-  const bool kind = go && fabsf(x0) <= THOR_VCORE_X && in_ball && !dust && xr <= 2.0f &&
-                    (split ? q <= 0.05f : m.a <= 0.05f * xr);
+  const bool kind = go && fabsf(x0) <= THOR_VCORE_X && in_ball && !dust && xr <= 2.0f;
   if (!accepted && kind) {  // rare: the second trial, from block 3 of the event as sample_upar takes it
     StreamKey r = ph.key;
     r.event = e;
@@ -515,7 +487,7 @@ __device__ __forceinline__ bool chain_event(const ShellModel& m, Photon& ph, con
 // core kind, or one scattering short of the cap (the general event runs that one, from slot
 // at.cur).  Returns the events done.
 __device__ __forceinline__ uint32_t chain_round(const ShellModel& m, Photon& ph, WordBuf& wb, bool mine, int D,
-                                                WordPos& at, bool& stuck) {
+                                                WordPos& at, bool& stuck, int first_vote) {
   form_words(m, ph, wb, mine, D, at);
   const uint32_t left = m.max_scat ? (m.max_scat > ph.nscat + 1u ? m.max_scat - ph.nscat - 1u : 0u) : (uint32_t)D;
   const int lim = (int)min(left, (uint32_t)D);
@@ -523,7 +495,7 @@ __device__ __forceinline__ uint32_t chain_round(const ShellModel& m, Photon& ph,
   uint32_t n = 0, second = 0;
   int d = 0;
   while (d < D) {
-    const int end = min(D, d + (int)kVoteEvents);
+    const int end = min(D, d + (d ? (int)kVoteEvents : first_vote));
 #pragma unroll 1
     for (; d < end; ++d) {
       const int s = d * at.P + at.rank;
@@ -543,26 +515,37 @@ __device__ __forceinline__ uint32_t chain_round(const ShellModel& m, Photon& ph,
   return n;
 }
 
+// The depth of a warp's next round from that of the last: gas that is not thick enough for core
+// events to follow one another (a crossing beyond ds/16 ends a round) would form slots and
+// evaluate events for nothing.
+__device__ __forceinline__ uint32_t next_depth(uint32_t depth, uint32_t most, unsigned tried, unsigned full) {
+  if (2 * __popc(full) >= __popc(tried)) return min(2u * depth, most);
+  return 8 * __popc(full) < __popc(tried) ? max(depth / 2u, 1u) : depth;
+}
+
 // Core events of a warp's packets until `depth` of them ran or the packet needs a general
 // event (`general` then stays set).  Several rounds where the slots of one do not reach
 // (P > kChainSlots / depth): the general events, which run for a few lanes at a time, come
 // once per `depth` events.  Returns this lane's events; `at`: the slots of its last round, if
 // no other round has overwritten them.
 __device__ __forceinline__ uint32_t core_events(const ShellModel& m, Photon& ph, WordBuf& wb, bool active,
-                                                uint32_t depth, bool& general, WordPos& at) {
+                                                uint32_t& depth_io, uint32_t most, bool& general, WordPos& at) {
   uint32_t n = 0;
+  const uint32_t depth = min(depth_io, most);
   bool go = active && chain_kind(m, ph);
+  const unsigned tried = __ballot_sync(kFull, go);
   for (uint32_t d = 0; d < depth; ) {
-    const int P = __popc(__ballot_sync(kFull, go));
+    const unsigned P = __popc(__ballot_sync(kFull, go));
     if (P == 0) break;
-    const uint32_t D = min(depth - d, (uint32_t)(kChainSlots / P));
+    // (one pass of the 32 lanes forms 32 slots anyway, and general events use what is left)
+    const uint32_t D = min(max(depth - d, min(32u / P, most)), (uint32_t)(kChainSlots / P));
     bool stuck = false;
-    __syncwarp();  // the round before is read
-    n += chain_round(m, ph, wb, go, (int)D, at, stuck);
+    n += chain_round(m, ph, wb, go, (int)D, at, stuck, (int)min(depth, kVoteEvents));
     go = go && !stuck;
     d += D;
   }
   general = active && !go;
+  if (tried) depth_io = next_depth(depth, most, tried, __ballot_sync(kFull, go));
   return n;
 }
 
@@ -578,20 +561,36 @@ __device__ __forceinline__ void general_words(const ShellModel& m, const Photon&
 // ---- power-law shells (Sec. 5.1) ---------------------------------------------------
 // Gas state at a point q (FP32, |q| <= 1) for direction k: radius, r_hat . k, density
 // relative to r = 1 and outflow speed.
-struct PLState { float r, mur, nr, v; };
+struct PLState { float r, mur, nr, v, ir; };
 __device__ __forceinline__ PLState pl_state(const ShellModel& m, float qx, float qy, float qz, float3 k) {
   const float r2 = __fmaf_rn(qx, qx, __fmaf_rn(qy, qy, qz * qz));
-  const float ir = rsqrtf(r2);
   PLState st;
-  st.r = r2 * ir;
-  st.mur = __fmaf_rn(qx, k.x, __fmaf_rn(qy, k.y, qz * k.z)) * ir;
+  st.ir = rsqrtf(r2);
+  st.r = r2 * st.ir;
+  st.mur = __fmaf_rn(qx, k.x, __fmaf_rn(qy, k.y, qz * k.z)) * st.ir;
   const float lr = __log2f(st.r);
   st.nr = ex2_approx(m.ar * lr);
   st.v = m.v1 * ex2_approx(m.av * lr);
   return st;
 }
-__device__ __forceinline__ void col_add(Photon& ph, float d) {
-  ph.col_lo += d;
+// The same at the packet's position, which a scattering does not change: from the event
+// before, where it was formed there (only the direction is new; the FP64 anchor's conversions
+// are saved too).
+__device__ __forceinline__ PLState pl_here(const ShellModel& m, Photon& ph) {
+  if (ph.pl_ir == 0.0f) {
+    ph.qx = (float)ph.px + ph.ox; ph.qy = (float)ph.py + ph.oy; ph.qz = (float)ph.pz + ph.oz;
+    return pl_state(m, ph.qx, ph.qy, ph.qz, ph.k);
+  }
+  PLState st;
+  st.ir = ph.pl_ir;
+  st.r = ph.pl_r;
+  st.mur = __fmaf_rn(ph.qx, ph.k.x, __fmaf_rn(ph.qy, ph.k.y, ph.qz * ph.k.z)) * st.ir;
+  st.nr = ph.pl_nr;
+  st.v = ph.pl_v;
+  return st;
+}
+__device__ __forceinline__ void col_add(Photon& ph, float n, float d) {  // n d
+  ph.col_lo = __fmaf_rn(n, d, ph.col_lo);
   if (ph.col_lo >= 0.00390625f) { ph.col_hi += ph.col_lo; ph.col_lo = 0.0f; }
 }
 
@@ -609,12 +608,62 @@ __device__ __forceinline__ float from_line2(const ShellModel& m, float X2) {
   return __fmaf_rn(-__fdividef(m.eps2, 1.0f + m.eps2), kCkms + X2, X2);
 }
 
-__device__ int shell_event_pl(const ShellModel& m, Photon& ph, const float* __restrict__ Ktab, const EventWords& w) {
+// X - v mu_r, the product rounded on its own (`apart`) or not: part of a history's bits.
+__device__ __forceinline__ float x_offset(float X, const PLState& st, bool apart) {
+  return apart ? __fsub_rn(X, __fmul_rn(st.v, st.mur)) : __fmaf_rn(-st.v, st.mur, X);
+}
+// fly_wing on a power-law shell, through the wings of its one or two lines, with the column.
+static __device__ __forceinline__ FlyOut fly_power(const ShellModel* __restrict__ mp, float p0x, float p0y, float p0z,
+                                                float3 k, float X, float s, float bound, float tau, float col_hi,
+                                                float col_lo, int most) {
+  const ShellModel& m = *mp;
+  FlyOut o{s, tau, col_hi, col_lo, 0u};
+  const float ds = m.ds_core;
+  const bool two = m.n_lines == 2;
+  while ((int)o.n < most && o.s + 4.25f * ds <= bound) {
+    float e[5], kap[4], nr[4];
+    e[0] = o.s;
+    bool wing = true;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      e[i + 1] = e[i] + ds;
+      const float sm = 0.5f * (e[i] + e[i + 1]);
+      const PLState st = pl_state(m, __fmaf_rn(sm, k.x, p0x), __fmaf_rn(sm, k.y, p0y), __fmaf_rn(sm, k.z, p0z), k);
+      nr[i] = st.nr;
+      const float vk = __fmul_rn(st.v, st.mur);  // rounded as the caller's sub-step rounds it
+      const float ax = fabsf(__fmul_rn(two ? __fsub_rn(X, vk) : __fmaf_rn(-st.v, st.mur, X), m.inv_vth));
+      wing = wing && ax >= 6.0f;
+      float H2 = 0.0f;
+      if (two) {
+        const float ax2 = fabsf(__fmul_rn(__fsub_rn(to_line2(m, X), vk), m.inv_vth));
+        H2 = voigt_wing<false>(m.a2, ax2 * ax2);
+        wing = wing && ax2 >= 6.0f;
+      }
+      kap[i] = __fmul_rn(st.nr, __fmaf_rn(m.kapn, voigt_wing<false>(m.a, ax * ax), __fmaf_rn(m.kapn2, H2, m.kapdn)));
+    }
+    if (!wing) return o;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float d = e[i + 1] - e[i], dt = __fmul_rn(kap[i], d);
+      if (dt >= o.tau) return o;
+      o.col_lo = __fmaf_rn(__fmul_rn(nr[i], m.invF), d, o.col_lo);
+      if (o.col_lo >= 0.00390625f) { o.col_hi += o.col_lo; o.col_lo = 0.0f; }
+      o.tau = __fsub_rn(o.tau, dt);
+      o.s = e[i + 1];
+      ++o.n;
+    }
+  }
+  return o;
+}
+
+__device__ int shell_event_pl(const ShellModel& m, const ShellModel* mp, Photon& ph, const float* __restrict__ Ktab,
+                              const EventWords& w) {
   const bool resumed = ph.fly != kFlyNone;
   float tau_rem = resumed ? ph.fly_tau : w.tau;
   float s_seg = ph.fly;
   ph.fly = kFlyNone;
   int turn_steps = kFlySteps;
+  const bool two = m.n_lines == 2;
   float kH, kH2 = 0.0f, kD;
   PLState site;
   for (;;) {
@@ -627,53 +676,60 @@ __device__ int shell_event_pl(const ShellModel& m, Photon& ph, const float* __re
       ph.px += s * kx; ph.py += s * ky; ph.pz += s * kz;
       ph.region = 0;
       ph.safe = 0.0f;
+      ph.pl_ir = 0.0f;
     }
+    float lower = 0.0f;  // of the distance to any boundary
     if (!(s_seg >= 0.0f)) {  // short step with the rate at the current point
-      const PLState st = pl_state(m, (float)ph.px + ph.ox, (float)ph.py + ph.oy, (float)ph.pz + ph.oz, ph.k);
-      const float x = (ph.X - st.v * st.mur) * m.inv_vth;
+      const PLState st = pl_here(m, ph);
+      lower = fminf(1.0f - st.r, st.r - (float)m.R_in) - 1e-6f;
+      const float x = __fmul_rn(x_offset(ph.X, st, true), m.inv_vth);
       const float H = voigt<false>(m.a, x, Ktab);
-      const float H2 = (m.n_lines == 2) ? voigt<false>(m.a2, (to_line2(m, ph.X) - st.v * st.mur) * m.inv_vth, Ktab)
+      const float H2 = (m.n_lines == 2) ? voigt<false>(m.a2, __fmul_rn(x_offset(to_line2(m, ph.X), st, true), m.inv_vth), Ktab)
                                          : 0.0f;
       const float kap = st.nr * __fmaf_rn(m.kapn, H, __fmaf_rn(m.kapn2, H2, m.kapdn));
       const float s0 = __fdividef(tau_rem, kap);
       ++ph.steps;
-      if (s0 <= ph.safe && s0 <= 0.0625f * m.ds_core) {
+      const bool is_short = s0 <= 0.0625f * m.ds_core;
+      // the safety distance (an FP64 square root) is formed where it decides
+      if (is_short && ph.safe == kSafePending) ph.safe = safe_distance(m, ph);
+      if (is_short && s0 <= ph.safe) {
         advance(ph, s0);
         ph.safe = __fmaf_rd(-s0, 1.000001f, ph.safe);
-        col_add(ph, st.nr * m.invF * s0);
+        col_add(ph, st.nr * m.invF, s0);
         kH = m.kapn * st.nr * H;
         kH2 = m.kapn2 * st.nr * H2;
         kD = m.kapdn * st.nr;
-        site = pl_state(m, (float)ph.px + ph.ox, (float)ph.py + ph.oy, (float)ph.pz + ph.oz, ph.k);
+        ph.qx = (float)ph.px + ph.ox; ph.qy = (float)ph.py + ph.oy; ph.qz = (float)ph.pz + ph.oz;
+        site = pl_state(m, ph.qx, ph.qy, ph.qz, ph.k);
         break;
       }
     }
     // general path: sub-steps of <= ds to the crossing or the next boundary, its distance
     // exact (FP64) where it counts
-    anchor(ph);
+    if (ph.ox != 0.0f || ph.oy != 0.0f || ph.oz != 0.0f || ph.pl_ir == 0.0f) {
+      anchor(ph);
+      ph.qx = (float)ph.px; ph.qy = (float)ph.py; ph.qz = (float)ph.pz;
+    }
     const double kx = ph.k.x, ky = ph.k.y, kz = ph.k.z;
-    const double b = ph.px * kx + ph.py * ky + ph.pz * kz;
-    const double pp = ph.px * ph.px + ph.py * ph.py + ph.pz * ph.pz;
-    const ShellSegment seg(m, b, pp);
     double S = 0.0;
     float Sf = 0.0f;
     int next = 1;
     bool have = false;
-    const float p0x = (float)ph.px, p0y = (float)ph.py, p0z = (float)ph.pz;
+    const float p0x = ph.qx, p0y = ph.qy, p0z = ph.qz;
     float s = fmaxf(s_seg, 0.0f), s_star = -1.0f;
     s_seg = kFlyNone;
     // one sub-step of opacity kap, density nr, [s, s1]: true where the crossing lies in it
     auto sub_step = [&](float s1, float kap, float nr) {
-      const float dtau = kap * (s1 - s);
+      const float dtau = __fmul_rn(kap, s1 - s);
       ++ph.steps;
       if (dtau >= tau_rem) {
         s_star = s + __fdividef(tau_rem, kap);
         if (have) s_star = fminf(s_star, Sf);
-        col_add(ph, nr * m.invF * (s_star - s));
+        col_add(ph, nr * m.invF, s_star - s);
         return true;
       }
-      col_add(ph, nr * m.invF * (s1 - s));
-      tau_rem -= dtau;
+      col_add(ph, nr * m.invF, s1 - s);
+      tau_rem = __fsub_rn(tau_rem, dtau);
       s = s1;
       return false;
     };
@@ -684,24 +740,31 @@ __device__ int shell_event_pl(const ShellModel& m, Photon& ph, const float* __re
       }
       --turn_steps;
       float s1 = s + m.ds_core;
-      if (!have && !(s1 <= seg.lower)) {
-        S = seg.exact(m, b, pp, next);
-        Sf = (float)S;
-        have = true;
+      if (!have && !(s1 <= lower)) {  // the bound from the radius alone, then along the ray, then exact
+        const double b = ph.px * kx + ph.py * ky + ph.pz * kz;
+        const double pp = ph.px * ph.px + ph.py * ph.py + ph.pz * ph.pz;
+        lower = ShellSegment(m, b, pp).lower;
+        if (!(s1 <= lower)) {
+          S = ShellSegment::exact(m, b, pp, next);
+          Sf = (float)S;
+          have = true;
+        }
       }
       if (have) {
         if (!(s < Sf)) break;
         s1 = fminf(Sf, s1);
       }
+      bool in_wing;
       {
         const float sm = 0.5f * (s + s1);
         const PLState st = pl_state(m, __fmaf_rn(sm, ph.k.x, p0x), __fmaf_rn(sm, ph.k.y, p0y),
                                     __fmaf_rn(sm, ph.k.z, p0z), ph.k);
-        const float x = (ph.X - st.v * st.mur) * m.inv_vth;
+        const float x = __fmul_rn(x_offset(ph.X, st, two), m.inv_vth);
         const float H = voigt<false>(m.a, x, Ktab);
-        const float H2 = (m.n_lines == 2) ? voigt<false>(m.a2, (to_line2(m, ph.X) - st.v * st.mur) * m.inv_vth, Ktab)
+        const float H2 = (m.n_lines == 2) ? voigt<false>(m.a2, __fmul_rn(x_offset(to_line2(m, ph.X), st, true), m.inv_vth), Ktab)
                                            : 0.0f;
         const float kap = st.nr * __fmaf_rn(m.kapn, H, __fmaf_rn(m.kapn2, H2, m.kapdn));
+        in_wing = fabsf(x) >= 6.0f;
         if (sub_step(s1, kap, st.nr)) {
           kH = m.kapn * st.nr * H;
           kH2 = m.kapn2 * st.nr * H2;
@@ -709,53 +772,23 @@ __device__ int shell_event_pl(const ShellModel& m, Photon& ph, const float* __re
           break;
         }
       }
-      // Free flight: four sub-steps at a time while all of them lie in the lines' wings.  Their
-      // opacities do not depend on one another, so they are formed side by side (a photon's
-      // flight is a chain of some 100 dependent instructions per sub-step otherwise); depth
-      // and column are summed in order.
-      bool cross = false;
-      while (turn_steps > 0 && s + 4.25f * m.ds_core <= (have ? Sf : seg.lower)) {
-        turn_steps -= 4;
-        float e[5], H[4], H2[4], nr[4];
-        e[0] = s;
-        bool wing = true;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          e[i + 1] = e[i] + m.ds_core;
-          const float sm = 0.5f * (e[i] + e[i + 1]);
-          const PLState st = pl_state(m, __fmaf_rn(sm, ph.k.x, p0x), __fmaf_rn(sm, ph.k.y, p0y),
-                                      __fmaf_rn(sm, ph.k.z, p0z), ph.k);
-          nr[i] = st.nr;
-          const float ax = fabsf((ph.X - st.v * st.mur) * m.inv_vth);
-          H[i] = voigt_wing<false>(m.a, ax * ax);
-          wing = wing && ax >= 6.0f;
-          H2[i] = 0.0f;
-          if (m.n_lines == 2) {
-            const float ax2 = fabsf((to_line2(m, ph.X) - st.v * st.mur) * m.inv_vth);
-            H2[i] = voigt_wing<false>(m.a2, ax2 * ax2);
-            wing = wing && ax2 >= 6.0f;
-          }
-        }
-        if (!wing) break;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float kap = nr[i] * __fmaf_rn(m.kapn, H[i], __fmaf_rn(m.kapn2, H2[i], m.kapdn));
-          if (!cross && sub_step(e[i + 1], kap, nr[i])) {
-            cross = true;
-            kH = m.kapn * nr[i] * H[i];
-            kH2 = m.kapn2 * nr[i] * H2[i];
-            kD = m.kapdn * nr[i];
-          }
-        }
-        if (cross) break;
+      const float bound = have ? Sf : lower;
+      if (in_wing && turn_steps > 0 && s + 4.25f * m.ds_core <= bound) {
+        const FlyOut f = fly_power(mp, p0x, p0y, p0z, ph.k, ph.X, s, bound, tau_rem, ph.col_hi, ph.col_lo, turn_steps);
+        s = f.s;
+        tau_rem = f.tau;
+        ph.col_hi = f.col_hi;
+        ph.col_lo = f.col_lo;
+        ph.steps += f.n;
+        turn_steps -= (int)f.n + 1;
       }
-      if (cross) break;
     }
     if (s_star >= 0.0f) {
       const double sd = s_star;
       ph.px += sd * kx; ph.py += sd * ky; ph.pz += sd * kz;
-      ph.safe = safe_distance(m, ph);
-      site = pl_state(m, (float)ph.px, (float)ph.py, (float)ph.pz, ph.k);
+      ph.safe = kSafePending;
+      ph.qx = (float)ph.px; ph.qy = (float)ph.py; ph.qz = (float)ph.pz;
+      site = pl_state(m, ph.qx, ph.qy, ph.qz, ph.k);
       break;
     }
     ph.px += S * kx; ph.py += S * ky; ph.pz += S * kz;
@@ -763,6 +796,7 @@ __device__ int shell_event_pl(const ShellModel& m, Photon& ph, const float* __re
     ph.region = 1;
   }
   ++ph.key.event;
+  ph.pl_r = site.r; ph.pl_ir = site.ir; ph.pl_nr = site.nr; ph.pl_v = site.v;
   // Interaction (Sec. 3.4): transition 1, transition 2 or dust in proportion to their
   // opacities (one uniform); dust absorbs.
   int ch = 0;
@@ -771,20 +805,19 @@ __device__ int shell_event_pl(const ShellModel& m, Photon& ph, const float* __re
     ch = (u < __fdividef(kH, kt)) ? 0 : ((u < __fdividef(kH + kH2, kt)) ? 1 : 2);
   }
   if (ch == 2) return 2;
-  const float qx = (float)ph.px + ph.ox, qy = (float)ph.py + ph.oy, qz = (float)ph.pz + ph.oz;
   float xo;
   if (ch == 0) {
-    xo = scatter_resonant((ph.X - site.v * site.mur) * m.inv_vth, m.a, m.phase, ph.k, w, ph.key, ph.iters, nullptr,
+    xo = scatter_resonant(__fmul_rn(x_offset(ph.X, site, false), m.inv_vth), m.a, m.phase, ph.k, w, ph.key, ph.iters, nullptr,
                           m.xcrit);
   } else {  // second transition: J = 1/2 upper level, isotropic
     EventWords wi = w;
     wi.mu = __fmaf_rn(2.0f, w.Rm, -1.0f);
     wi.st = sqrt_approx(fmaxf(0.0f, __fmaf_rn(-wi.mu, wi.mu, 1.0f)));
-    xo = scatter_resonant((to_line2(m, ph.X) - site.v * site.mur) * m.inv_vth, m.a2, PH_ISO, ph.k, wi, ph.key,
+    xo = scatter_resonant(__fmul_rn(x_offset(to_line2(m, ph.X), site, false), m.inv_vth), m.a2, PH_ISO, ph.k, wi, ph.key,
                           ph.iters, nullptr, 0.0f);
   }
   // back to the lab frame with the new direction: X = x v_th + v(r) r_hat . k_out
-  const float mur = __fmaf_rn(qx, ph.k.x, __fmaf_rn(qy, ph.k.y, qz * ph.k.z)) / site.r;
+  const float mur = __fmaf_rn(ph.qx, ph.k.x, __fmaf_rn(ph.qy, ph.k.y, ph.qz * ph.k.z)) / site.r;
   const float Xl = __fmaf_rn(xo, m.vth, site.v * mur);
   ph.X = (ch == 0) ? Xl : from_line2(m, Xl);
   ++ph.nscat;
@@ -862,6 +895,7 @@ __device__ __forceinline__ void load_rec(const ShellModel& m, const PhotonRec& r
   ph.X0 = r.X0; ph.col_hi = r.col_hi; ph.col_lo = r.col_lo;
   ph.k = make_float3(r.kx, r.ky, r.kz);
   ph.fly = r.fly; ph.fly_tau = r.fly_tau;
+  ph.pl_ir = 0.0f;
   ph.x = r.x; ph.X = r.X; ph.safe = r.safe;
   ph.region = r.region;
   ph.nscat = r.nscat; ph.ndust = r.ndust; ph.iters = r.iters; ph.steps = r.steps;
@@ -871,7 +905,7 @@ __device__ __forceinline__ void load_rec(const ShellModel& m, const PhotonRec& r
 }
 
 // ---- work sharing in the tail of a one-launch run (pool_take in thor_device.cuh) ----------
-constexpr uint32_t kShareEvents = 512;  // a warp with several live packets checks for waiting warps this often
+constexpr uint32_t kShareEvents = 256;  // a warp with several live packets checks for waiting warps this often
 __device__ __forceinline__ long long share_take(const Compact& c) { return pool_take(c.share, c.ready, c.n_total); }
 
 // Run-to-completion: all queue entries belong to one model (thor_run).  With kCompact,
@@ -892,6 +926,8 @@ __global__ void __launch_bounds__(256, 1) shell_run_kernel(const ShellModel* __r
   Photon ph;
   bool active = false, done = (int)lane >= c.per_warp;  // lanes above per_warp stay idle
   bool drained = false;  // warp-uniform: a refill found the photon queue exhausted
+  uint32_t depth = kFirstDepth;  // of the warp's next round of core events
+  uint32_t ran = 0;  // events of the warp since the queue ran dry
   LaneTally lt;
   for (;;) {
     unsigned need = __ballot_sync(kFull, !active && !done);
@@ -948,7 +984,7 @@ __global__ void __launch_bounds__(256, 1) shell_run_kernel(const ShellModel* __r
         if (lane == 0) { load_rec(m, c.pool[got], ph); active = true; }
         continue;
       }
-      if (__popc(live) >= 2) {  // give packets away while empty warps wait, keeping the lowest lane's
+      if (__popc(live) >= 2 && ran >= kShareEvents) {  // (short histories are over by then) give packets away while empty warps wait, keeping the lowest lane's
         const int leader = __ffs(live) - 1;
         long long give = 0;
         if ((int)lane == leader) give = pool_give_count(c.share, __popc(live));
@@ -962,10 +998,10 @@ __global__ void __launch_bounds__(256, 1) shell_run_kernel(const ShellModel* __r
           base = __shfl_sync(kFull, base, leader);
           if (giver) {
             const unsigned long long j = base + (unsigned long long)from_top;
-            save_rec(ph, c.pool[j]);
-            __threadfence();
-            *(volatile uint32_t*)&c.ready[j] = 1u;
-            active = false;
+            if (j < c.n_total) {  // an entry per photon
+              save_rec(ph, c.pool[j]);
+              if (pool_put(c.ready, j)) active = false;
+            }
           }
         }
       }
@@ -974,7 +1010,7 @@ __global__ void __launch_bounds__(256, 1) shell_run_kernel(const ShellModel* __r
     const int n_live = __popc(__ballot_sync(kFull, active));
     const bool check_share = c.pool && drained && n_live >= 2;
     const bool chain = kProfile == 0 && n_live <= c.core_lanes;
-    const uint32_t depth = n_live <= c.burst_lanes || n_live <= kChainSlots / (int)kChainDepth ? kChainDepth : kCrowdDepth;
+    const uint32_t most = n_live <= c.burst_lanes || n_live <= kChainSlots / (int)kChainDepth ? kChainDepth : kCrowdDepth;
     uint32_t n_ev = 0;
     // events until some lane of the warp finishes its packet: the refill and spill checks
     // above run only when the set of live lanes changed
@@ -983,7 +1019,7 @@ __global__ void __launch_bounds__(256, 1) shell_run_kernel(const ShellModel* __r
       fin = false;
       bool general = active;  // lanes whose next event is a general one
       WordPos at;
-      if (chain) core_events(m, ph, wb, active, depth, general, at);
+      if (chain) core_events(m, ph, wb, active, depth, most, general, at);
       // packets whose next event is not of the core kind take general events: one, and more
       // while at least half of the warp's packets need them
       uint32_t n_gen = 0;
@@ -991,7 +1027,7 @@ __global__ void __launch_bounds__(256, 1) shell_run_kernel(const ShellModel* __r
         general_words(m, ph, wb, general, at);
         if (general) {
           const EventWords w = read_words(wb, at.cur * at.P + at.rank);
-          const int st = kProfile ? shell_event_pl(m, ph, sK, w) : shell_event(m, ph, sK, w);
+          const int st = kProfile ? shell_event_pl(m, &sm, ph, sK, w) : shell_event(m, ph, sK, w);
           if (st >= 0) ++at.cur;
           if (st > 0) {
             if (st == 1) { ++lt.esc; tally_spectrum(m, ph.X); }
@@ -1007,8 +1043,9 @@ __global__ void __launch_bounds__(256, 1) shell_run_kernel(const ShellModel* __r
           general = active && !(chain && chain_kind(m, ph));
         }
       } while (!__any_sync(kFull, fin) && ++n_gen < kCrowdDepth &&
-               2 * __popc(__ballot_sync(kFull, general)) >= n_live);
-      n_ev += chain ? depth : n_gen;
+               (kProfile || 2 * __popc(__ballot_sync(kFull, general)) >= n_live));
+      n_ev += chain ? most : n_gen;
+      if (drained) ran += chain ? most : 8u * n_gen;  // (a turn on a power law may be 128 sub-steps)
     } while (!__any_sync(kFull, fin) && !(check_share && n_ev >= kShareEvents));
   }
   // flush lane tallies: warp reduce, one atomic per warp and field
@@ -1101,10 +1138,12 @@ __global__ void __launch_bounds__(256, 1) shell_slice_kernel(const ShellModel* _
     ph.X0 = 0.0f; ph.col_hi = 0.0f; ph.col_lo = 0.0f;  // raw records are not served
     ph.region = st.region[slot];
     ph.fly = st.fly[slot]; ph.fly_tau = st.fly_tau[slot];
+    ph.pl_ir = 0.0f;
     ph.nscat = st.nscat[slot]; ph.ndust = st.ndust[slot]; ph.iters = st.iters[slot]; ph.steps = st.steps[slot];
     active = true;
   }
   uint32_t ev = 0;  // event iterations of this launch (warp-uniform)
+  uint32_t depth = kFirstDepth;  // of the warp's next round of core events
   auto others_done = [&]() { return pri_warp && ev >= base_budget && (int64_t)vload(&in.live[4]) >= n_regular; };
   while (ev < budget && !others_done()) {
     const unsigned idle = __ballot_sync(kFull, !active && !done);
@@ -1149,22 +1188,22 @@ __global__ void __launch_bounds__(256, 1) shell_slice_kernel(const ShellModel* _
     do {
       fin = false;
       bool general = active;
-      const uint32_t depth = min(n_live <= kChainSlots / (int)kChainDepth ? kChainDepth : kCrowdDepth, budget - ev);
+      const uint32_t most = min(n_live <= kChainSlots / (int)kChainDepth ? kChainDepth : kCrowdDepth, budget - ev);
       WordPos at;
-      uint32_t n = core_events(mr, ph, wb, active && chain, depth, general, at);
+      uint32_t n = core_events(mr, ph, wb, active && chain, depth, most, general, at);
       if (kMixed) general = general || (active && !chain);
       uint32_t n_gen = 0;
       do {
         general_words(mr, ph, wb, general, at);
         if (general) {
           const EventWords w = read_words(wb, at.cur * at.P + at.rank);
-          const int r = (kMixed && mr.profile) ? shell_event_pl(mr, ph, sK, w) : shell_event(mr, ph, sK, w);
+          const int r = (kMixed && mr.profile) ? shell_event_pl(mr, mp, ph, sK, w) : shell_event(mr, ph, sK, w);
           if (r >= 0) ++at.cur;
           ++n;
           if (r > 0) { finish_global(mr, ph, r); active = false; fin = true; }
           general = active && !(chain && chain_kind(mr, ph));
         }
-      } while (!__any_sync(kFull, fin) && ++n_gen < kCrowdDepth && n_gen + depth < budget - ev &&
+      } while (!__any_sync(kFull, fin) && ++n_gen < kCrowdDepth && n_gen + most < budget - ev &&
                2 * __popc(__ballot_sync(kFull, general)) >= n_live);
       ev += max(1u, __reduce_max_sync(kFull, n));
     } while (ev < budget && !__any_sync(kFull, fin) && !others_done());
