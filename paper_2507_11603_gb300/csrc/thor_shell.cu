@@ -99,9 +99,22 @@ __device__ __forceinline__ void anchor(Photon& ph) {
   ph.ox = 0.0f; ph.oy = 0.0f; ph.oz = 0.0f;
 }
 
+// FP64 sums of three products and r^2 - R^2 as the two event functions round them: which
+// products are fused is part of a history's bits (kPower: the power-law event).
+template <bool kPower>
+__device__ __forceinline__ double dot3(double ax, double ay, double az, double bx, double by, double bz) {
+  return kPower ? __fma_rn(az, bz, __fma_rn(ay, by, __dmul_rn(ax, bx)))
+                : __fma_rn(az, bz, __fma_rn(ax, bx, __dmul_rn(ay, by)));
+}
+template <bool kPower>
+__device__ __forceinline__ double minus_r2(double pp, double R) {
+  return kPower ? __fma_rn(-R, R, pp) : __dadd_rn(pp, -__dmul_rn(R, R));
+}
+
 // Exact distance from p to the nearest boundary, rounded down (conservative).
+template <bool kPower>
 __device__ __forceinline__ float safe_distance(const ShellModel& m, const Photon& ph) {
-  const double r = sqrt(ph.px * ph.px + ph.py * ph.py + ph.pz * ph.pz);
+  const double r = sqrt(dot3<kPower>(ph.px, ph.py, ph.pz, ph.px, ph.py, ph.pz));
   double d = m.R_out - r;
   if (m.R_in > 0.0) d = fmin(d, r - m.R_in);
   return fmaxf(__double2float_rd(d) * 0.999999f, 0.0f);
@@ -126,16 +139,17 @@ struct ShellSegment {
     }
   }
   // the distance and what is met there (1 outside, 2 cavity)
+  template <bool kPower>
   static __device__ __forceinline__ double exact(const ShellModel& m, double b, double pp, int& next) {
     next = 1;
     if (m.R_in > 0.0 && b < 0.0) {
-      const double disc = b * b - (pp - m.R_in * m.R_in);
+      const double disc = __fma_rn(b, b, -minus_r2<kPower>(pp, m.R_in));
       if (disc > 0.0) {  // nearer than the outer sphere: -b - sqrt(disc) < -b < its distance
         next = 2;
         return fmax(-b - sqrt(disc), 0.0);
       }
     }
-    return fmax(-b + sqrt(fmax(b * b - (pp - m.R_out * m.R_out), 0.0)), 0.0);
+    return fmax(-b + sqrt(fmax(__fma_rn(b, b, -minus_r2<kPower>(pp, m.R_out)), 0.0)), 0.0);
   }
   // Whether the point at s along the segment is certainly nearer than the sub-step to a
   // boundary: r - R_in = (r^2 - R_in^2) / (r + R_in) <= (r^2 - R_in^2) / (2 R_in), likewise
@@ -225,10 +239,10 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
     if (ph.region) {  // empty cavity: straight to the inner sphere, lab X conserved
       anchor(ph);
       const double kx = ph.k.x, ky = ph.k.y, kz = ph.k.z;
-      const double b = ph.px * kx + ph.py * ky + ph.pz * kz;
-      const double c = ph.px * ph.px + ph.py * ph.py + ph.pz * ph.pz - m.R_in * m.R_in;
-      const double s = -b + sqrt(fmax(b * b - c, 0.0));
-      ph.px += s * kx; ph.py += s * ky; ph.pz += s * kz;
+      const double b = dot3<false>(ph.px, ph.py, ph.pz, kx, ky, kz);
+      const double c = minus_r2<false>(dot3<false>(ph.px, ph.py, ph.pz, ph.px, ph.py, ph.pz), m.R_in);
+      const double s = -b + sqrt(fmax(__fma_rn(b, b, -c), 0.0));
+      ph.px = __fma_rn(s, kx, ph.px); ph.py = __fma_rn(s, ky, ph.py); ph.pz = __fma_rn(s, kz, ph.pz);
       ph.region = 0;
       ph.x = (ph.X - m.vgrad * (float)(b + s)) * m.inv_vth;
       ph.safe = 0.0f;
@@ -287,8 +301,8 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
     // (FP64) where it counts
     anchor(ph);
     const double kx = ph.k.x, ky = ph.k.y, kz = ph.k.z;
-    const double b = ph.px * kx + ph.py * ky + ph.pz * kz;
-    const double pp = ph.px * ph.px + ph.py * ph.py + ph.pz * ph.pz;
+    const double b = dot3<false>(ph.px, ph.py, ph.pz, kx, ky, kz);
+    const double pp = dot3<false>(ph.px, ph.py, ph.pz, ph.px, ph.py, ph.pz);
     const ShellSegment seg(m, b, pp);
     const float x0 = ph.x;
     double S = 0.0;  // distance to the boundary, once needed (seg.exact), and what is there
@@ -296,7 +310,7 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
     int next = 1;
     float s_star = -1.0f;
     if (m.gam == 0.0f) {
-      S = seg.exact(m, b, pp, next);
+      S = ShellSegment::exact<false>(m, b, pp, next);
       Sf = (float)S;
       const float kap = kH + m.kapd;
       if (kap * Sf >= tau_rem) s_star = fminf(tau_rem / kap, Sf);
@@ -313,7 +327,7 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
         --turn_steps;
         float s1 = s + m.ds_core;
         if (!have && !(s1 <= seg.lower)) {
-          S = seg.exact(m, b, pp, next);
+          S = ShellSegment::exact<false>(m, b, pp, next);
           Sf = (float)S;
           have = true;
         }
@@ -344,16 +358,16 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
     }
     if (s_star >= 0.0f) {
       const double sd = s_star;
-      ph.px += sd * kx; ph.py += sd * ky; ph.pz += sd * kz;
+      ph.px = __fma_rn(sd, kx, ph.px); ph.py = __fma_rn(sd, ky, ph.py); ph.pz = __fma_rn(sd, kz, ph.pz);
       x_site = x0 - m.gam * s_star;
       if (m.gam != 0.0f) kH = m.kap0 * voigt<false>(m.a, x_site, Ktab);
       // the safety distance counts only from ds on: where it is certainly shorter (photons
       // trapped at the shell's edge, which come here event after event) its FP64 square root
       // is left out
-      ph.safe = (m.gam != 0.0f && seg.near_edge(m, s_star)) ? 0.0f : safe_distance(m, ph);
+      ph.safe = (m.gam != 0.0f && seg.near_edge(m, s_star)) ? 0.0f : safe_distance<false>(m, ph);
       break;
     }
-    ph.px += S * kx; ph.py += S * ky; ph.pz += S * kz;
+    ph.px = __fma_rn(S, kx, ph.px); ph.py = __fma_rn(S, ky, ph.py); ph.pz = __fma_rn(S, kz, ph.pz);
     const float x_end = x0 - m.gam * Sf;
     ph.X = __fmaf_rn(x_end, m.vth, m.vgrad * (float)(b + S));  // lab frequency at the boundary
     if (next == 1) return 1;
@@ -670,10 +684,10 @@ __device__ int shell_event_pl(const ShellModel& m, const ShellModel* mp, Photon&
     if (ph.region) {  // empty cavity: straight to the inner sphere, lab X conserved
       anchor(ph);
       const double kx = ph.k.x, ky = ph.k.y, kz = ph.k.z;
-      const double b = ph.px * kx + ph.py * ky + ph.pz * kz;
-      const double c = ph.px * ph.px + ph.py * ph.py + ph.pz * ph.pz - m.R_in * m.R_in;
-      const double s = -b + sqrt(fmax(b * b - c, 0.0));
-      ph.px += s * kx; ph.py += s * ky; ph.pz += s * kz;
+      const double b = dot3<true>(ph.px, ph.py, ph.pz, kx, ky, kz);
+      const double c = minus_r2<true>(dot3<true>(ph.px, ph.py, ph.pz, ph.px, ph.py, ph.pz), m.R_in);
+      const double s = -b + sqrt(fmax(__fma_rn(b, b, -c), 0.0));
+      ph.px = __fma_rn(s, kx, ph.px); ph.py = __fma_rn(s, ky, ph.py); ph.pz = __fma_rn(s, kz, ph.pz);
       ph.region = 0;
       ph.safe = 0.0f;
       ph.pl_ir = 0.0f;
@@ -691,7 +705,7 @@ __device__ int shell_event_pl(const ShellModel& m, const ShellModel* mp, Photon&
       ++ph.steps;
       const bool is_short = s0 <= 0.0625f * m.ds_core;
       // the safety distance (an FP64 square root) is formed where it decides
-      if (is_short && ph.safe == kSafePending) ph.safe = safe_distance(m, ph);
+      if (is_short && ph.safe == kSafePending) ph.safe = safe_distance<true>(m, ph);
       if (is_short && s0 <= ph.safe) {
         advance(ph, s0);
         ph.safe = __fmaf_rd(-s0, 1.000001f, ph.safe);
@@ -741,11 +755,11 @@ __device__ int shell_event_pl(const ShellModel& m, const ShellModel* mp, Photon&
       --turn_steps;
       float s1 = s + m.ds_core;
       if (!have && !(s1 <= lower)) {  // the bound from the radius alone, then along the ray, then exact
-        const double b = ph.px * kx + ph.py * ky + ph.pz * kz;
-        const double pp = ph.px * ph.px + ph.py * ph.py + ph.pz * ph.pz;
+        const double b = dot3<true>(ph.px, ph.py, ph.pz, kx, ky, kz);
+        const double pp = dot3<true>(ph.px, ph.py, ph.pz, ph.px, ph.py, ph.pz);
         lower = ShellSegment(m, b, pp).lower;
         if (!(s1 <= lower)) {
-          S = ShellSegment::exact(m, b, pp, next);
+          S = ShellSegment::exact<true>(m, b, pp, next);
           Sf = (float)S;
           have = true;
         }
@@ -785,13 +799,13 @@ __device__ int shell_event_pl(const ShellModel& m, const ShellModel* mp, Photon&
     }
     if (s_star >= 0.0f) {
       const double sd = s_star;
-      ph.px += sd * kx; ph.py += sd * ky; ph.pz += sd * kz;
+      ph.px = __fma_rn(sd, kx, ph.px); ph.py = __fma_rn(sd, ky, ph.py); ph.pz = __fma_rn(sd, kz, ph.pz);
       ph.safe = kSafePending;
       ph.qx = (float)ph.px; ph.qy = (float)ph.py; ph.qz = (float)ph.pz;
       site = pl_state(m, ph.qx, ph.qy, ph.qz, ph.k);
       break;
     }
-    ph.px += S * kx; ph.py += S * ky; ph.pz += S * kz;
+    ph.px = __fma_rn(S, kx, ph.px); ph.py = __fma_rn(S, ky, ph.py); ph.pz = __fma_rn(S, kz, ph.pz);
     if (next == 1) return 1;  // escapes with its lab X
     ph.region = 1;
   }
