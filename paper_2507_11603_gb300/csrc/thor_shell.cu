@@ -100,16 +100,14 @@ __device__ __forceinline__ void anchor(Photon& ph) {
 }
 
 // FP64 sums of three products and r^2 - R^2 as the two event functions round them: which
-// products are fused is part of a history's bits (kPower: the power-law event).
+// products are fused is part of a history's bits (kPower: the power-law event), so nothing
+// here is left to the compiler.
 template <bool kPower>
 __device__ __forceinline__ double dot3(double ax, double ay, double az, double bx, double by, double bz) {
   return kPower ? __fma_rn(az, bz, __fma_rn(ay, by, __dmul_rn(ax, bx)))
                 : __fma_rn(az, bz, __fma_rn(ax, bx, __dmul_rn(ay, by)));
 }
-template <bool kPower>
-__device__ __forceinline__ double minus_r2(double pp, double R) {
-  return kPower ? __fma_rn(-R, R, pp) : __dadd_rn(pp, -__dmul_rn(R, R));
-}
+__device__ __forceinline__ double minus_r2(double pp, double R) { return __dadd_rn(pp, -__dmul_rn(R, R)); }
 
 // Exact distance from p to the nearest boundary, rounded down (conservative).
 template <bool kPower>
@@ -139,17 +137,16 @@ struct ShellSegment {
     }
   }
   // the distance and what is met there (1 outside, 2 cavity)
-  template <bool kPower>
   static __device__ __forceinline__ double exact(const ShellModel& m, double b, double pp, int& next) {
     next = 1;
     if (m.R_in > 0.0 && b < 0.0) {
-      const double disc = __fma_rn(b, b, -minus_r2<kPower>(pp, m.R_in));
+      const double disc = __fma_rn(b, b, -minus_r2(pp, m.R_in));
       if (disc > 0.0) {  // nearer than the outer sphere: -b - sqrt(disc) < -b < its distance
         next = 2;
         return fmax(-b - sqrt(disc), 0.0);
       }
     }
-    return fmax(-b + sqrt(fmax(__fma_rn(b, b, -minus_r2<kPower>(pp, m.R_out)), 0.0)), 0.0);
+    return fmax(-b + sqrt(fmax(__fma_rn(b, b, -minus_r2(pp, m.R_out)), 0.0)), 0.0);
   }
   // Whether the point at s along the segment is certainly nearer than the sub-step to a
   // boundary: r - R_in = (r^2 - R_in^2) / (r + R_in) <= (r^2 - R_in^2) / (2 R_in), likewise
@@ -240,7 +237,7 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
       anchor(ph);
       const double kx = ph.k.x, ky = ph.k.y, kz = ph.k.z;
       const double b = dot3<false>(ph.px, ph.py, ph.pz, kx, ky, kz);
-      const double c = minus_r2<false>(dot3<false>(ph.px, ph.py, ph.pz, ph.px, ph.py, ph.pz), m.R_in);
+      const double c = minus_r2(dot3<false>(ph.px, ph.py, ph.pz, ph.px, ph.py, ph.pz), m.R_in);
       const double s = -b + sqrt(fmax(__fma_rn(b, b, -c), 0.0));
       ph.px = __fma_rn(s, kx, ph.px); ph.py = __fma_rn(s, ky, ph.py); ph.pz = __fma_rn(s, kz, ph.pz);
       ph.region = 0;
@@ -310,7 +307,7 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
     int next = 1;
     float s_star = -1.0f;
     if (m.gam == 0.0f) {
-      S = ShellSegment::exact<false>(m, b, pp, next);
+      S = ShellSegment::exact(m, b, pp, next);
       Sf = (float)S;
       const float kap = kH + m.kapd;
       if (kap * Sf >= tau_rem) s_star = fminf(tau_rem / kap, Sf);
@@ -327,7 +324,7 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
         --turn_steps;
         float s1 = s + m.ds_core;
         if (!have && !(s1 <= seg.lower)) {
-          S = ShellSegment::exact<false>(m, b, pp, next);
+          S = ShellSegment::exact(m, b, pp, next);
           Sf = (float)S;
           have = true;
         }
@@ -685,7 +682,7 @@ __device__ int shell_event_pl(const ShellModel& m, const ShellModel* mp, Photon&
       anchor(ph);
       const double kx = ph.k.x, ky = ph.k.y, kz = ph.k.z;
       const double b = dot3<true>(ph.px, ph.py, ph.pz, kx, ky, kz);
-      const double c = minus_r2<true>(dot3<true>(ph.px, ph.py, ph.pz, ph.px, ph.py, ph.pz), m.R_in);
+      const double c = minus_r2(dot3<true>(ph.px, ph.py, ph.pz, ph.px, ph.py, ph.pz), m.R_in);
       const double s = -b + sqrt(fmax(__fma_rn(b, b, -c), 0.0));
       ph.px = __fma_rn(s, kx, ph.px); ph.py = __fma_rn(s, ky, ph.py); ph.pz = __fma_rn(s, kz, ph.pz);
       ph.region = 0;
@@ -759,7 +756,7 @@ __device__ int shell_event_pl(const ShellModel& m, const ShellModel* mp, Photon&
         const double pp = dot3<true>(ph.px, ph.py, ph.pz, ph.px, ph.py, ph.pz);
         lower = ShellSegment(m, b, pp).lower;
         if (!(s1 <= lower)) {
-          S = ShellSegment::exact<true>(m, b, pp, next);
+          S = ShellSegment::exact(m, b, pp, next);
           Sf = (float)S;
           have = true;
         }
