@@ -47,9 +47,29 @@ void* thor_ctx::scratch(Buf& b, size_t bytes) {
   return b.p;
 }
 
+void* thor_ctx::pinned(size_t bytes) {
+  if (bytes > kPinnedMax) return nullptr;
+  if (pinned_cap >= bytes) return h_pinned;
+  if (h_pinned) {
+    cudaStreamSynchronize(stream);  // no copy out of the old block is in flight
+    cudaFreeHost(h_pinned);
+  }
+  h_pinned = nullptr;
+  pinned_cap = 0;
+  const size_t cap = bytes < 16384 ? 16384 : bytes;
+  if (cudaMallocHost(&h_pinned, cap) != cudaSuccess) {
+    h_pinned = nullptr;
+    cudaGetLastError();
+    return nullptr;
+  }
+  pinned_cap = cap;
+  return h_pinned;
+}
+
 thor_ctx::~thor_ctx() {
   cudaSetDevice(device);
-  for (Buf* b : {&b_models, &b_tally, &b_queue, &b_spec, &b_cube, &b_raw, &b_raw2, &b_diag, &b_stats, &b_spill, &b_cmp,
+  if (h_pinned) cudaFreeHost(h_pinned);
+  for (Buf* b : {&b_run, &b_cube, &b_raw, &b_raw2, &b_diag, &b_stats, &b_spill, &b_cmp,
                  &b_stage[0], &b_stage[1], &b_gslots, &b_share})
     if (b->p) cudaFree(b->p);
   for (cudaEvent_t e : {ev_copied[0], ev_copied[1], ev_done[0], ev_done[1]})
@@ -343,18 +363,26 @@ extern "C" int thor_grid_create(thor_ctx_t ctx, const float* n_HI, const float* 
   g->cell_cm = cell_cm;
   g->n_cells = n;
   const size_t fb = (size_t)n * sizeof(float);
-  float* stage = nullptr;
+  float *stage = nullptr, *own_stage = nullptr;
   int rc = THOR_OK;
-  if (cudaMalloc(&g->cells, (size_t)n * sizeof(GridCell)) != cudaSuccess ||
-      cudaMalloc(&g->cdf, (size_t)n * sizeof(double)) != cudaSuccess ||
-      cudaMalloc(&g->scan_tmp, scan_f64_scratch(n) + sizeof(unsigned long long)) != cudaSuccess) {
+  // one block: cells, emission CDF, scan scratch and the counter of unusable cells
+  auto r256 = [](size_t b) { return (b + 255) & ~(size_t)255; };
+  const size_t b_cells = r256((size_t)n * sizeof(GridCell)), b_cdf = r256((size_t)n * sizeof(double));
+  if (cudaMalloc(&g->cells, b_cells + b_cdf + scan_f64_scratch(n) + sizeof(unsigned long long)) != cudaSuccess) {
+    g->cells = nullptr;
     delete g;
     return ctx->fail(THOR_ERR_OOM, "thor_grid_create: cannot allocate %lld cells", (long long)n);
   }
+  g->cdf = (double*)((char*)g->cells + b_cells);
+  g->scan_tmp = (double*)((char*)g->cells + b_cells + b_cdf);
   const float *dn = n_HI, *dT = T, *dvx = v, *dvy = v + n, *dvz = v + 2 * n, *dd = dust;
   if (mem_kind == THOR_MEM_HOST) {  // stage the six fields on the device
     const int nf = dust ? 6 : 5;
-    if (cudaMalloc(&stage, fb * nf) != cudaSuccess) {
+    // small grids through the context's scratch, large ones through a block of their own
+    const bool kept = fb * nf <= ((size_t)64 << 20);
+    if (kept) stage = (float*)ctx->scratch(ctx->b_diag, fb * nf);
+    else if (cudaMalloc(&own_stage, fb * nf) == cudaSuccess) stage = own_stage;
+    if (!stage) {
       delete g;
       return ctx->fail(THOR_ERR_OOM, "thor_grid_create: cannot stage fields");
     }
@@ -371,16 +399,20 @@ extern "C" int thor_grid_create(thor_ctx_t ctx, const float* n_HI, const float* 
     rc = ctx->cuda(launch_grid_pack(dn, dT, dvx, dvy, dvz, dd, n, cell_cm, g->cells, g->cdf, d_bad, ctx->stream),
                    "grid pack");
   if (rc == THOR_OK) rc = ctx->cuda(launch_scan_f64(g->cdf, n, g->scan_tmp, ctx->stream), "emission CDF");
-  if (rc == THOR_OK) rc = ctx->cuda(cudaStreamSynchronize(ctx->stream), "grid create");
-  if (stage) cudaFree(stage);
+  struct Check { unsigned long long bad; double total; };
+  Check* chk = (Check*)ctx->pinned(sizeof(Check));
+  if (!chk && rc == THOR_OK) rc = ctx->fail(THOR_ERR_OOM, "thor_grid_create: staging");
+  if (rc == THOR_OK)
+    rc = ctx->cuda(cudaMemcpyAsync(&chk->bad, d_bad, sizeof chk->bad, cudaMemcpyDeviceToHost, ctx->stream), "grid check");
+  if (rc == THOR_OK)
+    rc = ctx->cuda(cudaMemcpyAsync(&chk->total, g->cdf + (n - 1), sizeof(double), cudaMemcpyDeviceToHost, ctx->stream),
+                   "grid CDF");
+  const int rs = ctx->cuda(cudaStreamSynchronize(ctx->stream), "grid create");
+  if (own_stage) cudaFree(own_stage);
+  if (rc == THOR_OK) rc = rs;
   if (rc != THOR_OK) { delete g; return rc; }
-  unsigned long long bad = 0;
-  double total = 0.0;
-  if ((rc = ctx->cuda(cudaMemcpy(&bad, d_bad, sizeof bad, cudaMemcpyDeviceToHost), "grid check")) ||
-      (rc = ctx->cuda(cudaMemcpy(&total, g->cdf + (n - 1), sizeof(double), cudaMemcpyDeviceToHost), "grid CDF"))) {
-    delete g;
-    return rc;
-  }
+  const unsigned long long bad = chk->bad;
+  const double total = chk->total;
   if (bad) {
     delete g;
     return ctx->fail(THOR_ERR_INVALID_ARG,
@@ -393,14 +425,20 @@ extern "C" int thor_grid_create(thor_ctx_t ctx, const float* n_HI, const float* 
 
 thor_geom::~thor_geom() {
   if (ctx) cudaSetDevice(ctx->device);
-  if (cells) cudaFree(cells);
-  if (cdf) cudaFree(cdf);
-  if (scan_tmp) cudaFree(scan_tmp);
+  if (cells) cudaFree(cells);  // the CDF and the scan scratch lie in the same block
 }
 
 extern "C" void thor_geom_destroy(thor_geom_t g) { delete g; }
 
 // ------------------------------------------------------------------------------ run
+// A run's device record, uploaded by one copy and read back by one: queue, model, tally,
+// counters and (for host callers) the spectrum.  A small run is bound by its calls: 256 photons
+// through a thin sphere took 167 us, of them about 45 in the kernel, with five small uploads
+// and clears and three results one after another; 141 us now.
+constexpr size_t kRunModel = 256, kRunTally = 1024, kRunStats = kRunTally + sizeof(Tally), kRunShare = kRunStats + 64,
+                 kRunSpec = 1536;
+static_assert(kRunModel + sizeof(ShellModel) <= kRunTally && kRunShare + 64 <= kRunSpec, "run record layout");
+
 int thor::prepare_outputs(thor_ctx* ctx, const thor_output_spec* spec, uint64_t n_photons, bool grid, OutBufs* o) {
   if (!spec || !spec->spectrum) return ctx->fail(THOR_ERR_INVALID_ARG, "output spec / spectrum is NULL");
   if (spec->n_bins <= 0 || !(spec->X_max > spec->X_min)) return ctx->fail(THOR_ERR_INVALID_ARG, "bad spectrum binning");
@@ -408,9 +446,12 @@ int thor::prepare_outputs(thor_ctx* ctx, const thor_output_spec* spec, uint64_t 
     return ctx->fail(THOR_ERR_INVALID_ARG, "bad output mem_kind");
   const bool dev = spec->mem_kind == THOR_MEM_DEVICE;
   const size_t sb = (size_t)(spec->n_bins + 2) * sizeof(uint64_t);
-  o->spec = dev ? (unsigned long long*)spec->spectrum : (unsigned long long*)ctx->scratch(ctx->b_spec, sb);
-  if (!o->spec) return ctx->fail(THOR_ERR_OOM, "spectrum buffer");
-  if (int rc = ctx->cuda(cudaMemsetAsync(o->spec, 0, sb, ctx->stream), "clear spectrum")) return rc;
+  // a host spectrum is tallied in the run's record (cleared with it)
+  char* rec = (char*)ctx->scratch(ctx->b_run, kRunSpec + (dev ? 0 : sb));
+  if (!rec) return ctx->fail(THOR_ERR_OOM, "run record");
+  o->spec = dev ? (unsigned long long*)spec->spectrum : (unsigned long long*)(rec + kRunSpec);
+  if (dev)
+    if (int rc = ctx->cuda(cudaMemsetAsync(o->spec, 0, sb, ctx->stream), "clear spectrum")) return rc;
   o->cube = nullptr;
   if (grid && spec->peel) {
     if (!spec->cube || spec->img_n <= 0 || spec->peel_bins <= 0 || !(spec->peel_X_max > spec->peel_X_min))
@@ -452,9 +493,8 @@ int thor::prepare_outputs(thor_ctx* ctx, const thor_output_spec* spec, uint64_t 
 int thor::finish_outputs(thor_ctx* ctx, const thor_output_spec* spec, uint64_t n_photons, bool grid, const OutBufs& o) {
   if (spec->mem_kind == THOR_MEM_DEVICE) return THOR_OK;
   cudaStream_t s = ctx->stream;
-  int rc = ctx->cuda(cudaMemcpyAsync(spec->spectrum, o.spec, (size_t)(spec->n_bins + 2) * 8, cudaMemcpyDeviceToHost, s),
-                     "copy spectrum");
-  if (rc == THOR_OK && o.cube)
+  int rc = THOR_OK;
+  if (o.cube)
     rc = ctx->cuda(cudaMemcpyAsync(spec->cube, o.cube, (size_t)3 * spec->img_n * spec->img_n * spec->peel_bins * 4,
                                    cudaMemcpyDeviceToHost, s), "copy cube");
   if (rc == THOR_OK && o.raw_X) {
@@ -543,15 +583,27 @@ extern "C" int thor_run(thor_ctx_t ctx, thor_geom_t g, const thor_source* src, u
   OutBufs o;
   if (int rc = prepare_outputs(ctx, spec, n_photons, grid, &o)) return rc;
   cudaStream_t s = ctx->stream;
-  // per-run device scratch: tally, queue counter + tables, model record, peel statistics
-  Tally* d_tally = (Tally*)ctx->scratch(ctx->b_tally, sizeof(Tally));
-  char* qb = (char*)ctx->scratch(ctx->b_queue, 256);
-  unsigned long long* d_stats = (unsigned long long*)ctx->scratch(ctx->b_stats, 2 * sizeof(unsigned long long));
-  if (!d_tally || !qb || !d_stats) return ctx->fail(THOR_ERR_OOM, "run scratch");
+  char* rec = (char*)ctx->b_run.p;
+  Tally* d_tally = (Tally*)(rec + kRunTally);
+  unsigned long long* d_stats = (unsigned long long*)(rec + kRunStats);
   struct QHost { unsigned long long next, prefix[2], first_id; int32_t model; } qh{0, {0, n_photons}, first_id, 0};
-  if (int rc = ctx->cuda(cudaMemcpyAsync(qb, &qh, sizeof qh, cudaMemcpyHostToDevice, s), "queue upload")) return rc;
-  if (int rc = ctx->cuda(cudaMemsetAsync(d_tally, 0, sizeof(Tally), s), "clear tally")) return rc;
-  if (int rc = ctx->cuda(cudaMemsetAsync(d_stats, 0, 16, s), "clear stats")) return rc;
+  static_assert(sizeof(QHost) <= kRunModel, "run record layout");
+  const bool dev_out = spec->mem_kind == THOR_MEM_DEVICE;
+  const size_t sb = dev_out ? 0 : (size_t)(spec->n_bins + 2) * 8;
+  // the record's image in page-locked memory; a spectrum too long for it is cleared and copied
+  // by itself
+  const bool spec_in = kRunSpec + sb <= ((size_t)1 << 20);
+  const size_t rec_bytes = kRunSpec + (spec_in ? sb : 0);
+  char* img = (char*)ctx->pinned(rec_bytes);
+  if (!img) return ctx->fail(THOR_ERR_OOM, "run staging");
+  std::memset(img, 0, rec_bytes);
+  std::memcpy(img, &qh, sizeof qh);
+  auto upload = [&]() {
+    int e = ctx->cuda(cudaMemcpyAsync(rec, img, rec_bytes, cudaMemcpyHostToDevice, s), "run record upload");
+    if (!e && !spec_in) e = ctx->cuda(cudaMemsetAsync(o.spec, 0, sb, s), "clear spectrum");
+    return e;
+  };
+  char* qb = rec;
   unsigned long long n_launch = 0;
   WorkQueue q;
   q.next = (unsigned long long*)(qb + offsetof(QHost, next));
@@ -561,6 +613,8 @@ extern "C" int thor_run(thor_ctx_t ctx, thor_geom_t g, const thor_source* src, u
   q.model = (const int32_t*)(qb + offsetof(QHost, model));
   q.n_entries = 1;
   int rc = THOR_OK;
+  bool shared = false;  // the run shared its tail: pool
+  PhotonRec* pool = nullptr;
   if (!grid) {
     ShellModel m = g->shell;
     if ((rc = fill_shell_source(ctx, src, &m))) return rc;
@@ -577,10 +631,13 @@ extern "C" int thor_run(thor_ctx_t ctx, thor_geom_t g, const thor_source* src, u
     m.raw_X = o.raw_X; m.raw_nscat = o.raw_n; m.raw_status = o.raw_s;
     m.id_base = first_id;
     m.n_photons = n_photons;
-    ShellModel* d_m = (ShellModel*)ctx->scratch(ctx->b_models, sizeof(ShellModel));
-    if (!d_m) return ctx->fail(THOR_ERR_OOM, "model table");
-    if ((rc = ctx->cuda(cudaMemcpyAsync(d_m, &m, sizeof m, cudaMemcpyHostToDevice, s), "model upload"))) return rc;
-    const int gsz = shell_grid(ctx->block, ctx->blocks_per_sm, false);
+    ShellModel* d_m = (ShellModel*)(rec + kRunModel);
+    std::memcpy(img + kRunModel, &m, sizeof m);
+    if ((rc = upload())) return rc;
+    thor_ctx::GridSize& gs = ctx->shell_size;
+    if (gs.block != ctx->block || gs.per_sm != ctx->blocks_per_sm)
+      gs = {ctx->block, ctx->blocks_per_sm, shell_grid(ctx->block, ctx->blocks_per_sm, false)};
+    const int gsz = gs.size;
     // fewer photons than lanes: spread them over all warps (each runs closer to alone)
     const unsigned long long warps0 = (unsigned long long)gsz * (ctx->block / 32);
     const unsigned long long pw0 = (n_photons + warps0 - 1) / warps0;
@@ -592,48 +649,21 @@ extern "C" int thor_run(thor_ctx_t ctx, thor_geom_t g, const thor_source* src, u
       if (share) {
         auto r256 = [](size_t b) { return (b + 255) & ~(size_t)255; };
         const size_t b_pool = r256((size_t)n_photons * sizeof(PhotonRec)), b_ready = r256((size_t)n_photons * 4);
-        char* sb = (char*)ctx->scratch(ctx->b_share, b_pool + b_ready + 64);
-        if (!sb) return ctx->fail(THOR_ERR_OOM, "tail work-sharing pool");
-        sh.pool = (PhotonRec*)sb;
-        sh.ready = (uint32_t*)(sb + b_pool);
-        sh.share = (unsigned long long*)(sb + b_pool + b_ready);
+        char* pb = (char*)ctx->scratch(ctx->b_share, b_pool + b_ready);
+        if (!pb) return ctx->fail(THOR_ERR_OOM, "tail work-sharing pool");
+        sh.pool = (PhotonRec*)pb;
+        sh.ready = (uint32_t*)(pb + b_pool);
+        sh.share = (unsigned long long*)(rec + kRunShare);
         sh.n_total = n_photons;
-        if ((rc = ctx->cuda(cudaMemsetAsync(sh.ready, 0, b_ready + 64, s), "clear sharing pool"))) return rc;
+        if ((rc = ctx->cuda(cudaMemsetAsync(sh.ready, 0, b_ready, s), "clear sharing pool"))) return rc;
       }
       cudaEventRecord(ctx->ev0, s);
       rc = ctx->cuda(launch_shell_run(d_m, q, ctx->d_ktab, gsz, ctx->block, m.profile, per_warp0, ctx->core_lanes,
                                       ctx->burst_lanes, s, share ? &sh : nullptr),
                      "shell photon loop");
       ++n_launch;
-      if (!rc && share) {
-        // packets left in the pool (every waiting warp gave up first) finish in a relaunch
-        unsigned long long h[2];
-        if ((rc = ctx->cuda(cudaMemcpyAsync(h, sh.share, sizeof h, cudaMemcpyDeviceToHost, s), "sharing counters")))
-          return rc;
-        if ((rc = ctx->cuda(cudaStreamSynchronize(s), "shell photon loop"))) return rc;
-        h[0] = h[0] < n_photons ? h[0] : n_photons;
-        if (h[1] < h[0]) {
-          unsigned long long* ctr = (unsigned long long*)ctx->scratch(ctx->b_cmp, 4 * sizeof(unsigned long long));
-          if (!ctr) return ctx->fail(THOR_ERR_OOM, "resume counters");
-          if ((rc = ctx->cuda(cudaMemsetAsync(ctr, 0, 2 * sizeof(unsigned long long), s), "clear counters"))) return rc;
-          Compact c{};
-          c.resume = sh.pool + h[1];
-          c.n_resume = h[0] - h[1];
-          c.resume_next = ctr;
-          c.spill = nullptr;
-          c.n_spill = ctr + 1;
-          c.spill_below = 0;
-          c.per_warp = 1;
-          c.core_lanes = ctx->core_lanes;
-          c.burst_lanes = ctx->burst_lanes;
-          const unsigned long long want = (c.n_resume * 32 + ctx->block - 1) / ctx->block;
-          const int g = (int)(want < (unsigned long long)gsz ? want : gsz);
-          if ((rc = ctx->cuda(launch_shell_run_compact(d_m, q, c, ctx->d_ktab, g, ctx->block, m.profile, s),
-                              "shell photon loop (pool)")))
-            return rc;
-          ++n_launch;
-        }
-      }
+      shared = !rc && share;
+      pool = sh.pool;
       cudaEventRecord(ctx->ev1, s);
     } else {
       // Tail compaction: launch, then relaunch over the saved survivors until none are
@@ -718,7 +748,11 @@ extern "C" int thor_run(thor_ctx_t ctx, thor_geom_t g, const thor_source* src, u
     m.n_photons = n_photons; m.id_base = first_id;
     m.peel_rays = d_stats; m.peel_cells = d_stats + 1;
     m.raw_X = o.raw_X; m.raw_nscat = o.raw_n; m.raw_status = o.raw_s;
-    const int gsz = grid_grid(ctx->block, ctx->blocks_per_sm);
+    if ((rc = upload())) return rc;
+    thor_ctx::GridSize& gs = ctx->grid_size;
+    if (gs.block != ctx->block || gs.per_sm != ctx->blocks_per_sm)
+      gs = {ctx->block, ctx->blocks_per_sm, grid_grid(ctx->block, ctx->blocks_per_sm)};
+    const int gsz = gs.size;
     // few photons: spread them so that each runs in a warp of its own where possible
     const unsigned long long warps = (unsigned long long)gsz * (ctx->block / 32);
     auto per_warp = [&](unsigned long long n) {
@@ -737,12 +771,50 @@ extern "C" int thor_run(thor_ctx_t ctx, thor_geom_t g, const thor_source* src, u
     }
   }
   if (rc) return rc;
+  auto read_back = [&]() {
+    return ctx->cuda(cudaMemcpyAsync(img + kRunTally, rec + kRunTally, rec_bytes - kRunTally, cudaMemcpyDeviceToHost, s),
+                     "run record");
+  };
+  if ((rc = read_back())) return rc;
+  if (shared) {
+    // packets left in the pool (every waiting warp gave up first) finish in a relaunch
+    if ((rc = ctx->cuda(cudaStreamSynchronize(s), "shell photon loop"))) return rc;
+    unsigned long long h[2];  // entries reserved, tickets taken
+    std::memcpy(h, img + kRunShare, sizeof h);
+    if (h[0] > n_photons) h[0] = n_photons;
+    if (h[1] < h[0]) {
+      unsigned long long* ctr = (unsigned long long*)ctx->scratch(ctx->b_cmp, 4 * sizeof(unsigned long long));
+      if (!ctr) return ctx->fail(THOR_ERR_OOM, "resume counters");
+      if ((rc = ctx->cuda(cudaMemsetAsync(ctr, 0, 2 * sizeof(unsigned long long), s), "clear counters"))) return rc;
+      Compact c{};
+      c.resume = pool + h[1];
+      c.n_resume = h[0] - h[1];
+      c.resume_next = ctr;
+      c.n_spill = ctr + 1;
+      c.per_warp = 1;
+      c.core_lanes = ctx->core_lanes;
+      c.burst_lanes = ctx->burst_lanes;
+      const unsigned long long want = (c.n_resume * 32 + ctx->block - 1) / ctx->block;
+      const int gw = (int)(want < (unsigned long long)ctx->shell_size.size ? want : ctx->shell_size.size);
+      if ((rc = ctx->cuda(launch_shell_run_compact((ShellModel*)(rec + kRunModel), q, c, ctx->d_ktab, gw, ctx->block,
+                                                   g->shell.profile, s),
+                          "shell photon loop (pool)")))
+        return rc;
+      ++n_launch;
+      cudaEventRecord(ctx->ev1, s);
+      if ((rc = read_back())) return rc;
+    }
+  }
+  if (!spec_in)
+    rc = ctx->cuda(cudaMemcpyAsync(spec->spectrum, o.spec, sb, cudaMemcpyDeviceToHost, s), "copy spectrum");
+  if (!rc) rc = finish_outputs(ctx, spec, n_photons, grid, o);
+  if (!rc) rc = ctx->cuda(cudaStreamSynchronize(s), "photon loop");
+  if (rc) return rc;
   Tally t;
   unsigned long long st[2];
-  if ((rc = ctx->cuda(cudaMemcpyAsync(&t, d_tally, sizeof t, cudaMemcpyDeviceToHost, s), "copy tally"))) return rc;
-  if ((rc = ctx->cuda(cudaMemcpyAsync(st, d_stats, sizeof st, cudaMemcpyDeviceToHost, s), "copy stats"))) return rc;
-  if ((rc = finish_outputs(ctx, spec, n_photons, grid, o))) return rc;
-  if ((rc = ctx->cuda(cudaStreamSynchronize(s), "photon loop"))) return rc;
+  std::memcpy(&t, img + kRunTally, sizeof t);
+  std::memcpy(st, img + kRunStats, sizeof st);
+  if (spec_in && !dev_out) std::memcpy(spec->spectrum, img + kRunSpec, sb);
   std::memset(out, 0, sizeof *out);
   tally_to_result(t, n_photons, out);
   out->n_peel_rays = st[0];
@@ -903,6 +975,8 @@ extern "C" int thor_reweight(thor_ctx_t ctx, int64_t n, const float* X0, const f
   char* in = (char*)d_prm + ((pb + 255) & ~(size_t)255);
   const float *x0 = X0, *x = X, *c = col;
   const uint8_t* st = status;
+  // results through page-locked memory where they fit: scaled out of it in one pass
+  double* h_out = (double*)ctx->pinned(ob);
   int rc = ctx->cuda(cudaMemsetAsync(d_out, 0, ob, s), "clear reweight output");
   if (!rc) rc = ctx->cuda(cudaMemcpyAsync(d_prm, prm.data(), pb, cudaMemcpyHostToDevice, s), "reweight params");
   if (!rc && mem_kind == THOR_MEM_HOST) {
@@ -921,12 +995,14 @@ extern "C" int thor_reweight(thor_ctx_t ctx, int64_t n, const float* X0, const f
   rc = ctx->cuda(launch_reweight(n, x0, x, c, st, d_prm, n_targets, n_bins, X_min, X_max, d_out, ctx->sm_count, s),
                  "reweight kernel");
   cudaEventRecord(ctx->ev1, s);
-  if (!rc) rc = ctx->cuda(cudaMemcpyAsync(out, d_out, ob, cudaMemcpyDeviceToHost, s), "reweight output");
+  if (!rc)
+    rc = ctx->cuda(cudaMemcpyAsync(h_out ? h_out : out, d_out, ob, cudaMemcpyDeviceToHost, s), "reweight output");
   if (!rc) rc = ctx->cuda(cudaStreamSynchronize(s), "thor_reweight");
   if (rc) return rc;
   cudaEventElapsedTime(&ctx->last_ms, ctx->ev0, ctx->ev1);
   const double inv = 1.0 / (double)n;
-  for (size_t i = 0; i < (size_t)n_targets * (n_bins + 2); ++i) out[i] *= inv;
+  const double* from = h_out ? h_out : out;
+  for (size_t i = 0; i < (size_t)n_targets * (n_bins + 2); ++i) out[i] = from[i] * inv;
   ctx->last_error.clear();
   return THOR_OK;
 }

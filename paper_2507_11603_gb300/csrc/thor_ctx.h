@@ -24,7 +24,14 @@ struct thor_ctx {
   float last_ms = 0.0f;
   std::string last_error;
   // grow-only scratch buffers reused across calls
-  Buf b_models, b_tally, b_queue, b_spec, b_cube, b_raw, b_raw2, b_diag, b_stats, b_spill, b_cmp;
+  Buf b_run;                        // a run's record: queue, model, tally, counters, host spectrum
+  Buf b_cube, b_raw, b_raw2, b_diag, b_stats, b_spill, b_cmp;
+  // page-locked staging of small uploads and results (grow-only, at most kPinnedMax bytes)
+  static constexpr size_t kPinnedMax = (size_t)16 << 20;
+  void* h_pinned = nullptr;
+  size_t pinned_cap = 0;
+  // persistent grid sizes for the launch shape they were asked for (block 0: not yet)
+  struct GridSize { int block = 0, per_sm = 0, size = 0; } shell_size, grid_size;
   Buf b_stage[2];                   // host-input staging, double-buffered (forest)
   cudaStream_t copy_stream = nullptr;  // host<->device copies overlapped with kernels
   cudaEvent_t ev_copied[2] = {nullptr, nullptr}, ev_done[2] = {nullptr, nullptr};
@@ -47,6 +54,7 @@ struct thor_ctx {
   int cuda(cudaError_t e, const char* what);
   int select();
   void* scratch(Buf& b, size_t bytes);
+  void* pinned(size_t bytes);  // NULL beyond kPinnedMax or if it cannot be had
   ~thor_ctx();
 };
 
