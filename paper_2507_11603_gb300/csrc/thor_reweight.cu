@@ -53,6 +53,40 @@ struct TwoSum {
   }
 };
 
+// Few photons and targets: one CTA per 256 photons and target, weights added to an FP32 histogram
+// in shared memory.
+__global__ void __launch_bounds__(kRwThreads) reweight_few_kernel(int64_t n, const float* __restrict__ X0,
+                                                                  const float* __restrict__ X,
+                                                                  const float* __restrict__ col,
+                                                                  const uint8_t* __restrict__ status,
+                                                                  const float* __restrict__ params, int n_bins,
+                                                                  float X_min, float inv_dX, double* __restrict__ out) {
+  extern __shared__ float hist[];  // n_bins + 2
+  const int t = blockIdx.y;
+  for (int b = threadIdx.x; b < n_bins + 2; b += blockDim.x) hist[b] = 0.0f;
+  const Spectrum ps{params[0], params[1], params[2], params[3]};
+  const float* q = params + 5 * (t + 1);
+  const Spectrum pt{q[0], q[1], q[2], q[3]};
+  const float tau_d = q[4];
+  __syncthreads();
+  const int64_t i = (int64_t)blockIdx.x * kRwThreads + threadIdx.x;
+  if (i < n && status[i] == 1) {
+    const float x0 = X0[i];
+    const float s = pdf(ps, x0);
+    const float w = (s > 0.0f) ? __fmul_rn(__fdiv_rn(pdf(pt, x0), s), expf(-tau_d * col[i])) : 0.0f;
+    const float f = (X[i] - X_min) * inv_dX;
+    int b;
+    if (!(f >= 0.0f)) b = n_bins;
+    else if (f >= (float)n_bins) b = n_bins + 1;
+    else b = (int)f;
+    atomicAdd(&hist[b], w);
+  }
+  __syncthreads();
+  double* o = out + (size_t)t * (n_bins + 2);
+  for (int b = threadIdx.x; b < n_bins + 2; b += blockDim.x)
+    if (hist[b] != 0.0f) atomicAdd(&o[b], (double)hist[b]);
+}
+
 // chunk: photons per CTA (a power of two in [256, kRwChunk]).  A CTA of blockIdx.y handles the
 // target groups y, y + gridDim.y, ... of 2^group_log2 targets; its lanes split into
 // 32 / 2^group_log2 parts per warp, and warps beyond the groups into further parts.
@@ -151,6 +185,17 @@ __global__ void __launch_bounds__(kRwThreads) reweight_kernel(int64_t n, const f
 cudaError_t launch_reweight(int64_t n, const float* X0, const float* X, const float* col, const uint8_t* status,
                             const float* d_params, int n_targets, int n_bins, double X_min, double X_max,
                             double* d_out, int n_sm, cudaStream_t s) {
+  // Sorting a chunk costs a CTA some 8 us, whatever the targets: below about 2^21 photon-targets
+  // (of few photons; 3 * 2^18 of many, where an atomic per bin, target and 256 photons weighs
+  // more) a CTA per 256 photons and target is done earlier.  us, few / chunks, 300 bins: 5000 x 1
+  // 7 / 10, x 64 10 / 20, x 256 17 / 25; 2e4 x 64 16 / 24, x 256 44 / 43; 6e4 x 16 16 / 19, x 32
+  // 24 / 26, x 64 41 / 38; 2e5 x 2 18 / 24, x 4 27 / 26, x 8 36 / 28, x 256 747 / 181.
+  if (n * n_targets <= (n <= 65536 ? (int64_t)1 << 21 : (int64_t)3 << 18)) {
+    const dim3 grid((unsigned)((n + kRwThreads - 1) / kRwThreads), (unsigned)n_targets);
+    reweight_few_kernel<<<grid, kRwThreads, (size_t)(n_bins + 2) * sizeof(float), s>>>(
+        n, X0, X, col, status, d_params, n_bins, (float)X_min, (float)(n_bins / (X_max - X_min)), d_out);
+    return cudaGetLastError();
+  }
   // One target per lane: groups of 32 targets, or of the next power of two where there are
   // fewer (the lanes then split the records).
   int group_log2 = 0;

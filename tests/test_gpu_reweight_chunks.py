@@ -1,6 +1,6 @@
 """The reweighting kernel's chunks, target groups and bins against FP64, element by element (1e-5
 relative, as the other reweighting test): photon counts around the sorted chunks, target counts
-around the 32 lanes, one bin and the most bins, photons outside the range or not escaped."""
+around the 32 lanes, both sides of the line between the two kernels, one bin and the most bins, photons outside the range or not escaped."""
 import numpy as np
 import pytest
 
@@ -24,7 +24,9 @@ def ctx():
 
 
 @pytest.mark.parametrize("n,K,nb", [(1, 1, 1), (255, 2, 7), (256, 33, 50), (257, 31, 4096), (2047, 3, 100),
-                                    (2049, 64, 5), (70000, 5, 300), (70001, 300, 1), (400000, 40, 400)])
+                                    (2049, 64, 5), (70000, 5, 300), (70001, 300, 1), (400000, 40, 400),
+                                    (257, 8300, 40), (2047, 1030, 100), (2049, 1025, 5), (65536, 32, 60),
+                                    (65537, 33, 60)])
 def test_chunks_against_fp64(ctx, n, K, nb):
     rng = np.random.default_rng(n + K)
     X0 = rng.uniform(-2500.0, 2500.0, n).astype(np.float32)
