@@ -300,8 +300,8 @@ def run_shell_bench(args):
                               "pipelined_event_lanes": args.pipe_lanes if args.pipe_lanes >= 0 else 32,
                               "core_burst_lanes": args.burst_lanes if args.burst_lanes >= 0 else 1,
                               "tail_work_sharing": not args.no_tail_share}},
-        "e2e": {"value": e2e_value, "unit": "scatterings/s", "h2d_bytes_per_step": 256 + 48,
-                "d2h_bytes_per_step": (RUN["n_bins"] + 2) * 8 + 96, "steps": n_e2e,
+        "e2e": {"value": e2e_value, "unit": "scatterings/s", "h2d_bytes_per_step": 1536 + (RUN["n_bins"] + 2) * 8,
+                "d2h_bytes_per_step": (RUN["n_bins"] + 2) * 8 + 512, "steps": n_e2e,
                 "photon_ids": f"those of the first {n_e2e} timed steps",
                 "device_timed_value_same_steps": same_value},
         "gpu_launches": launches,
@@ -314,8 +314,8 @@ def run_shell_bench(args):
                      "simt_efficiency": simt,
                      "lane_frac": lane_achieved / (32.0 * peak_issue),
                      "lane_per_unit": f"{thread_inst_per_scat:g} thread instructions per scattering (ncu)",
-                     "lane_note": "the idle lanes of a cooperative burst form Philox blocks and evaluate throw-away "
-                                  "events; their instructions count as executed, so the lane figures overstate "
+                     "lane_note": "the idle lanes of a warp form the words of its packets' next events, of which some are "
+                                  "not used; their instructions count as executed, so the lane figures overstate "
                                   "useful lane work",
                      "tail": {"longest_photon_events": [c for c, _ in longest],
                               "lone_event_us": us_per_event, "lone_events_timed": lone_events,
@@ -673,11 +673,11 @@ def main():
                     help="events of the longest photon run alone to time the lone-lane event latency")
     ap.add_argument("--block", type=int, default=0)
     ap.add_argument("--pipe-lanes", type=int, default=-1,
-                    help="pipelined events in warps with at most this many live packets (-1 = library default)")
+                    help="core events in rounds in warps with at most this many live packets (-1 = library default)")
     ap.add_argument("--no-tail-share", action="store_true",
                     help="shell workload: no work sharing in the tail of the one-launch run")
     ap.add_argument("--burst-lanes", type=int, default=-1,
-                    help="core bursts in warps with at most this many live packets (-1 = library default)")
+                    help="deep rounds in warps with at most this many live packets (-1 = library default)")
     ap.add_argument("--blocks-per-sm", type=int, default=0)
     ap.add_argument("--inst-per-scat", type=float, default=365.0,
                     help="warp instructions per scattering of the shell photon loop (ncu, photons 0..19999 of the "

@@ -319,7 +319,7 @@ __device__ __forceinline__ float envelope_D(float xr, float a, float u0) {
 // Near-resonance split point (the x <= 2 rule): u0 = x - d, d = sqrt(a/(2 pi x)) e^{x^2/2},
 // clamped at 0; and q = a / d = sqrt(2 pi a x) e^{-x^2/2}, formed directly (no division).
 // Where u0 > 0 and q <= 1/20, w1 = atan2(a, x - u0) = atan(q) = q (1 - q^2/3 + q^4/5) to
-// 3e-9 relative.  The photon loops' core bursts use these same functions, so both evaluate
+// 3e-9 relative.  The photon loops' core rounds use these same functions, so both evaluate
 // an event identically.
 __device__ __forceinline__ float u0_core(float xr, float a) {
   const float d = sqrt_approx(a * (0.5f / kPiF)) * rsqrtf(xr) * exp_fast(fminf(0.5f * xr * xr, 80.0f));

@@ -417,9 +417,10 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
 // 64-byte slot.  The general event evaluates these events with the same helpers
 // (start_step, dust_channel, u0_core, upar_q / atan_small, upar_trial, x_after_scatter) on
 // the same words, so both paths give bit-identical results.
-// Measured (GB300, 2070 MHz): a photon alone in a static sphere 0.36 us per event (0.47 us
-// when its own lane formed the directions' angles and the words came by shuffle); the
-// expanding shell of 1e5 photons at N_HI = 1e20 3.29 s (5.35 s).  The general events run for
+// Measured (GB300, 2070 MHz): a photon alone in a static sphere 0.345 us per event (0.47 us
+// when its own lane formed the directions' angles and the words came by shuffle), at 1e3 K
+// 0.40 us (1.76 us); 5000 photons in a sphere of tau0 = 1e4 73 ms (107 ms); 1e5 photons in an
+// expanding shell of N_HI = 1e19 365 ms (576 ms), of 1e20 3.1 s (5.35 s).  The general events run for
 // all the packets that wait for one, at most once per `depth` core events: a general event
 // costs several core events, and one lane in sixty needs one at any time.
 constexpr int kChainSlots = kWordSlots;  // events per warp and round
