@@ -679,12 +679,12 @@ def main():
     ap.add_argument("--burst-lanes", type=int, default=-1,
                     help="deep rounds in warps with at most this many live packets (-1 = library default)")
     ap.add_argument("--blocks-per-sm", type=int, default=0)
-    ap.add_argument("--inst-per-scat", type=float, default=365.0,
+    ap.add_argument("--inst-per-scat", type=float, default=231.0,
                     help="warp instructions per scattering of the shell photon loop (ncu, photons 0..19999 of the "
                          "bench workload)")
-    ap.add_argument("--thread-inst-per-scat", type=float, default=9276.0,
+    ap.add_argument("--thread-inst-per-scat", type=float, default=6181.0,
                     help="thread instructions per scattering of the shell photon loop (ncu, same capture)")
-    ap.add_argument("--launch-dram-bytes", type=float, default=798976.0,
+    ap.add_argument("--launch-dram-bytes", type=float, default=1103872.0,
                     help="DRAM bytes read + written by one launch of the shell kernel (ncu, same capture; fixed per "
                          "launch: code, constants, tables)")
     ap.add_argument("--cpu-seconds", type=float, default=15.0)
