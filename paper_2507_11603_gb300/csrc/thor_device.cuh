@@ -135,8 +135,6 @@ struct Rng : StreamKey {
     keys(seed, pid);
     start_event(0u, nblk);
   }
-  // next interaction event of the photon
-  __device__ __forceinline__ void next_event(uint32_t nblk) { start_event(event + 1u, nblk); }
   __device__ __forceinline__ float u(int j) const { return uni32(v[j]); }
 };
 
