@@ -21,7 +21,9 @@
 //   near   the other cells (the core |x| < 6, the wing next to it, and the cells opposite the
 //          interval, where the nearest image changes side) are evaluated at each bin.
 // The node sums become Chebyshev coefficients once per interval and each bin evaluates them.
-// FP32 accumulation in two levels (blocks of 32 cells, then the running total).
+// FP32 accumulation in two levels (blocks of 32 cells, then the running total of the blocks in
+// order), whatever the number of sightlines of a call: a sightline has the same bits alone, in a
+// sub-range, in staged rows and in the whole box.
 #include "thor_device.cuh"
 #include "thor_internal.h"
 
@@ -45,6 +47,15 @@ constexpr float kFar = 2.25f;
 __device__ __forceinline__ float wing_tP(float a2, float x2) {
   const float t = rcp_approx(x2 + a2);
   return t * wing_g(t);
+}
+
+// Interval iv of 2^iv_log2 holds the bins whose centres lie in it: from first_bin(iv) to first_bin(iv + 1).
+__device__ __forceinline__ int first_bin(int iv, int iv_log2, int n_bins) {
+  return (2 * iv * n_bins + (1 << iv_log2) - 1) >> (iv_log2 + 1);
+}
+// The bin centre's velocity in fixed point.
+__device__ __forceinline__ uint32_t bin_fix(int b, double dv_bin, double to_fix) {
+  return (uint32_t)(unsigned long long)llrint(((double)b + 0.5) * dv_bin * to_fix);
 }
 
 struct ForestCells {
@@ -112,18 +123,28 @@ __device__ __forceinline__ float cheb_eval(const float* c, float xi) {  // Clens
 }
 
 // n_iv = 2^iv_log2 intervals; the CTA's blockIdx.y takes the iv_cta intervals from iv_cta
-// blockIdx.y on; `splits` warps share an interval's cells where there are fewer intervals
-// than warps.
+// blockIdx.y on.  Where there are fewer intervals than warps, `splits` warps share an interval's
+// blocks of 32 cells: kPartBlocks / iv_cta blocks of each interval at a time go to dynamic shared
+// memory, and their partial sums are added in order (all blocks of a chunk at once leave two
+// CTAs per SM instead of four: 60 sightlines of 1024 cells x 2048 bins 175 instead of 130 us).
+constexpr int kPartBlocks = 32;
+struct BlockSums {  // of one interval's bins and nodes (lanes 0-15 and 16-31 as node_terms has them)
+  float bins[kIvBins], nodes[32];
+};
+
+template <bool kSplit>
 __global__ void __launch_bounds__(kForestThreads, 4) forest_kernel(
     const float* __restrict__ nHI, const float* __restrict__ T, const float* __restrict__ vlos, int nx, int ny,
     int nz, int64_t first, double ds_cm, double dv_cell, int n_bins, double dv_bin, int iv_log2, int iv_cta,
     float* __restrict__ tau, const float* __restrict__ gK) {
   __shared__ __align__(16) float sK[THOR_VOIGT_NINT * THOR_VOIGT_NCOEF];
   __shared__ ForestCells sc;
-  __shared__ float sAcc[kMaxIv * kIvBins];       // direct sums: task, bin of the interval
-  __shared__ float sFine[kMaxIv * kNodes];       // node sums per task, then coefficients per interval
+  __shared__ float sAcc[kMaxIv * kIvBins];       // direct sums: interval, bin
+  __shared__ float sFine[kMaxIv * kNodes];       // node sums, then coefficients
   __shared__ float sCoarse[kCoarse][kNodes];     // node sums, then coefficients
   __shared__ float sCos[64];                     // cos(pi m / 32)
+  __shared__ uint32_t sV[kSplit ? kForestThreads : 1];
+  extern __shared__ BlockSums part[];
   load_ktab(sK, gK);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t sl = first + blockIdx.x;
@@ -134,23 +155,23 @@ __global__ void __launch_bounds__(kForestThreads, 4) forest_kernel(
   const double amp1 = THOR_SIG1 * ds_cm;
   const int64_t plane = (int64_t)nx * ny;
   const int n_iv = 1 << iv_log2, iv0 = blockIdx.y * iv_cta;
-  const int splits = iv_cta >= kForestWarps ? 1 : kForestWarps / iv_cta, n_task = iv_cta * splits;
+  const int splits = kSplit ? kForestWarps / iv_cta : 1, n_task = iv_cta * splits;
+  const int batch = kSplit ? kPartBlocks / iv_cta : kCellChunk / 32;  // blocks of 32 cells at a time
   const uint32_t h = iv_log2 ? 1u << (31 - iv_log2) : 0x80000000u;  // half-width of an interval
   const bool far_on = iv_log2 >= 3, coarse_on = iv_log2 >= 4;
   constexpr uint32_t hc = 0x80000000u / kCoarse;
   const int coarse_shift = iv_log2 - 3;
   if (tid < 64) sCos[tid] = cospif((float)tid / 32.0f);
-  for (int j = tid; j < kMaxIv * kIvBins; j += kForestThreads) sAcc[j] = 0.0f;
-  for (int j = tid; j < kMaxIv * kNodes; j += kForestThreads) sFine[j] = 0.0f;
+  for (int j = tid; j < iv_cta * kIvBins; j += kForestThreads) sAcc[j] = 0.0f;
+  for (int j = tid; j < iv_cta * kNodes; j += kForestThreads) sFine[j] = 0.0f;
   if (tid < kCoarse * kNodes) sCoarse[tid / kNodes][tid % kNodes] = 0.0f;
   __syncthreads();
   const float xi_node = sCos[2 * (lane & 15) + 1];
   const int32_t off_fine = __float2int_rn(xi_node * (float)h), off_coarse = __float2int_rn(xi_node * (float)hc);
-  auto first_bin = [&](int iv) { return (2 * iv * n_bins + n_iv - 1) >> (iv_log2 + 1); };  // centre at or after its start
-  auto bin_fix = [&](int b) {
-    return (uint32_t)(unsigned long long)llrint(((double)b + 0.5) * dv_bin * to_fix);
-  };
 
+  // kSplit: the bins' velocities (FP64 arithmetic) once for the warps that share an interval
+  if (kSplit && tid < iv_cta * kIvBins)
+    sV[tid] = bin_fix(first_bin(iv0 + tid / kIvBins, iv_log2, n_bins) + tid % kIvBins, dv_bin, to_fix);
   for (int k0 = 0; k0 < nz; k0 += kCellChunk) {
     const int nk = min(kCellChunk, nz - k0);
     __syncthreads();
@@ -185,41 +206,78 @@ __global__ void __launch_bounds__(kForestThreads, 4) forest_kernel(
         if (lane < kNodes) sCoarse[c][lane] += sum;
       }
     }
-    for (int task = warp; task < n_task; task += kForestWarps) {
-      const int iv = iv0 + task / splits, split = task % splits;
-      const uint32_t vc = (uint32_t)iv * (2u * h) + h;  // interval centre
-      const uint32_t vcc = (uint32_t)(iv >> (coarse_on ? coarse_shift : 0)) * (2u * hc) + hc;
-      const int b0 = first_bin(iv), nb = first_bin(iv + 1) - b0;
-      const uint32_t v0 = bin_fix(b0 + lane), v1 = bin_fix(b0 + lane + 32);
-      const bool two = nb > 32;
-      float acc0 = 0.0f, acc1 = 0.0f, sum = 0.0f;
-      for (int j0 = 32 * split; j0 < nk; j0 += 32 * splits) {
-        const int j = j0 + lane;
-        bool near = false, fine = false;
-        if (j < nk) {
-          const uint32_t vk = __float_as_uint(sc.p[j].x), core = sc.core[j];
-          const bool coarse = coarse_on && is_far(vcc - vk, hc, core);
-          fine = far_on && !coarse && is_far(vc - vk, h, core);
-          near = !fine && !coarse;
+    float acc = 0.0f, nodes = 0.0f;  // kSplit: totals of one bin per thread, one interval's nodes per warp
+    for (int jb = 0; jb < nk; jb += 32 * batch) {
+      const int je = min(nk, jb + 32 * batch);
+      for (int task = warp; task < n_task; task += kForestWarps) {
+        const int i = task / splits, iv = iv0 + i, split = task % splits;
+        const uint32_t vc = (uint32_t)iv * (2u * h) + h;  // interval centre
+        const uint32_t vcc = (uint32_t)(iv >> (coarse_on ? coarse_shift : 0)) * (2u * hc) + hc;
+        const int b0 = first_bin(iv, iv_log2, n_bins), nb = first_bin(iv + 1, iv_log2, n_bins) - b0;
+        const uint32_t v0 = kSplit ? sV[i * kIvBins + lane] : bin_fix(b0 + lane, dv_bin, to_fix);
+        const uint32_t v1 = kSplit ? sV[i * kIvBins + lane + 32] : bin_fix(b0 + lane + 32, dv_bin, to_fix);
+        const bool two = nb > 32;
+        float acc0 = 0.0f, acc1 = 0.0f, sum = 0.0f;
+        for (int j0 = jb + 32 * split; j0 < je; j0 += 32 * splits) {
+          const int j = j0 + lane;
+          bool near = false, fine = false;
+          if (j < nk) {
+            const uint32_t vk = __float_as_uint(sc.p[j].x), core = sc.core[j];
+            const bool coarse = coarse_on && is_far(vcc - vk, hc, core);
+            fine = far_on && !coarse && is_far(vc - vk, h, core);
+            near = !fine && !coarse;
+          }
+          unsigned mask = __ballot_sync(kFull, near);
+          const float node = node_terms(sc, j0, __ballot_sync(kFull, fine), vc + (uint32_t)off_fine, 0.0f);
+          float p0 = 0.0f, p1 = 0.0f;
+          while (mask) {
+            const int k = j0 + __ffs(mask) - 1;
+            mask &= mask - 1u;
+            const float4 c = sc.p[k];
+            const float2 am = sc.amp[k];
+            p0 = profile_at(v0, c, am, sK, p0);
+            if (two) p1 = profile_at(v1, c, am, sK, p1);
+          }
+          if (!kSplit) {
+            acc0 += p0;
+            acc1 += p1;
+            sum += node;
+          } else {
+            BlockSums& o = part[i * batch + ((j0 - jb) >> 5)];
+            o.bins[lane] = p0;
+            o.bins[lane + 32] = p1;
+            o.nodes[lane] = node;
+          }
         }
-        unsigned mask = __ballot_sync(kFull, near);
-        sum += node_terms(sc, j0, __ballot_sync(kFull, fine), vc + (uint32_t)off_fine, 0.0f);
-        float p0 = 0.0f, p1 = 0.0f;
-        while (mask) {
-          const int k = j0 + __ffs(mask) - 1;
-          mask &= mask - 1u;
-          const float4 c = sc.p[k];
-          const float2 am = sc.amp[k];
-          p0 = profile_at(v0, c, am, sK, p0);
-          if (two) p1 = profile_at(v1, c, am, sK, p1);
+        if (!kSplit) {
+          sum += __shfl_down_sync(kFull, sum, 16);
+          if (lane < kNodes) sFine[i * kNodes + lane] += sum;
+          sAcc[i * kIvBins + lane] += acc0;
+          sAcc[i * kIvBins + lane + 32] += acc1;
         }
-        acc0 += p0;
-        acc1 += p1;
       }
-      sum += __shfl_down_sync(kFull, sum, 16);
-      if (lane < kNodes) sFine[task * kNodes + lane] += sum;
-      sAcc[task * kIvBins + lane] += acc0;
-      sAcc[task * kIvBins + lane + 32] += acc1;
+      if (kSplit) {
+        __syncthreads();
+        const int n = (je - jb + 31) >> 5;
+        if (tid < iv_cta * kIvBins) {
+          const BlockSums* o = part + tid / kIvBins * batch;
+#pragma unroll 4
+          for (int b = 0; b < n; ++b) acc += o[b].bins[tid % kIvBins];
+        }
+        if (warp < iv_cta) {
+          const BlockSums* o = part + warp * batch;
+#pragma unroll 4
+          for (int b = 0; b < n; ++b) nodes += o[b].nodes[lane];
+        }
+        if (je < nk) __syncthreads();
+      }
+    }
+    if (kSplit) {
+      if (tid < iv_cta * kIvBins) sAcc[tid] += acc;
+      if (warp < iv_cta) {
+        nodes += __shfl_down_sync(kFull, nodes, 16);
+        if (lane < kNodes) sFine[warp * kNodes + lane] += nodes;
+      }
     }
   }
   __syncthreads();
@@ -233,15 +291,14 @@ __global__ void __launch_bounds__(kForestThreads, 4) forest_kernel(
   for (int i = warp; i < iv_cta; i += kForestWarps) {
     const int iv = iv0 + i;
     if (far_on) {
-      float f = 0.0f;
-      for (int s = 0; s < splits; ++s) f += sFine[(i * splits + s) * kNodes + (lane & 15)];
+      float f = sFine[i * kNodes + (lane & 15)];
       if (coarse_on) {
         const int c = iv >> coarse_shift;
         const uint32_t v = (uint32_t)iv * (2u * h) + h + (uint32_t)off_fine, vc = (uint32_t)c * (2u * hc) + hc;
         f += cheb_eval(sCoarse[c], (float)(int32_t)(v - vc) * (1.0f / (float)hc));
       }
       __syncwarp();
-      float* row = sFine + i * splits * kNodes;
+      float* row = sFine + i * kNodes;
       if (lane < kNodes) row[lane] = f;
       __syncwarp();
       const float c = cheb_coef(row, lane & 15, sCos);
@@ -249,13 +306,13 @@ __global__ void __launch_bounds__(kForestThreads, 4) forest_kernel(
       if (lane < kNodes) row[lane] = c;
       __syncwarp();
     }
-    const int b0 = first_bin(iv), nb = first_bin(iv + 1) - b0;
+    const int b0 = first_bin(iv, iv_log2, n_bins), nb = first_bin(iv + 1, iv_log2, n_bins) - b0;
     const uint32_t vc = (uint32_t)iv * (2u * h) + h;
     for (int q = lane; q < nb; q += 32) {
-      float t = 0.0f;
-      for (int s = 0; s < splits; ++s) t += sAcc[(i * splits + s) * kIvBins + q];
+      float t = sAcc[i * kIvBins + q];
       if (far_on)
-        t += cheb_eval(sFine + i * splits * kNodes, (float)(int32_t)(bin_fix(b0 + q) - vc) * (1.0f / (float)h));
+        t += cheb_eval(sFine + i * kNodes, (float)(int32_t)((kSplit ? sV[i * kIvBins + q] : bin_fix(b0 + q, dv_bin, to_fix)) - vc) *
+                                               (1.0f / (float)h));
       tau[(size_t)blockIdx.x * n_bins + b0 + q] = t;
     }
   }
@@ -278,10 +335,16 @@ cudaError_t launch_forest(const float* nHI, const float* T, const float* vlos, i
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   int iv_cta = 1 << iv_log2;
   while (iv_cta > 1 && count * ((1 << iv_log2) / iv_cta) < 2 * (int64_t)sms) iv_cta >>= 1;
+  const size_t part = iv_cta < kForestWarps ? kPartBlocks * sizeof(BlockSums) : 0;
+  if (part) {  // above the default limit together with the static part
+    const cudaError_t e = cudaFuncSetAttribute(forest_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)part);
+    if (e != cudaSuccess) return e;
+  }
   int64_t done = 0;
   while (done < count) {  // grid.x limit
     const int64_t n = count - done < (int64_t)0x7fffffff ? count - done : (int64_t)0x7fffffff;
-    forest_kernel<<<dim3((unsigned)n, (unsigned)((1 << iv_log2) / iv_cta)), kForestThreads, 0, s>>>(
+    (part ? forest_kernel<true> : forest_kernel<false>)<<<dim3((unsigned)n, (unsigned)((1 << iv_log2) / iv_cta)),
+                                                         kForestThreads, part, s>>>(
         nHI, T, vlos, nx, ny, nz, first + done, ds_cm, dv_cell, n_bins, dv_bin, iv_log2, iv_cta,
         tau + (size_t)done * n_bins, d_ktab);
     cudaError_t e = cudaGetLastError();
