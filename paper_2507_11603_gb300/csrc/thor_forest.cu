@@ -20,6 +20,8 @@
 //          rounding; all contributions are positive, so it is the same for the sum;
 //   near   the other cells (the core |x| < 6, the wing next to it, and the cells opposite the
 //          interval, where the nearest image changes side) are evaluated at each bin.
+// A chunk of cells most of whose pairs are near (hot gas, or a box narrower than some 12 Doppler
+// widths) is evaluated at every bin without sorting its cells (kDirect).
 // The node sums become Chebyshev coefficients once per interval and each bin evaluates them.
 // FP32 accumulation in two levels (blocks of 32 cells, then the running total of the blocks in
 // order), whatever the number of sightlines of a call: a sightline has the same bits alone, in a
@@ -40,6 +42,11 @@ constexpr int kMaxIv = kMaxBins / kIvBins;
 constexpr int kCoarse = 8;        // coarse intervals
 constexpr int kNodes = 16;        // Chebyshev nodes per interval
 constexpr float kFar = 2.25f;
+// Share of near pairs from which on a chunk is evaluated directly, all its cells at up to eight
+// bins per lane.  Sorted, a near pair costs some 14% more (one read of the cell per two bins, the
+// walk through the mask), a far pair about a quarter.  2048 sightlines of 1024 cells x 2048 bins,
+// ms, sorted / direct: cells around 1e6 K 4.6 / 4.8, 2e6 K 5.7 / 5.4, 1e7 K 7.6 / 6.7.
+constexpr float kDirect = 0.6f;
 
 // Wing (|x| >= 6) without the a/sqrt(pi) factor: t g(t), t = 1/(x^2 + a^2), g the
 // degree-4 fit of thor_device.cuh (one polynomial for the whole wing, no branch).  MUFU
@@ -53,6 +60,9 @@ __device__ __forceinline__ float wing_tP(float a2, float x2) {
 __device__ __forceinline__ int first_bin(int iv, int iv_log2, int n_bins) {
   return (2 * iv * n_bins + (1 << iv_log2) - 1) >> (iv_log2 + 1);
 }
+__device__ __forceinline__ int interval_of(int b, int iv_log2, int n_bins) {
+  return ((2 * b + 1) << iv_log2) / (2 * n_bins);
+}
 // The bin centre's velocity in fixed point.
 __device__ __forceinline__ uint32_t bin_fix(int b, double dv_bin, double to_fix) {
   return (uint32_t)(unsigned long long)llrint(((double)b + 0.5) * dv_bin * to_fix);
@@ -64,12 +74,15 @@ struct ForestCells {
   uint32_t core[kCellChunk];   // |x| = 6 in fixed point, rounded up; 2^32 - 1: always near
 };
 
+// Distance from an interval's centre (half-width h) from which on a cell is far.
+__device__ __forceinline__ uint32_t far_from(uint32_t h, uint32_t core) {
+  return max((uint32_t)(kFar * (float)h), core + min(h, ~core));
+}
 // A cell's line centre d from an interval's centre (fixed point, wrapped), half-width h: far?
 // The interval must also lie on one side of the cell's antipode (nearest image).
 __device__ __forceinline__ bool is_far(uint32_t d, uint32_t h, uint32_t core) {
   const uint32_t ad = (d & 0x80000000u) ? 0u - d : d;
-  const uint32_t lim = max((uint32_t)(kFar * (float)h), core + min(h, ~core));
-  return ad >= lim && ad <= 0x80000000u - h - 2u;
+  return ad >= far_from(h, core) && ad <= 0x80000000u - h - 2u;
 }
 
 // One wing term at a node or bin at fixed-point velocity v.
@@ -101,6 +114,60 @@ __device__ __forceinline__ float node_terms(const ForestCells& sc, int j0, unsig
     sum += on ? w : 0.0f;
   }
   return sum;
+}
+
+// Cells [0, nk) at N bins per lane (v[q]), in the order of the near cells' sums: blocks of 32
+// cells, then the blocks.
+template <int N>
+__device__ __forceinline__ void direct_terms(const ForestCells& sc, int nk, const float* sK, const uint32_t (&v)[8],
+                                             float (&acc)[8]) {
+#pragma unroll 1
+  for (int j0 = 0; j0 < nk; j0 += 32) {
+    const int je = min(nk, j0 + 32);
+    float p[N];
+#pragma unroll
+    for (int q = 0; q < N; ++q) p[q] = 0.0f;
+#pragma unroll 4
+    for (int j = j0; j < je; ++j) {
+      const float4 c = sc.p[j];
+      const float2 am = sc.amp[j];
+#pragma unroll
+      for (int q = 0; q < N; ++q) p[q] = profile_at(v[q], c, am, sK, p[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < N; ++q) acc[q] += p[q];
+  }
+}
+
+// The chunk's cells at all bins of the CTA (intervals iv0 .. iv0 + iv_cta), added to sAcc.  Out of
+// line, so that the interval code keeps its registers (inlined, cold boxes took 3% longer).
+__device__ __noinline__ void direct_chunk(const ForestCells* sc, int nk, const float* sK, float* sAcc, int iv0,
+                                          int iv_cta, int iv_log2, int n_bins, double dv_bin, double to_fix) {
+  __builtin_assume(__isShared(sc));
+  __builtin_assume(__isShared(sK));
+  __builtin_assume(__isShared(sAcc));
+  const int b0 = first_bin(iv0, iv_log2, n_bins), nb = first_bin(iv0 + iv_cta, iv_log2, n_bins) - b0;
+  const int n = (nb + kForestThreads - 1) / kForestThreads;  // bins per lane: 1 to 8
+  uint32_t v[8];
+  float acc[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    v[q] = q < n ? bin_fix(b0 + q * kForestThreads + (int)threadIdx.x, dv_bin, to_fix) : 0u;
+    acc[q] = 0.0f;
+  }
+  if (n > 6) direct_terms<8>(*sc, nk, sK, v, acc);
+  else if (n > 4) direct_terms<6>(*sc, nk, sK, v, acc);
+  else if (n > 2) direct_terms<4>(*sc, nk, sK, v, acc);
+  else if (n == 2) direct_terms<2>(*sc, nk, sK, v, acc);
+  else if ((int)(threadIdx.x & ~31u) < nb) direct_terms<1>(*sc, nk, sK, v, acc);
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int b = q * kForestThreads + (int)threadIdx.x;
+    if (b < nb) {
+      const int iv = interval_of(b0 + b, iv_log2, n_bins);
+      sAcc[(iv - iv0) * kIvBins + b0 + b - first_bin(iv, iv_log2, n_bins)] += acc[q];
+    }
+  }
 }
 
 // Chebyshev coefficient k of node values f: (2/16) sum_n f_n cos(k pi (n + 1/2) / 16).
@@ -174,6 +241,7 @@ __global__ void __launch_bounds__(kForestThreads, 4) forest_kernel(
     sV[tid] = bin_fix(first_bin(iv0 + tid / kIvBins, iv_log2, n_bins) + tid % kIvBins, dv_bin, to_fix);
   for (int k0 = 0; k0 < nz; k0 += kCellChunk) {
     const int nk = min(kCellChunk, nz - k0);
+    uint32_t near_sum = 0u, cells = 0u;  // near share of this thread's pairs, 2^-16 each
     __syncthreads();
     for (int j = tid; j < nk; j += kForestThreads) {
       const int64_t c = (int64_t)(k0 + j) * plane + (int64_t)iy * nx + ix;
@@ -189,9 +257,17 @@ __global__ void __launch_bounds__(kForestThreads, 4) forest_kernel(
       // the plain sum
       const float w = __fdividef(6.00002f, iv);
       sc.core[j] = (w < 2.0e9f && w > 0.0f && fabsf(ampw) < 1e30f) ? (uint32_t)w + 2u : 0xffffffffu;
+      near_sum += min((min(far_from(h, sc.core[j]), 0x80000000u) >> 15) + (h >> 15), 65536u);
+      ++cells;
     }
-    __syncthreads();
-    if (coarse_on) {  // one coarse interval per warp
+    // (every CTA of a sightline decides alike: the votes are over all its cells)
+    const int votes = __syncthreads_count(far_on && cells && (float)near_sum >= kDirect * 65536.0f * (float)cells);
+    const bool direct = 2 * votes > min(nk, kForestThreads);
+    if (!kSplit && direct) {
+      direct_chunk(&sc, nk, sK, sAcc, iv0, iv_cta, iv_log2, n_bins, dv_bin, to_fix);
+      continue;
+    }
+    if (coarse_on && !direct) {  // one coarse interval per warp
       const int c = warp;
       if ((((c + 1) << coarse_shift) > iv0) && ((c << coarse_shift) < iv0 + iv_cta)) {
         const uint32_t vc = (uint32_t)c * (2u * hc) + hc;
@@ -223,8 +299,8 @@ __global__ void __launch_bounds__(kForestThreads, 4) forest_kernel(
           bool near = false, fine = false;
           if (j < nk) {
             const uint32_t vk = __float_as_uint(sc.p[j].x), core = sc.core[j];
-            const bool coarse = coarse_on && is_far(vcc - vk, hc, core);
-            fine = far_on && !coarse && is_far(vc - vk, h, core);
+            const bool coarse = coarse_on && !direct && is_far(vcc - vk, hc, core);
+            fine = far_on && !direct && !coarse && is_far(vc - vk, h, core);
             near = !fine && !coarse;
           }
           unsigned mask = __ballot_sync(kFull, near);
