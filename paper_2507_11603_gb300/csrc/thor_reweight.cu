@@ -13,6 +13,8 @@
 // the photons, shared FP32 atomics are compare-and-swap loops, and each CTA ended with an
 // atomic per occupied bin, 38e6 of them.)  Weights add in FP32 over blocks of 256 photons and
 // in two-float arithmetic (error-free sums) above that.
+#include <algorithm>
+
 #include "thor_internal.h"
 
 namespace thor {
@@ -53,6 +55,17 @@ struct TwoSum {
   }
 };
 
+// A photon's weight for a target, and its bin (n_bins: below the range, n_bins + 1: above).
+__device__ __forceinline__ float weight(const Spectrum& ps, const Spectrum& pt, float tau_d, float x0, float col) {
+  const float s = pdf(ps, x0);
+  return (s > 0.0f) ? __fmul_rn(__fdiv_rn(pdf(pt, x0), s), expf(-tau_d * col)) : 0.0f;
+}
+__device__ __forceinline__ int bin_of(float X, float X_min, float inv_dX, int n_bins) {
+  const float f = (X - X_min) * inv_dX;
+  if (!(f >= 0.0f)) return n_bins;
+  return f >= (float)n_bins ? n_bins + 1 : (int)f;
+}
+
 // Few photons and targets: one CTA per 256 photons and target, weights added to an FP32 histogram
 // in shared memory.
 __global__ void __launch_bounds__(kRwThreads) reweight_few_kernel(int64_t n, const float* __restrict__ X0,
@@ -70,21 +83,64 @@ __global__ void __launch_bounds__(kRwThreads) reweight_few_kernel(int64_t n, con
   const float tau_d = q[4];
   __syncthreads();
   const int64_t i = (int64_t)blockIdx.x * kRwThreads + threadIdx.x;
-  if (i < n && status[i] == 1) {
-    const float x0 = X0[i];
-    const float s = pdf(ps, x0);
-    const float w = (s > 0.0f) ? __fmul_rn(__fdiv_rn(pdf(pt, x0), s), expf(-tau_d * col[i])) : 0.0f;
-    const float f = (X[i] - X_min) * inv_dX;
-    int b;
-    if (!(f >= 0.0f)) b = n_bins;
-    else if (f >= (float)n_bins) b = n_bins + 1;
-    else b = (int)f;
-    atomicAdd(&hist[b], w);
-  }
+  if (i < n && status[i] == 1)
+    atomicAdd(&hist[bin_of(X[i], X_min, inv_dX, n_bins)], weight(ps, pt, tau_d, X0[i], col[i]));
   __syncthreads();
   double* o = out + (size_t)t * (n_bins + 2);
   for (int b = threadIdx.x; b < n_bins + 2; b += blockDim.x)
     if (hist[b] != 0.0f) atomicAdd(&o[b], (double)hist[b]);
+}
+
+// Many photons, few targets: a CTA strides through the photons for one target.  Up to kFoldBins
+// bins the weights add in FP32 and each bin's sum moves to FP64 after 256 photons (up to four
+// times as many where they spread over more than 16 bins); with more bins that would cost more
+// than the photons, and they are spread enough to add in FP64 at once (a compare-and-swap loop as
+// in FP32, which few bins make slow: 1e7 photons, 50 bins 160 us, 84 with FP32 sums).
+constexpr int kFoldBins = 1022;
+template <bool kWide>
+__global__ void __launch_bounds__(kRwThreads) reweight_long_kernel(int64_t n, const float* __restrict__ X0,
+                                                                   const float* __restrict__ X,
+                                                                   const float* __restrict__ col,
+                                                                   const uint8_t* __restrict__ status,
+                                                                   const float* __restrict__ params, int n_bins,
+                                                                   float X_min, float inv_dX, double* __restrict__ out) {
+  extern __shared__ double sum[];  // n_bins + 2, and as many FP32 sums behind them
+  float* hist = reinterpret_cast<float*>(sum + n_bins + 2);
+  const int t = blockIdx.y;
+  for (int b = threadIdx.x; b < n_bins + 2; b += blockDim.x) {
+    sum[b] = 0.0;
+    if (!kWide) hist[b] = 0.0f;
+  }
+  const Spectrum ps{params[0], params[1], params[2], params[3]};
+  const float* q = params + 5 * (t + 1);
+  const Spectrum pt{q[0], q[1], q[2], q[3]};
+  const float tau_d = q[4];
+  __syncthreads();
+  auto fold = [&]() {
+    __syncthreads();
+    for (int b = threadIdx.x; b < n_bins + 2; b += blockDim.x) {
+      const float v = hist[b];
+      if (v != 0.0f) { sum[b] += (double)v; hist[b] = 0.0f; }
+    }
+    __syncthreads();
+  };
+  const int most = min(max(n_bins / 16, 1), 4);
+  int rounds = 0;
+  for (int64_t base = (int64_t)blockIdx.x * kRwThreads; base < n; base += (int64_t)gridDim.x * kRwThreads) {
+    const int64_t i = base + threadIdx.x;
+    if (i < n && status[i] == 1) {
+      const float w = weight(ps, pt, tau_d, X0[i], col[i]);
+      const int b = bin_of(X[i], X_min, inv_dX, n_bins);
+      if (kWide) atomicAdd(&sum[b], (double)w);
+      else atomicAdd(&hist[b], w);
+    }
+    if (!kWide && ++rounds == most) { fold(); rounds = 0; }
+  }
+  if (!kWide) fold();
+  else __syncthreads();
+  double* o = out + (size_t)t * (n_bins + 2);
+  for (int b = threadIdx.x; b < n_bins + 2; b += blockDim.x)
+    if (sum[b] != 0.0) atomicAdd(&o[b], sum[b]);
 }
 
 // chunk: photons per CTA (a power of two in [256, kRwChunk]).  A CTA of blockIdx.y handles the
@@ -115,12 +171,7 @@ __global__ void __launch_bounds__(kRwThreads) reweight_kernel(int64_t n, const f
     for (int j = tid; j < chunk; j += kRwThreads) {
       uint32_t k = kRwNone;
       if (base + j < n && status[base + j] == 1) {
-        const float f = (X[base + j] - X_min) * inv_dX;
-        int b;
-        if (!(f >= 0.0f)) b = n_bins;
-        else if (f >= (float)n_bins) b = n_bins + 1;
-        else b = (int)f;
-        k = ((uint32_t)b << 11) | (uint32_t)j;
+        k = ((uint32_t)bin_of(X[base + j], X_min, inv_dX, n_bins) << 11) | (uint32_t)j;
         ++valid;
       }
       key[j] = k;
@@ -185,15 +236,43 @@ __global__ void __launch_bounds__(kRwThreads) reweight_kernel(int64_t n, const f
 cudaError_t launch_reweight(int64_t n, const float* X0, const float* X, const float* col, const uint8_t* status,
                             const float* d_params, int n_targets, int n_bins, double X_min, double X_max,
                             double* d_out, int n_sm, cudaStream_t s) {
-  // Sorting a chunk costs a CTA some 8 us, whatever the targets: below about 2^21 photon-targets
-  // (of few photons; 3 * 2^18 of many, where an atomic per bin, target and 256 photons weighs
-  // more) a CTA per 256 photons and target is done earlier.  us, few / chunks, 300 bins: 5000 x 1
-  // 7 / 10, x 64 10 / 20, x 256 17 / 25; 2e4 x 64 16 / 24, x 256 44 / 43; 6e4 x 16 16 / 19, x 32
-  // 24 / 26, x 64 41 / 38; 2e5 x 2 18 / 24, x 4 27 / 26, x 8 36 / 28, x 256 747 / 181.
-  if (n * n_targets <= (n <= 65536 ? (int64_t)1 << 21 : (int64_t)3 << 18)) {
+  const float lo = (float)X_min, inv = (float)(n_bins / (X_max - X_min));
+  const bool wide = n_bins > kFoldBins;
+  // Sorting a chunk costs a CTA some 8 us, whatever the targets: up to some 2^21 photon-targets
+  // (of few photons; less of many, where an atomic per bin, target and 256 photons weighs more) a
+  // CTA per 256 photons and target is done earlier.  us, few / chunks, 300 bins: 5000 x 1 7 / 10,
+  // x 64 10 / 20, x 256 17 / 25; 2e4 x 64 16 / 24, x 256 44 / 43; 6e4 x 16 16 / 19, x 32 24 / 26,
+  // x 64 41 / 38; 2e5 x 2 18 / 24, x 4 24 / 26, x 8 36 / 28, x 256 747 / 181; 50 bins: 6e4 x 36
+  // 25 / 28, x 50 32 / 29; 2e5 x 5 23 / 33; 4000 bins: 2e5 x 4 26 / 20.
+  const int64_t few = n <= 1 << 16   ? (n_bins < 100 ? (int64_t)1 << 21 : (int64_t)3 << 20)
+                      : n <= 1 << 18 ? (wide ? (int64_t)3 << 18 : (int64_t)1 << 20)
+                                     : n <= 1 << 19 ? (int64_t)3 << 18 : 0;
+  if (n * n_targets <= few) {
     const dim3 grid((unsigned)((n + kRwThreads - 1) / kRwThreads), (unsigned)n_targets);
-    reweight_few_kernel<<<grid, kRwThreads, (size_t)(n_bins + 2) * sizeof(float), s>>>(
-        n, X0, X, col, status, d_params, n_bins, (float)X_min, (float)(n_bins / (X_max - X_min)), d_out);
+    reweight_few_kernel<<<grid, kRwThreads, (size_t)(n_bins + 2) * sizeof(float), s>>>(n, X0, X, col, status, d_params,
+                                                                                       n_bins, lo, inv, d_out);
+    return cudaGetLastError();
+  }
+  // Many photons, few targets: sorting a photon costs more than its few weights.  us, chunks /
+  // striding CTAs: 50 bins, 1e7 x 1 446 / 84, x 3 444 / 232, x 6 462 / 448, x 8 460 / 594; 3e5 x 4
+  // 49 / 30; 400 bins, 3e5 x 3 32 / 35, x 4 32 / 38, 1e6 x 4 74 / 66; 4000 bins, 1e6 x 3 80 / 59,
+  // x 4 81 / 81, 1e7 x 6 672 / 523.  With fewer bins a chunk's sums collide more (4 bins, 3e5 x 4
+  // 102 / 26), but the FP32 sums move to FP64 after every 256 photons (10 bins, 3e6 x 6 185 / 153,
+  // 1e7 x 4 573 / 426, x 5 462 / 530), and with one or two bins the shared sums collide (1 bin, 1e7
+  // x 3 679 / 1117).
+  const bool many = n >= 1 << 20;
+  const int strided = n_bins < 4      ? 2
+                      : n_bins < 32   ? (!many ? 8 : n < 1 << 22 ? 6 : 4)
+                      : n_bins <= 100 ? 6
+                      : !wide         ? (many ? 6 : 3)
+                                      : (n >= 1 << 21 ? 6 : many ? 3 : 2);
+  if (n_targets <= strided) {
+    const size_t smem = (size_t)(n_bins + 2) * (wide ? 8 : 12);
+    const int64_t want = (n + kRwThreads - 1) / kRwThreads;
+    const int64_t cap = n_sm * std::min<int64_t>(8, (200 << 10) / smem);  // resident CTAs
+    (wide ? reweight_long_kernel<true> : reweight_long_kernel<false>)<<<
+        dim3((unsigned)std::min(want, cap), (unsigned)n_targets), kRwThreads, smem, s>>>(n, X0, X, col, status, d_params,
+                                                                                         n_bins, lo, inv, d_out);
     return cudaGetLastError();
   }
   // One target per lane: groups of 32 targets, or of the next power of two where there are
@@ -211,8 +290,8 @@ cudaError_t launch_reweight(int64_t n, const float* X0, const float* X, const fl
   int64_t gy = (4 * (int64_t)n_sm + gx - 1) / gx;
   if (gy > n_groups) gy = n_groups;
   const dim3 grid((unsigned)gx, (unsigned)gy);
-  reweight_kernel<<<grid, kRwThreads, 0, s>>>(n, X0, X, col, status, d_params, n_targets, group_log2, chunk, n_bins,
-                                              (float)X_min, (float)(n_bins / (X_max - X_min)), d_out);
+  reweight_kernel<<<grid, kRwThreads, 0, s>>>(n, X0, X, col, status, d_params, n_targets, group_log2, chunk, n_bins, lo,
+                                              inv, d_out);
   return cudaGetLastError();
 }
 
