@@ -191,8 +191,8 @@ __device__ __forceinline__ float cheb_eval(const float* c, float xi) {  // Clens
 
 // n_iv = 2^iv_log2 intervals; the CTA's blockIdx.y takes the iv_cta intervals from iv_cta
 // blockIdx.y on.  Where there are fewer intervals than warps, `splits` warps share an interval's
-// blocks of 32 cells: kPartBlocks / iv_cta blocks of each interval at a time go to dynamic shared
-// memory, and their partial sums are added in order (all blocks of a chunk at once leave two
+// blocks of 32 cells: kPartBlocks / iv_cta blocks of each interval at a time go to shared memory
+// (`part`), and their partial sums are added in order (all blocks of a chunk at once leave two
 // CTAs per SM instead of four: 60 sightlines of 1024 cells x 2048 bins 175 instead of 130 us).
 constexpr int kPartBlocks = 32;
 struct BlockSums {  // of one interval's bins and nodes (lanes 0-15 and 16-31 as node_terms has them)
@@ -206,12 +206,13 @@ __global__ void __launch_bounds__(kForestThreads, 4) forest_kernel(
     float* __restrict__ tau, const float* __restrict__ gK) {
   __shared__ __align__(16) float sK[THOR_VOIGT_NINT * THOR_VOIGT_NCOEF];
   __shared__ ForestCells sc;
-  __shared__ float sAcc[kMaxIv * kIvBins];       // direct sums: interval, bin
-  __shared__ float sFine[kMaxIv * kNodes];       // node sums, then coefficients
+  constexpr int kIv = kSplit ? kForestWarps / 2 : kMaxIv;
+  __shared__ float sAcc[kIv * kIvBins];          // direct sums: interval, bin
+  __shared__ float sFine[kIv * kNodes];          // node sums, then coefficients
   __shared__ float sCoarse[kCoarse][kNodes];     // node sums, then coefficients
   __shared__ float sCos[64];                     // cos(pi m / 32)
-  __shared__ uint32_t sV[kSplit ? kForestThreads : 1];
-  extern __shared__ BlockSums part[];
+  __shared__ uint32_t sV[kSplit ? kIv * kIvBins : 1];
+  __shared__ BlockSums part[kSplit ? kPartBlocks : 1];
   load_ktab(sK, gK);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t sl = first + blockIdx.x;
@@ -411,16 +412,11 @@ cudaError_t launch_forest(const float* nHI, const float* T, const float* vlos, i
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   int iv_cta = 1 << iv_log2;
   while (iv_cta > 1 && count * ((1 << iv_log2) / iv_cta) < 2 * (int64_t)sms) iv_cta >>= 1;
-  const size_t part = iv_cta < kForestWarps ? kPartBlocks * sizeof(BlockSums) : 0;
-  if (part) {  // above the default limit together with the static part
-    const cudaError_t e = cudaFuncSetAttribute(forest_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)part);
-    if (e != cudaSuccess) return e;
-  }
   int64_t done = 0;
   while (done < count) {  // grid.x limit
     const int64_t n = count - done < (int64_t)0x7fffffff ? count - done : (int64_t)0x7fffffff;
-    (part ? forest_kernel<true> : forest_kernel<false>)<<<dim3((unsigned)n, (unsigned)((1 << iv_log2) / iv_cta)),
-                                                         kForestThreads, part, s>>>(
+    (iv_cta < kForestWarps ? forest_kernel<true> : forest_kernel<false>)<<<dim3((unsigned)n, (unsigned)((1 << iv_log2) / iv_cta)),
+                                                         kForestThreads, 0, s>>>(
         nHI, T, vlos, nx, ny, nz, first + done, ds_cm, dv_cell, n_bins, dv_bin, iv_log2, iv_cta,
         tau + (size_t)done * n_bins, d_ktab);
     cudaError_t e = cudaGetLastError();
