@@ -427,6 +427,12 @@ constexpr int kChainSlots = kWordSlots;  // events per warp and round
 constexpr uint32_t kChainDepth = 32;  // ... and per packet, in warps with few packets
 constexpr uint32_t kCrowdDepth = 16;  // ... and per packet, in the others (kept until a general event runs)
 constexpr uint32_t kFirstDepth = 4;   // ... at first: doubled where a round runs full, halved where it mostly does not
+// ... and in a served warp while another packet waits for a general event: the packets of a warp
+// belong to several requests there, and with 16 core events to each general one a thin request's
+// packets got one event in 17 of those a round is charged.  256 requests of up to N_HI = 1e21, 28
+// per second: p50 32 -> 24 ms, p90 520 -> 432 ms, all at once no slower (64 requests 2.50 -> 2.42 s;
+// depth 2 the same, 1 2.78 s, 8 2.51 s).
+constexpr uint32_t kSharedDepth = 4;
 constexpr uint32_t kVoteEvents = 4;   // core events between two votes on whether any packet goes on
 __device__ __forceinline__ void form_words(const ShellModel& m, const Photon& ph, WordBuf& wb, bool mine, int D,
                                            WordPos& at) {
@@ -1200,7 +1206,11 @@ __global__ void __launch_bounds__(256, 1) shell_slice_kernel(const ShellModel* _
     do {
       fin = false;
       bool general = active;
-      const uint32_t most = min(n_live <= kChainSlots / (int)kChainDepth ? kChainDepth : kCrowdDepth, budget - ev);
+      const bool waiting = __any_sync(kFull, active && !(chain && chain_kind(mr, ph)));
+      const uint32_t most = min(waiting                                       ? kSharedDepth
+                                : n_live <= kChainSlots / (int)kChainDepth ? kChainDepth
+                                                                           : kCrowdDepth,
+                                budget - ev);
       WordPos at;
       uint32_t n = core_events(mr, ph, wb, active && chain, depth, most, general, at);
       if (kMixed) general = general || (active && !chain);
