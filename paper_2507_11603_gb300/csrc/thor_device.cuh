@@ -694,7 +694,7 @@ __device__ __forceinline__ float scatter_resonant(float x, float a, int phase, f
   const bool core = fabsf(x - upar) < 0.2f;
   if (phase == PH_MIXED && core && w.mixed < (1.0f / 3.0f)) {
     mu = __fmaf_rn(2.0f, w.Rm, -1.0f);
-    st = sqrt_approx(fmaxf(0.0f, 1.0f - mu * mu));
+    st = sqrt_approx(fmaxf(0.0f, mul_add(-mu, mu, 1.0f)));
     ko = turn<kFormIso>(k, e1, e2, mu, st, w.cp, w.sp);
   }
   if (af) { af->upar = upar; af->u1 = u1; af->u2 = u2; af->e1 = e1; af->e2 = e2; af->core = core; }
@@ -712,7 +712,7 @@ __device__ __forceinline__ void scatter_dust(float g, float3& k, float Rm, float
   const float mu = mu_hg(Rm, g);
   float3 e1, e2;
   basis(k.x, k.y, k.z, e1, e2);
-  const float st = sqrtf(fmaxf(0.0f, 1.0f - mu * mu));
+  const float st = sqrtf(fmaxf(0.0f, mul_add(-mu, mu, 1.0f)));
   k = turn<kTurnShell>(k, e1, e2, mu, st, cp, sp);
 }
 __device__ __forceinline__ void scatter_dust(float g, float3& k, const Rng& rng) {

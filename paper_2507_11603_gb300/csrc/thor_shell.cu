@@ -241,7 +241,7 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
       const double s = -b + sqrt(fmax(__fma_rn(b, b, -c), 0.0));
       ph.px = __fma_rn(s, kx, ph.px); ph.py = __fma_rn(s, ky, ph.py); ph.pz = __fma_rn(s, kz, ph.pz);
       ph.region = 0;
-      ph.x = (ph.X - m.vgrad * (float)(b + s)) * m.inv_vth;
+      ph.x = __fmul_rn(__fmaf_rn(-m.vgrad, (float)(b + s), ph.X), m.inv_vth);
       ph.safe = 0.0f;
     }
     // ---- fast path: the next (sub-)step lies inside the safety ball
@@ -272,22 +272,22 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
         break;
       }
       const float ds = m.ds_core;
-      const float xm = ph.x - m.gam * 0.5f * ds;
+      const float xm = __fmaf_rn(-__fmul_rn(m.gam, 0.5f), ds, ph.x);
       const float kap = __fmaf_rn(m.kap0, voigt<false>(m.a, xm, Ktab), m.kapd);
-      const float dtau = kap * ds;
+      const float dtau = __fmul_rn(kap, ds);
       ++ph.steps;
       if (dtau >= tau_rem) {
         const float s = __fdividef(tau_rem, kap);
         advance(ph, s);
         ph.safe = __fmaf_rd(-s, 1.000001f, ph.safe);
-        x_site = ph.x - m.gam * s;
-        kH = m.kap0 * voigt<false>(m.a, x_site, Ktab);
+        x_site = __fmaf_rn(-m.gam, s, ph.x);
+        kH = __fmul_rn(m.kap0, voigt<false>(m.a, x_site, Ktab));
         break;
       }
-      tau_rem -= dtau;
+      tau_rem = __fsub_rn(tau_rem, dtau);
       advance(ph, ds);
       ph.safe = __fmaf_rd(-ds, 1.000001f, ph.safe);
-      ph.x -= m.gam * ds;
+      ph.x = __fsub_rn(ph.x, __fmul_rn(m.gam, ds));
       if (--turn_steps <= 0) {
         ph.fly = kFlyBall; ph.fly_tau = tau_rem;
         return -1;
@@ -309,9 +309,9 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
     if (m.gam == 0.0f) {
       S = ShellSegment::exact(m, b, pp, next);
       Sf = (float)S;
-      const float kap = kH + m.kapd;
-      if (kap * Sf >= tau_rem) s_star = fminf(tau_rem / kap, Sf);
-      else tau_rem -= kap * Sf;
+      const float kap = __fadd_rn(kH, m.kapd), t = __fmul_rn(kap, Sf);
+      if (t >= tau_rem) s_star = fminf(__fdiv_rn(tau_rem, kap), Sf);
+      else tau_rem = __fsub_rn(tau_rem, t);
     } else {
       float s = fmaxf(s_seg, 0.0f);
       s_seg = kFlyNone;
@@ -332,16 +332,16 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
           if (!(s < Sf)) break;
           s1 = fminf(Sf, s1);
         }
-        const float xm = x0 - m.gam * 0.5f * (s + s1);
+        const float xm = __fmaf_rn(-__fmul_rn(m.gam, 0.5f), s + s1, x0);
         const float kap = __fmaf_rn(m.kap0, voigt<false>(m.a, xm, Ktab), m.kapd);
-        const float dtau = kap * (s1 - s);
+        const float dtau = __fmul_rn(kap, s1 - s);
         ++ph.steps;
         if (dtau >= tau_rem) {
-          s_star = s + tau_rem / kap;
+          s_star = __fadd_rn(s, __fdiv_rn(tau_rem, kap));
           if (have) s_star = fminf(s_star, Sf);
           break;
         }
-        tau_rem -= dtau;
+        tau_rem = __fsub_rn(tau_rem, dtau);
         s = s1;
         const float bound = have ? Sf : seg.lower;
         if (turn_steps > 0 && s + 4.25f * m.ds_core <= bound && fabsf(xm) >= 6.0f) {
@@ -356,8 +356,8 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
     if (s_star >= 0.0f) {
       const double sd = s_star;
       ph.px = __fma_rn(sd, kx, ph.px); ph.py = __fma_rn(sd, ky, ph.py); ph.pz = __fma_rn(sd, kz, ph.pz);
-      x_site = x0 - m.gam * s_star;
-      if (m.gam != 0.0f) kH = m.kap0 * voigt<false>(m.a, x_site, Ktab);
+      x_site = __fmaf_rn(-m.gam, s_star, x0);
+      if (m.gam != 0.0f) kH = __fmul_rn(m.kap0, voigt<false>(m.a, x_site, Ktab));
       // the safety distance counts only from ds on: where it is certainly shorter (photons
       // trapped at the shell's edge, which come here event after event) its FP64 square root
       // is left out
@@ -365,8 +365,8 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
       break;
     }
     ph.px = __fma_rn(S, kx, ph.px); ph.py = __fma_rn(S, ky, ph.py); ph.pz = __fma_rn(S, kz, ph.pz);
-    const float x_end = x0 - m.gam * Sf;
-    ph.X = __fmaf_rn(x_end, m.vth, m.vgrad * (float)(b + S));  // lab frequency at the boundary
+    const float x_end = __fmaf_rn(-m.gam, Sf, x0);
+    ph.X = __fmaf_rn(x_end, m.vth, __fmul_rn(m.vgrad, (float)(b + S)));  // lab frequency at the boundary
     if (next == 1) return 1;
     ph.region = 1;
   }
@@ -391,8 +391,8 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
   ++ph.nscat;
   if (m.max_scat && ph.nscat >= m.max_scat) {
     anchor(ph);
-    const float b = (float)(ph.px * ph.k.x + ph.py * ph.k.y + ph.pz * ph.k.z);
-    ph.X = __fmaf_rn(ph.x, m.vth, m.vgrad * b);
+    const float b = (float)dot3<false>(ph.px, ph.py, ph.pz, ph.k.x, ph.k.y, ph.k.z);
+    ph.X = __fmaf_rn(ph.x, m.vth, __fmul_rn(m.vgrad, b));
     return 3;
   }
   return 0;
@@ -704,7 +704,7 @@ __device__ int shell_event_pl(const ShellModel& m, const ShellModel* mp, Photon&
       const float H = voigt<false>(m.a, x, Ktab);
       const float H2 = (m.n_lines == 2) ? voigt<false>(m.a2, __fmul_rn(x_offset(to_line2(m, ph.X), st, true), m.inv_vth), Ktab)
                                          : 0.0f;
-      const float kap = st.nr * __fmaf_rn(m.kapn, H, __fmaf_rn(m.kapn2, H2, m.kapdn));
+      const float kap = __fmul_rn(st.nr, __fmaf_rn(m.kapn, H, __fmaf_rn(m.kapn2, H2, m.kapdn)));
       const float s0 = __fdividef(tau_rem, kap);
       ++ph.steps;
       const bool is_short = s0 <= 0.0625f * m.ds_core;
@@ -714,9 +714,9 @@ __device__ int shell_event_pl(const ShellModel& m, const ShellModel* mp, Photon&
         advance(ph, s0);
         ph.safe = __fmaf_rd(-s0, 1.000001f, ph.safe);
         col_add(ph, st.nr * m.invF, s0);
-        kH = m.kapn * st.nr * H;
-        kH2 = m.kapn2 * st.nr * H2;
-        kD = m.kapdn * st.nr;
+        kH = __fmul_rn(__fmul_rn(m.kapn, st.nr), H);
+        kH2 = __fmul_rn(__fmul_rn(m.kapn2, st.nr), H2);
+        kD = __fmul_rn(m.kapdn, st.nr);
         ph.qx = (float)ph.px + ph.ox; ph.qy = (float)ph.py + ph.oy; ph.qz = (float)ph.pz + ph.oz;
         site = pl_state(m, ph.qx, ph.qy, ph.qz, ph.k);
         break;
@@ -781,12 +781,12 @@ __device__ int shell_event_pl(const ShellModel& m, const ShellModel* mp, Photon&
         const float H = voigt<false>(m.a, x, Ktab);
         const float H2 = (m.n_lines == 2) ? voigt<false>(m.a2, __fmul_rn(x_offset(to_line2(m, ph.X), st, true), m.inv_vth), Ktab)
                                            : 0.0f;
-        const float kap = st.nr * __fmaf_rn(m.kapn, H, __fmaf_rn(m.kapn2, H2, m.kapdn));
+        const float kap = __fmul_rn(st.nr, __fmaf_rn(m.kapn, H, __fmaf_rn(m.kapn2, H2, m.kapdn)));
         in_wing = fabsf(x) >= 6.0f;
         if (sub_step(s1, kap, st.nr)) {
-          kH = m.kapn * st.nr * H;
-          kH2 = m.kapn2 * st.nr * H2;
-          kD = m.kapdn * st.nr;
+          kH = __fmul_rn(__fmul_rn(m.kapn, st.nr), H);
+          kH2 = __fmul_rn(__fmul_rn(m.kapn2, st.nr), H2);
+          kD = __fmul_rn(m.kapdn, st.nr);
           break;
         }
       }
@@ -819,8 +819,8 @@ __device__ int shell_event_pl(const ShellModel& m, const ShellModel* mp, Photon&
   // opacities (one uniform); dust absorbs.
   int ch = 0;
   if (kD > 0.0f || m.n_lines == 2) {
-    const float u = w.channel, kt = kH + kH2 + kD;
-    ch = (u < __fdividef(kH, kt)) ? 0 : ((u < __fdividef(kH + kH2, kt)) ? 1 : 2);
+    const float u = w.channel, kt = __fadd_rn(__fadd_rn(kH, kH2), kD);
+    ch = (u < __fdividef(kH, kt)) ? 0 : ((u < __fdividef(__fadd_rn(kH, kH2), kt)) ? 1 : 2);
   }
   if (ch == 2) return 2;
   float xo;
