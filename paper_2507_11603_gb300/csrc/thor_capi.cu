@@ -47,28 +47,21 @@ void* thor_ctx::scratch(Buf& b, size_t bytes) {
   return b.p;
 }
 
+static bool lock_host(void** p, size_t bytes) {
+  if (cudaMallocHost(p, bytes) == cudaSuccess) return true;
+  cudaGetLastError();
+  return false;
+}
+thor_ctx::thor_ctx() : staging_block(lock_host, [](void* p) { cudaFreeHost(p); }, (size_t)16 << 20) {}
 void* thor_ctx::pinned(size_t bytes) {
-  if (bytes > kPinnedMax) return nullptr;
-  if (pinned_cap >= bytes) return h_pinned;
-  if (h_pinned) {
-    cudaStreamSynchronize(stream);  // no copy out of the old block is in flight
-    cudaFreeHost(h_pinned);
-  }
-  h_pinned = nullptr;
-  pinned_cap = 0;
-  const size_t cap = bytes < 16384 ? 16384 : bytes;
-  if (cudaMallocHost(&h_pinned, cap) != cudaSuccess) {
-    h_pinned = nullptr;
-    cudaGetLastError();
-    return nullptr;
-  }
-  pinned_cap = cap;
-  return h_pinned;
+  return staging_block.locked(bytes, [this]() { cudaStreamSynchronize(stream); });
+}
+void* thor_ctx::staging(size_t bytes) {
+  return staging_block.any(bytes, [this]() { cudaStreamSynchronize(stream); });
 }
 
 thor_ctx::~thor_ctx() {
   cudaSetDevice(device);
-  if (h_pinned) cudaFreeHost(h_pinned);
   for (Buf* b : {&b_run, &b_cube, &b_raw, &b_raw2, &b_diag, &b_stats, &b_spill, &b_cmp,
                  &b_stage[0], &b_stage[1], &b_gslots, &b_share})
     if (b->p) cudaFree(b->p);
@@ -400,7 +393,7 @@ extern "C" int thor_grid_create(thor_ctx_t ctx, const float* n_HI, const float* 
                    "grid pack");
   if (rc == THOR_OK) rc = ctx->cuda(launch_scan_f64(g->cdf, n, g->scan_tmp, ctx->stream), "emission CDF");
   struct Check { unsigned long long bad; double total; };
-  Check* chk = (Check*)ctx->pinned(sizeof(Check));
+  Check* chk = (Check*)ctx->staging(sizeof(Check));
   if (!chk && rc == THOR_OK) rc = ctx->fail(THOR_ERR_OOM, "thor_grid_create: staging");
   if (rc == THOR_OK)
     rc = ctx->cuda(cudaMemcpyAsync(&chk->bad, d_bad, sizeof chk->bad, cudaMemcpyDeviceToHost, ctx->stream), "grid check");
@@ -590,11 +583,10 @@ extern "C" int thor_run(thor_ctx_t ctx, thor_geom_t g, const thor_source* src, u
   static_assert(sizeof(QHost) <= kRunModel, "run record layout");
   const bool dev_out = spec->mem_kind == THOR_MEM_DEVICE;
   const size_t sb = dev_out ? 0 : (size_t)(spec->n_bins + 2) * 8;
-  // the record's image in page-locked memory; a spectrum too long for it is cleared and copied
-  // by itself
+  // the record's image in host memory; a spectrum too long for it is cleared and copied by itself
   const bool spec_in = kRunSpec + sb <= ((size_t)1 << 20);
   const size_t rec_bytes = kRunSpec + (spec_in ? sb : 0);
-  char* img = (char*)ctx->pinned(rec_bytes);
+  char* img = (char*)ctx->staging(rec_bytes);
   if (!img) return ctx->fail(THOR_ERR_OOM, "run staging");
   std::memset(img, 0, rec_bytes);
   std::memcpy(img, &qh, sizeof qh);

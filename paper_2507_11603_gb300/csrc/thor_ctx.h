@@ -8,6 +8,7 @@
 
 #include "../../include/thor.h"
 #include "thor_internal.h"
+#include "thor_staging.h"
 
 struct thor_ctx {
   struct Buf {
@@ -26,10 +27,8 @@ struct thor_ctx {
   // grow-only scratch buffers reused across calls
   Buf b_run;                        // a run's record: queue, model, tally, counters, host spectrum
   Buf b_cube, b_raw, b_raw2, b_diag, b_stats, b_spill, b_cmp;
-  // page-locked staging of small uploads and results (grow-only, at most kPinnedMax bytes)
-  static constexpr size_t kPinnedMax = (size_t)16 << 20;
-  void* h_pinned = nullptr;
-  size_t pinned_cap = 0;
+  // staging of small uploads and results (page-locked up to 16 MiB)
+  thor::HostStaging staging_block;
   // persistent grid sizes for the launch shape they were asked for (block 0: not yet)
   struct GridSize { int block = 0, per_sm = 0, size = 0; } shell_size, grid_size;
   Buf b_stage[2];                   // host-input staging, double-buffered (forest)
@@ -54,7 +53,9 @@ struct thor_ctx {
   int cuda(cudaError_t e, const char* what);
   int select();
   void* scratch(Buf& b, size_t bytes);
-  void* pinned(size_t bytes);  // NULL beyond kPinnedMax or if it cannot be had
+  void* pinned(size_t bytes);   // page-locked, or NULL
+  void* staging(size_t bytes);  // page-locked where it can be had, else ordinary memory
+  thor_ctx();
   ~thor_ctx();
 };
 

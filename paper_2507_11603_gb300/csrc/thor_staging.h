@@ -1,0 +1,60 @@
+// thor_staging.h -- host memory through which a context's small uploads and results pass
+// (grow-only; contents are not kept across a growth).  Page-locked where it can be had: one
+// asynchronous copy instead of a staged one.  Where it cannot, ordinary memory does: a call is
+// slower then, not refused.
+#pragma once
+
+#include <cstddef>
+#include <cstdlib>
+
+namespace thor {
+
+class HostStaging {
+ public:
+  using Lock = bool (*)(void**, std::size_t);  // page-locked allocation; false where there is none
+  using Unlock = void (*)(void*);
+  HostStaging(Lock lock, Unlock unlock, std::size_t max_locked) : lock_(lock), unlock_(unlock), max_(max_locked) {}
+  HostStaging(const HostStaging&) = delete;
+  HostStaging& operator=(const HostStaging&) = delete;
+  ~HostStaging() {
+    if (locked_) unlock_(locked_);
+    std::free(plain_);
+  }
+  // Page-locked memory, or NULL beyond max_locked or where it cannot be had.  `drain` waits for
+  // the copies out of and into the block that a growth frees.
+  template <class Drain>
+  void* locked(std::size_t bytes, Drain drain) {
+    if (bytes > max_) return nullptr;
+    if (locked_cap_ >= bytes) return locked_;
+    if (locked_) {
+      drain();
+      unlock_(locked_);
+    }
+    locked_ = nullptr;
+    locked_cap_ = 0;
+    const std::size_t cap = bytes < 16384 ? 16384 : bytes;
+    if (!lock_(&locked_, cap)) return locked_ = nullptr;
+    locked_cap_ = cap;
+    return locked_;
+  }
+  // Page-locked memory, else ordinary memory; NULL only where there is no memory at all.
+  template <class Drain>
+  void* any(std::size_t bytes, Drain drain) {
+    if (void* p = locked(bytes, drain)) return p;
+    if (plain_cap_ >= bytes) return plain_;
+    drain();
+    std::free(plain_);
+    plain_ = std::malloc(bytes);
+    plain_cap_ = plain_ ? bytes : 0;
+    return plain_;
+  }
+
+ private:
+  Lock lock_;
+  Unlock unlock_;
+  std::size_t max_;
+  void *locked_ = nullptr, *plain_ = nullptr;
+  std::size_t locked_cap_ = 0, plain_cap_ = 0;
+};
+
+}  // namespace thor
