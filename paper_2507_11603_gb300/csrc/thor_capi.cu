@@ -590,6 +590,7 @@ extern "C" int thor_run(thor_ctx_t ctx, thor_geom_t g, const thor_source* src, u
   if (!img) return ctx->fail(THOR_ERR_OOM, "run staging");
   std::memset(img, 0, rec_bytes);
   std::memcpy(img, &qh, sizeof qh);
+  DrainGuard drain([s]() { cudaStreamSynchronize(s); });
   auto upload = [&]() {
     int e = ctx->cuda(cudaMemcpyAsync(rec, img, rec_bytes, cudaMemcpyHostToDevice, s), "run record upload");
     if (!e && !spec_in) e = ctx->cuda(cudaMemsetAsync(o.spec, 0, sb, s), "clear spectrum");
@@ -802,6 +803,7 @@ extern "C" int thor_run(thor_ctx_t ctx, thor_geom_t g, const thor_source* src, u
   if (!rc) rc = finish_outputs(ctx, spec, n_photons, grid, o);
   if (!rc) rc = ctx->cuda(cudaStreamSynchronize(s), "photon loop");
   if (rc) return rc;
+  drain.done();
   Tally t;
   unsigned long long st[2];
   std::memcpy(&t, img + kRunTally, sizeof t);
@@ -969,6 +971,7 @@ extern "C" int thor_reweight(thor_ctx_t ctx, int64_t n, const float* X0, const f
   const uint8_t* st = status;
   // results through page-locked memory where they fit: scaled out of it in one pass
   double* h_out = (double*)ctx->pinned(ob);
+  DrainGuard drain([s]() { cudaStreamSynchronize(s); });
   int rc = ctx->cuda(cudaMemsetAsync(d_out, 0, ob, s), "clear reweight output");
   if (!rc) rc = ctx->cuda(cudaMemcpyAsync(d_prm, prm.data(), pb, cudaMemcpyHostToDevice, s), "reweight params");
   if (!rc && mem_kind == THOR_MEM_HOST) {
@@ -991,6 +994,7 @@ extern "C" int thor_reweight(thor_ctx_t ctx, int64_t n, const float* X0, const f
     rc = ctx->cuda(cudaMemcpyAsync(h_out ? h_out : out, d_out, ob, cudaMemcpyDeviceToHost, s), "reweight output");
   if (!rc) rc = ctx->cuda(cudaStreamSynchronize(s), "thor_reweight");
   if (rc) return rc;
+  drain.done();
   cudaEventElapsedTime(&ctx->last_ms, ctx->ev0, ctx->ev1);
   const double inv = 1.0 / (double)n;
   const double* from = h_out ? h_out : out;

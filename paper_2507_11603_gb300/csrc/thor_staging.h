@@ -57,4 +57,23 @@ class HostStaging {
   std::size_t locked_cap_ = 0, plain_cap_ = 0;
 };
 
+// Waits for the copies in flight on every return but the one after done(): a call that fails half
+// way through leaves none that would read the staging block, or write the device record, when the
+// next call (on another stream, maybe) uses them again.
+template <class Drain>
+class DrainGuard {
+ public:
+  explicit DrainGuard(Drain drain) : drain_(drain) {}
+  DrainGuard(const DrainGuard&) = delete;
+  DrainGuard& operator=(const DrainGuard&) = delete;
+  ~DrainGuard() {
+    if (armed_) drain_();
+  }
+  void done() { armed_ = false; }
+
+ private:
+  Drain drain_;
+  bool armed_ = true;
+};
+
 }  // namespace thor

@@ -1,7 +1,7 @@
 """The context's staging memory (csrc/thor_staging.h) where page-locked memory cannot be had: runs and
 grid creation go on through ordinary memory instead of being refused, page-locked memory is used
-again once there is some, every block is freed once, and no block in use is freed before its copies
-are waited for."""
+again once there is some, every block is freed once, no block in use is freed before its copies are
+waited for, and a call that fails half way waits for its own."""
 import os
 import shutil
 import subprocess
@@ -41,6 +41,18 @@ int main() {
     assert(s.any(30000, drain) && live == 1 && !s.locked((1 << 20) + 1, drain));
   }
   assert(live == 0);
+  drains = 0;
+  auto call = [&](int fails_at) {  // a call that fails at step 0, 1 or 2, or not at all
+    if (fails_at == 0) return 1;   // nothing in flight yet
+    thor::DrainGuard g(drain);
+    if (fails_at == 1) return 2;
+    if (fails_at == 2) return 3;
+    g.done();
+    return 0;
+  };
+  assert(call(0) == 1 && drains == 0);
+  assert(call(1) == 2 && drains == 1 && call(2) == 3 && drains == 2);
+  assert(call(3) == 0 && drains == 2);
   std::puts("ok");
 }
 """
@@ -63,3 +75,16 @@ def test_runs_and_grids_use_the_fallback():
     with open(os.path.join(ROOT, "paper_2507_11603_gb300", "csrc", "thor_capi.cu")) as f:
         calls = [line.strip() for line in f if "ctx->pinned(" in line]
     assert calls == ["double* h_out = (double*)ctx->pinned(ob);"]
+
+
+def test_no_copy_outlives_a_failed_call():
+    """Calls that upload from the staging block drain the stream on every early return: the guard
+    stands before the first copy, and is released only after the call's last synchronisation."""
+    with open(os.path.join(ROOT, "paper_2507_11603_gb300", "csrc", "thor_capi.cu")) as f:
+        text = f.read()
+    for name in ("thor_run", "thor_reweight"):
+        body = text[text.index(f'extern "C" int {name}(thor_ctx_t'):]
+        body = body[:body.index("\n}\n")]
+        guard, done = body.index("DrainGuard drain("), body.index("drain.done();")
+        assert guard < body.index("cudaMemcpyAsync(") and done > body.rindex("cudaStreamSynchronize(s),")
+        assert body.count("drain.done();") == 1
