@@ -1,7 +1,9 @@
 // thor_staging.h -- host memory through which a context's small uploads and results pass
 // (grow-only; contents are not kept across a growth).  Page-locked where it can be had: one
 // asynchronous copy instead of a staged one.  Where it cannot, ordinary memory does: a call is
-// slower then, not refused.
+// slower then, not refused.  Locking and unlocking takes some 0.3 ms, which a copy saves some 10 us
+// of, so the first kPlain requests are served from ordinary memory (a context made for one tiny
+// run: 0.14 ms, 0.48 with the lock) and the block grows by powers of two.
 #pragma once
 
 #include <cstddef>
@@ -20,11 +22,16 @@ class HostStaging {
     if (locked_) unlock_(locked_);
     std::free(plain_);
   }
-  // Page-locked memory, or NULL beyond max_locked or where it cannot be had.  `drain` waits for
-  // the copies out of and into the block that a growth frees.
+  static constexpr int kPlain = 2;
+  // Page-locked memory, or NULL beyond max_locked, for the first kPlain requests, or where it
+  // cannot be had.  `drain` waits for the copies out of and into the block that a growth frees.
   template <class Drain>
   void* locked(std::size_t bytes, Drain drain) {
     if (bytes > max_) return nullptr;
+    if (requests_ < kPlain) {
+      ++requests_;
+      return nullptr;
+    }
     if (locked_cap_ >= bytes) return locked_;
     if (locked_) {
       drain();
@@ -32,7 +39,9 @@ class HostStaging {
     }
     locked_ = nullptr;
     locked_cap_ = 0;
-    const std::size_t cap = bytes < 16384 ? 16384 : bytes;
+    std::size_t cap = 16384;
+    while (cap < bytes) cap *= 2;
+    if (cap > max_) cap = max_;
     if (!lock_(&locked_, cap)) return locked_ = nullptr;
     locked_cap_ = cap;
     return locked_;
@@ -53,6 +62,7 @@ class HostStaging {
   Lock lock_;
   Unlock unlock_;
   std::size_t max_;
+  int requests_ = 0;
   void *locked_ = nullptr, *plain_ = nullptr;
   std::size_t locked_cap_ = 0, plain_cap_ = 0;
 };

@@ -1,7 +1,8 @@
 """The context's staging memory (csrc/thor_staging.h) where page-locked memory cannot be had: runs and
 grid creation go on through ordinary memory instead of being refused, page-locked memory is used
-again once there is some, every block is freed once, no block in use is freed before its copies are
-waited for, and a call that fails half way waits for its own."""
+again once there is some, none is locked for a context of few calls, every block is freed once, no
+block in use is freed before its copies are waited for, and a call that fails half way waits for
+its own."""
 import os
 import shutil
 import subprocess
@@ -21,6 +22,7 @@ int main() {
   auto drain = []() { ++drains; };
   {
     thor::HostStaging s(lock, unlock, 1 << 20);
+    for (int i = 0; i < thor::HostStaging::kPlain; ++i) assert(!s.locked(100, drain));
     assert(!s.locked(100, drain));                   // none to be had
     char* a = (char*)s.any(100, drain);
     assert(a); std::memset(a, 1, 100);
@@ -34,11 +36,17 @@ int main() {
     assert(c && live == 1 && c == s.locked(16384, drain));
     std::memset(c, 4, 16384);
     drains = 0;
-    assert(s.locked(20000, drain) && drains == 1 && live == 1);
+    assert(s.locked(20000, drain) && drains == 1 && live == 1 && s.locked(32768, drain) && drains == 1);
     allow = 0;
-    assert(!s.locked(30000, drain) && live == 0 && s.any(30000, drain));
+    assert(!s.locked(40000, drain) && live == 0 && s.any(40000, drain));
     allow = 1;
-    assert(s.any(30000, drain) && live == 1 && !s.locked((1 << 20) + 1, drain));
+    assert(s.any(40000, drain) && live == 1 && !s.locked((1 << 20) + 1, drain) && s.locked(1 << 20, drain));
+  }
+  assert(live == 0);
+  {  // nothing is locked for a context of few calls
+    thor::HostStaging s(lock, unlock, 1 << 20);
+    for (int i = 0; i < thor::HostStaging::kPlain; ++i) assert(s.any(100, drain) && live == 0);
+    assert(s.any(100, drain) && live == 1);
   }
   assert(live == 0);
   drains = 0;
