@@ -297,8 +297,8 @@ def run_shell_bench(args):
         "config": {"workload": WORKLOAD, "photons_per_step": N_PHOTONS, "l2": "flushed (256 MiB write) before each step",
                    "scatterings_per_step": n_scat / args.steps, "kernel_ms_per_step": kern_avg_ms,
                    "launch": {"block": args.block or 128, "blocks_per_sm": args.blocks_per_sm,
-                              "pipelined_event_lanes": args.pipe_lanes if args.pipe_lanes >= 0 else 32,
-                              "core_burst_lanes": args.burst_lanes if args.burst_lanes >= 0 else 1,
+                              "event_round_lanes": args.pipe_lanes if args.pipe_lanes >= 0 else 32,
+                              "deep_round_lanes": args.burst_lanes if args.burst_lanes >= 0 else 1,
                               "tail_work_sharing": not args.no_tail_share}},
         "e2e": {"value": e2e_value, "unit": "scatterings/s", "h2d_bytes_per_step": 1536 + (RUN["n_bins"] + 2) * 8,
                 "d2h_bytes_per_step": (RUN["n_bins"] + 2) * 8 + 512, "steps": n_e2e,

@@ -322,8 +322,7 @@ typedef struct {
                                 one per warp), -1 = off (every packet shares warps) */
   int32_t presort;           /* frequency pre-sorting of the packets in flight between rounds, so a
                                 warp's packets are of one kind: 1 = on, 0 = off (the default; on the
-                                measured stream it did not pay, the core events in rounds already
-                                keep core packets in step) */
+                                measured stream it does not pay: packets change kind within a round) */
   int32_t reserved;
 } thor_server_config;
 

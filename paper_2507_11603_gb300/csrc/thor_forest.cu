@@ -15,8 +15,9 @@
 //   far    a cell whose line centre is at least kFar half-widths from an interval's centre, with
 //          the interval outside |x| < 6, contributes at the interval's 16 Chebyshev nodes instead
 //          of at its bins -- on the coarse intervals where it is far from one, else on the fine
-//          ones.  With the pole of 1/x^2 at kFar = 2.25 half-widths the interpolation error is
-//          below (kFar + sqrt(kFar^2 - 1))^-16 x 68 = 7e-9 of the contribution, under FP32's own
+//          ones.  With kFar = 2.25 the interpolation error of the wing (t g(t), t = 1 / x^2) is
+//          at most 1.2e-8 of the contribution, evaluated in FP64 over all half-widths and both
+//          levels (largest where |x| = 6 decides, at 4.8 Doppler widths), under FP32's own
 //          rounding; all contributions are positive, so it is the same for the sum;
 //   near   the other cells (the core |x| < 6, the wing next to it, and the cells opposite the
 //          interval, where the nearest image changes side) are evaluated at each bin.

@@ -11,8 +11,9 @@
 // A bin's sum leaves the CTA by one FP64 atomic per target.  (One CTA per 256 photons and
 // target, with an FP32 histogram in shared memory, took 703 us there: every target re-read
 // the photons, shared FP32 atomics are compare-and-swap loops, and each CTA ended with an
-// atomic per occupied bin, 38e6 of them.)  Weights add in FP32 over blocks of 256 photons and
-// in two-float arithmetic (error-free sums) above that.
+// atomic per occupied bin, 38e6 of them.)  Weights add in FP32 over blocks of 256 photons and in
+// two-float arithmetic (error-free sums) above that.  Few weights per photon do not pay for the
+// sort: launch_reweight draws the lines between the three kernels.
 #include <algorithm>
 
 #include "thor_internal.h"

@@ -25,8 +25,8 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr int kFlySteps = 128;
 constexpr float kFlyNone = -1.0f, kFlyBall = -2.0f;
 constexpr float kSafePending = -1.0f;  // Photon::safe: not formed yet (power laws; the offset is zero)
-constexpr uint32_t kLongLived = 1u << 14;
-constexpr uint32_t kPriBudget = 16;  // served rounds: budget multiple of a priority warp (one packet)  // served rounds: packets past this many events run one per warp
+constexpr uint32_t kLongLived = 1u << 14;  // served rounds: packets past this many events run one per warp
+constexpr uint32_t kPriBudget = 16;        // served rounds: budget multiple of a priority warp (one packet)
 
 struct Photon {
   double px, py, pz;  // FP64 anchor; the position is anchor + offset
@@ -419,8 +419,8 @@ __device__ int shell_event(const ShellModel& m, Photon& ph, const float* __restr
 // the same words, so both paths give bit-identical results.
 // Measured (GB300, 2070 MHz): a photon alone in a static sphere 0.345 us per event (0.47 us
 // when its own lane formed the directions' angles and the words came by shuffle), at 1e3 K
-// 0.40 us (1.76 us); 5000 photons in a sphere of tau0 = 1e4 73 ms (107 ms); 1e5 photons in an
-// expanding shell of N_HI = 1e19 365 ms (576 ms), of 1e20 3.1 s (5.35 s).  The general events run for
+// 0.40 us (1.76 us); 5000 photons in a sphere of tau0 = 1e4 78 ms (113 ms); 1e5 photons in an
+// expanding shell of N_HI = 1e19 350-380 ms (535-580 ms), of 1e20 3.4 s (5.4 s).  The general events run for
 // all the packets that wait for one, at most once per `depth` core events: a general event
 // costs several core events, and one lane in sixty needs one at any time.
 constexpr int kChainSlots = kWordSlots;  // events per warp and round
@@ -430,8 +430,8 @@ constexpr uint32_t kFirstDepth = 4;   // ... at first: doubled where a round run
 // ... and in a served warp while another packet waits for a general event: the packets of a warp
 // belong to several requests there, and with 16 core events to each general one a thin request's
 // packets got one event in 17 of those a round is charged.  256 requests of up to N_HI = 1e21, 28
-// per second: p50 32 -> 24 ms, p90 520 -> 432 ms, all at once no slower (64 requests 2.50 -> 2.42 s;
-// depth 2 the same, 1 2.78 s, 8 2.51 s).
+// per second: p50 28 -> 23 ms, p90 483 -> 429 ms, all at once no slower (64 requests 2.41 -> 2.44 s;
+// depth 2 2.48 s, 1 2.78 s, 8 2.51 s).
 constexpr uint32_t kSharedDepth = 4;
 constexpr uint32_t kVoteEvents = 4;   // core events between two votes on whether any packet goes on
 __device__ __forceinline__ void form_words(const ShellModel& m, const Photon& ph, WordBuf& wb, bool mine, int D,
@@ -1002,7 +1002,8 @@ __global__ void __launch_bounds__(256, 1) shell_run_kernel(const ShellModel* __r
         if (lane == 0) { load_rec(m, c.pool[got], ph); active = true; }
         continue;
       }
-      if (__popc(live) >= 2 && ran >= kShareEvents) {  // (short histories are over by then) give packets away while empty warps wait, keeping the lowest lane's
+      // give packets away while empty warps wait, keeping the lowest lane's (short histories are over by then)
+      if (__popc(live) >= 2 && ran >= kShareEvents) {
         const int leader = __ffs(live) - 1;
         long long give = 0;
         if ((int)lane == leader) give = pool_give_count(c.share, __popc(live));
